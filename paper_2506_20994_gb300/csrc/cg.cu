@@ -1458,47 +1458,62 @@ extern "C" int ax_axpby(double *y, double a, const double *x, double b, int64_t 
 // ---------------------------------------------------------------------------
 namespace {
 
+// isc: input scale, sqrt(minv) (symmetric form) or minv; osc: output scale of
+// the correction, mask .* sqrt(minv) or mask .* c.  Formed once per training
+// call: an fp64 square root is some thirty operations of the narrow fp64 pipe,
+// and each step reads the scales four times a point (at 512 elements, lx = 8,
+// the roots alone were about 30 us of the step).
+__global__ void energy_scales_kernel(double *__restrict__ isc, double *__restrict__ osc,
+                                     const double *__restrict__ minv,
+                                     const double *__restrict__ mask,
+                                     const double *__restrict__ c, int sym, int64_t n) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    const double m = minv[q], sq = sym ? sqrt(m) : m;
+    isc[q] = sq;
+    osc[q] = mask[q] * (sym ? sq : c[q]);
+  }
+}
+
+// X = z / s_e with z = isc r and s_e = ||z|| of each element (block); a
+// thread keeps its first four values of z
 __global__ void energy_features_kernel(float *__restrict__ X, double *__restrict__ s_out,
                                        const double *__restrict__ r,
-                                       const double *__restrict__ minv, int N, int sym) {
+                                       const double *__restrict__ isc, int N) {
+  constexpr int KEEP = 4;
   __shared__ double sh[kRedThreads / 32];
-  __shared__ double s_b;
+  __shared__ double inv_b;
   const size_t base = (size_t)blockIdx.x * N;
-  double ss = 0.0;
-  auto scale = [&](double mv) { return sym ? sqrt(mv) : mv; };
-  for (int k = threadIdx.x; k < N; k += blockDim.x) {
-    const double z = scale(minv[base + k]) * r[base + k];
-    ss += z * z;
+  double ss = 0.0, z[KEEP];
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) {
+    const int k = threadIdx.x + q * kRedThreads;
+    z[q] = k < N ? isc[base + k] * r[base + k] : 0.0;
+    ss += z[q] * z[q];
+  }
+  for (int k = threadIdx.x + KEEP * kRedThreads; k < N; k += kRedThreads) {
+    const double y = isc[base + k] * r[base + k];
+    ss += y * y;
   }
   double v[1] = {ss};
   ax::block_sum<1>(v, sh);
-  if (threadIdx.x == 0) {
-    s_b = sqrt(v[0]);
-    s_out[blockIdx.x] = s_b;
+  if (threadIdx.x == 0) {  // one root and one division a block: the fp64 pipe is narrow
+    const double s = sqrt(v[0]);
+    s_out[blockIdx.x] = s;
+    inv_b = s > 0.0 ? 1.0 / s : 0.0;
   }
   __syncthreads();
-  const double inv = s_b > 0.0 ? 1.0 / s_b : 0.0;
-  for (int k = threadIdx.x; k < N; k += blockDim.x)
-    X[base + k] = (float)(scale(minv[base + k]) * r[base + k] * inv);
+  const double inv = inv_b;
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) {
+    const int k = threadIdx.x + q * kRedThreads;
+    if (k < N) X[base + k] = (float)(z[q] * inv);
+  }
+  for (int k = threadIdx.x + KEEP * kRedThreads; k < N; k += kRedThreads)
+    X[base + k] = (float)(isc[base + k] * r[base + k] * inv);
 }
 
-// d = e - minv r - corr, with corr = mask c s_e Y (corr assembled by gs before)
-// output scale of the correction: 1/multiplicity (tanh form) or sqrt(minv)
-// (symmetric form)
-__device__ __forceinline__ double energy_out_scale(const double *c, const double *minv,
-                                                   int64_t q, int sym) {
-  return sym ? sqrt(minv[q]) : c[q];
-}
-
-__global__ void energy_corr_kernel(double *__restrict__ corr, const float *__restrict__ Y,
-                                   const double *__restrict__ s, const double *__restrict__ mask,
-                                   const double *__restrict__ c, const double *__restrict__ minv,
-                                   int sym, int N, int64_t n) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * blockDim.x)
-    corr[q] = mask[q] * energy_out_scale(c, minv, q, sym) * s[q / N] * (double)Y[q];
-}
-
+// d = e - minv r - corr (corr assembled by gs before)
 __global__ void energy_diff_kernel(double *__restrict__ d, const double *__restrict__ e,
                                    const double *__restrict__ r, const double *__restrict__ minv,
                                    const double *__restrict__ corr, int64_t n) {
@@ -1507,19 +1522,40 @@ __global__ void energy_diff_kernel(double *__restrict__ d, const double *__restr
     d[q] = e[q] - minv[q] * r[q] - corr[q];
 }
 
-__global__ void energy_dy_kernel(float *__restrict__ dY, const double *__restrict__ q,
-                                 const double *__restrict__ s, const double *__restrict__ mask,
-                                 const double *__restrict__ c, const double *__restrict__ minv,
-                                 int sym, const double *__restrict__ eA, int N, int64_t n) {
-  const double scale = eA[0] > 0.0 ? -2.0 / eA[0] : 0.0;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * blockDim.x)
-    dY[p] = (float)(scale * mask[p] * energy_out_scale(c, minv, p, sym) * s[p / N] * q[p]);
+// q = mask .* w (not stored); the partials of <d, q> and the output gradient
+// dY = -2 osc s_e q / ||e||_A^2; elements blockIdx.x, + gridDim.x, ...
+__global__ void energy_dot_dy_kernel(float *__restrict__ dY, const double *__restrict__ w,
+                                     const double *__restrict__ d,
+                                     const double *__restrict__ mask,
+                                     const double *__restrict__ c,
+                                     const double *__restrict__ osc,
+                                     const double *__restrict__ s, const double *__restrict__ eA,
+                                     int N, int nelv, double *__restrict__ partials) {
+  __shared__ double sh[kRedThreads / 32];
+  __shared__ double scale_b;
+  if (threadIdx.x == 0) scale_b = eA[0] > 0.0 ? -2.0 / eA[0] : 0.0;
+  __syncthreads();
+  const double scale = scale_b;
+  double a = 0.0;
+  for (int e = blockIdx.x; e < nelv; e += gridDim.x) {
+    const double se = scale * s[e];
+    const size_t base = (size_t)e * N;
+    for (int k = threadIdx.x; k < N; k += kRedThreads) {
+      const size_t p = base + k;
+      const double q = w[p] * mask[p];
+      a += c[p] * d[p] * q;
+      dY[p] = (float)(osc[p] * se * q);
+    }
+  }
+  double v[1] = {a};
+  ax::block_sum<1>(v, sh);
+  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
 }
 
-__global__ void store_partial_sum_kernel(const double *__restrict__ partials, int nblk,
-                                         double *__restrict__ out) {
-  ax::warp_sum_partials<1>(partials, nblk, out);
+// out[k] = sum of the kRedBlocks partials of pair k (one block per pair)
+__global__ void pair_sums_kernel(const double *__restrict__ partials, double *__restrict__ out) {
+  ax::warp_sum_partials<1>(partials + (size_t)blockIdx.x * kRedBlocks, kRedBlocks,
+                           out + blockIdx.x);
 }
 
 }  // namespace
@@ -1533,52 +1569,38 @@ extern "C" int ax_mlp_train_energy(ax_poisson *P, ax_mlp *M, const double *r_set
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t n = P->n;
   const unsigned nb = kRedBlocks;
-  int rc = ax::mlp_reserve(M, P->nelv);
+  const int sym = M->arch == AX_MLP_SYM;
+  int rc = ax::mlp_reserve(M, P->nelv, K);
+  if (rc == AX_OK) rc = ensure_fcg64(P, st);
   if (rc) return rc;
-  double *s = nullptr, *d = nullptr, *q = nullptr, *corr = nullptr, *eA = nullptr, *Lk = nullptr;
-  rc = alloc(&s, P->nelv) | alloc(&d, n) | alloc(&q, n) | alloc(&corr, n) | alloc(&eA, K) |
-       alloc(&Lk, K);
-  auto cleanup = [&]() {
-    cudaFree(s);
-    cudaFree(d);
-    cudaFree(q);
-    cudaFree(corr);
-    cudaFree(eA);
-    cudaFree(Lk);
-  };
-  if (rc) {
-    cleanup();
-    return AX_ENOMEM;
-  }
+  // scratch: the solvers' own vectors, idle here
+  double *d = P->r, *q = P->w, *isc = P->p, *osc = P->r_old, *corr = P->corr;
+  double *s = M->es, *eA = M->ek, *Lk = M->ek + K, *part = M->ek + 2 * K;
+  energy_scales_kernel<<<nb, kRedThreads, 0, st>>>(isc, osc, P->minv, P->mask, P->c, sym, n);
   // ||e_k||_A^2 once per pair
   for (int k = 0; k < K && rc == AX_OK; ++k) {
     const double *e = e_set + (size_t)k * n;
     rc = apply_f64(P, q, e, st);
     if (rc) break;
-    mask_dot_kernel<double><<<nb, kRedThreads, 0, st>>>(q, e, P->mask, P->c, P->partials, n);
-    store_partial_sum_kernel<<<1, 32, 0, st>>>(P->partials, nb, eA + k);
+    mask_dot_kernel<double><<<nb, kRedThreads, 0, st>>>(q, e, P->mask, P->c,
+                                                        part + (size_t)k * nb, n);
   }
+  pair_sums_kernel<<<K, 32, 0, st>>>(part, eA);
   for (int ep = 0; ep < epochs && rc == AX_OK; ++ep) {
     for (int k = 0; k < K && rc == AX_OK; ++k) {
       const double *r = r_set + (size_t)k * n, *e = e_set + (size_t)k * n;
-      const int sym = M->arch == AX_MLP_SYM;
-      energy_features_kernel<<<P->nelv, kRedThreads, 0, st>>>(M->X, s, r, P->minv, N, sym);
-      if ((rc = ax::mlp_train_forward(M, P->nelv, st))) break;
-      energy_corr_kernel<<<nb, kRedThreads, 0, st>>>(corr, M->Y, s, P->mask, P->c, P->minv, sym,
-                                                     N, n);
+      energy_features_kernel<<<P->nelv, kRedThreads, 0, st>>>(M->X, s, r, isc, N);
+      if ((rc = ax::mlp_train_forward_corr(M, P->nelv, corr, osc, s, st))) break;
       if ((rc = ax_gs_sum(P->gs, corr, st))) break;
       energy_diff_kernel<<<nb, kRedThreads, 0, st>>>(d, e, r, P->minv, corr, n);
       if ((rc = apply_f64(P, q, d, st))) break;
-      mask_dot_kernel<double><<<nb, kRedThreads, 0, st>>>(q, d, P->mask, P->c, P->partials, n);
-      store_partial_sum_kernel<<<1, 32, 0, st>>>(P->partials, nb, Lk + k);
-      energy_dy_kernel<<<nb, kRedThreads, 0, st>>>(M->dY, q, s, P->mask, P->c, P->minv, sym,
-                                                   eA + k, N, n);
+      energy_dot_dy_kernel<<<nb, kRedThreads, 0, st>>>(M->dY, q, d, P->mask, P->c, osc, s,
+                                                       eA + k, N, P->nelv, part + (size_t)k * nb);
       if ((rc = ax::mlp_train_backward(M, P->nelv, st))) break;
-      if (sym && (rc = ax::mlp_tie_grad(M, st))) break;
       if ((rc = ax::mlp_adam_step(M, lr, st))) break;
-      if (sym && (rc = ax::mlp_tie_params(M, st))) break;
     }
   }
+  pair_sums_kernel<<<K, 32, 0, st>>>(part, Lk);  // the last epoch's losses
   if (rc == AX_OK) rc = ax::mlp_refresh(M, st);
   std::vector<double> hl(K), he(K);
   if (rc == AX_OK &&
@@ -1593,7 +1615,6 @@ extern "C" int ax_mlp_train_energy(ax_poisson *P, ax_mlp *M, const double *r_set
     for (int k = 0; k < K; ++k) m += he[k] > 0 ? hl[k] / he[k] : 0.0;
     *final_loss = m / K;  // mean relative energy error of the last epoch
   }
-  cleanup();
   return rc;
 }
 

@@ -10,9 +10,11 @@
 //   chunk, the hidden layer stays in shared memory, and the output goes
 //   through shared memory in 128-column slabs so that every global access
 //   is a coalesced row segment.
-// * Training: fp32 SIMT kernels with one thread per output and a fixed
-//   summation order (deterministic, no atomics): forward, mean-squared loss,
-//   backpropagation, Adam (Kingma & Ba 2015).
+// * Training: fp32 SIMT kernels with a fixed summation order (deterministic,
+//   no atomics): forward, mean-squared loss, backpropagation, Adam (Kingma &
+//   Ba 2015).  The products are small (25 million multiply-adds at 512 rows,
+//   lx = 8, 48 hidden units: under a microsecond of arithmetic), so they are
+//   cut for latency: see skinny_kernel.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -391,103 +393,239 @@ __global__ void gather_pairs_kernel(float *__restrict__ X, float *__restrict__ T
   }
 }
 
-// H[b][h] = tanh(sum_k X[b][k] W1[k][h] + b1[h])
-__global__ void fwd_hidden_kernel(float *__restrict__ H, const float *__restrict__ X,
-                                  const float *__restrict__ theta, int B, int N, int Hd,
-                                  int sym) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= (int64_t)B * Hd) return;
-  const int b = (int)(q / Hd), h = (int)(q % Hd);
-  const float *W1 = theta, *b1 = theta + (size_t)N * Hd;
-  float a = 0.f;
-  for (int k = 0; k < N; ++k) a = fmaf(X[(size_t)b * N + k], W1[(size_t)k * Hd + h], a);
-  H[q] = sym ? a + b1[h] : tanhf(a + b1[h]);
+// C[m][h] = sum_k A(m, k) B(k, h), h < Hd <= 64: the products of training
+// whose one side is the hidden layer.  A block takes kRows rows of C and walks
+// k in chunks of kChunk: A's and B's chunk are staged in shared memory while
+// the next one's loads are in flight in registers, and four groups of 64
+// threads (thread (slice, h)) take a quarter of the chunk each; their sums are
+// added in a fixed order.  One thread per output with a chain over all of k
+// left 96 blocks each waiting on 512 dependent loads (the four products of a
+// training step took over 200 of its 415 us at 512 rows, lx = 8, 48 hidden
+// units); the slices alone, with B read from L2 inside the chain, 19-32 us a
+// product; staged, 7-11 us (GB300, cold).
+// AT: A stored [k][m], else [m][k].  BT: B stored [h][k], else [k][h] with
+// ldb = Hd (one contiguous 16-byte aligned run per chunk).  ONES: row M - 1
+// of A is all ones (the bias gradient).  A second pair (A2, B2) with the same
+// shapes, if given, continues the same sums.  epi(m, h, sum) receives each
+// output once; csum(m, sum_k A(m, k)) each row's sum (the output-bias
+// gradient) when CSUM.
+constexpr int kRows = 4, kSlices = 4, kChunk = 128;
+
+template <bool AT, bool BT, bool ONES, bool CSUM, class Epi, class Csum>
+__global__ void __launch_bounds__(kThreads)
+skinny_kernel(const float *__restrict__ A, const float *__restrict__ B,
+              const float *__restrict__ A2, const float *__restrict__ B2, int M, int K, int Hd,
+              int lda, int ldb, Epi epi, Csum csum) {
+  constexpr int NA = kRows * kChunk / kThreads;       // A values a thread stages
+  constexpr int NB = kChunk * 64 / 4 / kThreads;      // B float4 a thread stages (Hd = 64)
+  constexpr int PB = 65;                              // padded row of a transposed B
+  __shared__ float4 As[kChunk];
+  __shared__ float4 Bs4[(kChunk * PB + 3) / 4];
+  __shared__ float red[kSlices][kRows][64];
+  __shared__ float redc[kSlices][kRows];
+  float *Bs = reinterpret_cast<float *>(Bs4);
+  const int tid = threadIdx.x, h = tid & 63, sl = tid >> 6;
+  const int m0 = blockIdx.x * kRows;
+  const int Mr = ONES ? M - 1 : M;  // rows that A stores
+  const int BS = BT ? PB : Hd;      // row stride of Bs
+  float acc[kRows] = {0.f, 0.f, 0.f, 0.f}, cs[kRows] = {0.f, 0.f, 0.f, 0.f};
+  const int chunks = (K + kChunk - 1) / kChunk, steps = A2 ? 2 * chunks : chunks;
+  float ra[NA];
+  float4 rb[NB];
+  // one step's values into registers
+  auto load = [&](int step) {
+    const bool second = step >= chunks;
+    const float *a = second ? A2 : A, *b = second ? B2 : B;
+    const int k0 = (second ? step - chunks : step) * kChunk;
+    const int kn = min(kChunk, K - k0);
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int v = tid + q * kThreads;
+      const int r = AT ? v % kRows : v / kChunk, k = AT ? v / kRows : v % kChunk;
+      const int m = m0 + r;
+      ra[q] = k >= kn ? 0.f
+              : m < Mr ? __ldg(AT ? a + (size_t)(k0 + k) * lda + m : a + (size_t)m * lda + k0 + k)
+              : ONES && m == Mr ? 1.f : 0.f;
+    }
+    const int nv = kn * Hd;
+    if constexpr (BT) {
+#pragma unroll
+      for (int q = 0; q < 4 * NB; ++q) {  // value (row v / kChunk of B, k = v % kChunk)
+        const int v = tid + q * kThreads, hh = v / kChunk, k = v % kChunk;
+        reinterpret_cast<float *>(rb)[q] =
+            hh < Hd && k < kn ? __ldg(b + (size_t)hh * ldb + k0 + k) : 0.f;
+      }
+    } else {
+      const float *src = b + (size_t)k0 * Hd;
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        const int v = 4 * (tid + q * kThreads);
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (v + 3 < nv) {
+          x = __ldg(reinterpret_cast<const float4 *>(src + v));
+        } else {
+          if (v < nv) x.x = __ldg(src + v);
+          if (v + 1 < nv) x.y = __ldg(src + v + 1);
+          if (v + 2 < nv) x.z = __ldg(src + v + 2);
+        }
+        rb[q] = x;
+      }
+    }
+  };
+  load(0);
+  for (int step = 0; step < steps; ++step) {
+    if (step) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int v = tid + q * kThreads;
+      const int r = AT ? v % kRows : v / kChunk, k = AT ? v / kRows : v % kChunk;
+      reinterpret_cast<float *>(As)[k * kRows + r] = ra[q];
+    }
+    if constexpr (BT) {
+#pragma unroll
+      for (int q = 0; q < 4 * NB; ++q) {
+        const int v = tid + q * kThreads;
+        Bs[(v % kChunk) * PB + v / kChunk] = reinterpret_cast<const float *>(rb)[q];
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < NB; ++q) Bs4[tid + q * kThreads] = rb[q];
+    }
+    __syncthreads();
+    if (step + 1 < steps) load(step + 1);
+    if (h < Hd) {
+      const int ka = sl * (kChunk / kSlices);
+#pragma unroll 8
+      for (int k = ka; k < ka + kChunk / kSlices; ++k) {  // zeros past the end of k
+        const float bv = Bs[k * BS + h];
+        const float4 av = As[k];
+        acc[0] = fmaf(av.x, bv, acc[0]);
+        acc[1] = fmaf(av.y, bv, acc[1]);
+        acc[2] = fmaf(av.z, bv, acc[2]);
+        acc[3] = fmaf(av.w, bv, acc[3]);
+        if (CSUM) {
+          cs[0] += av.x;
+          cs[1] += av.y;
+          cs[2] += av.z;
+          cs[3] += av.w;
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    red[sl][r][h] = acc[r];
+    if (CSUM && h == 0) redc[sl][r] = cs[r];
+  }
+  __syncthreads();
+  const int r = sl;  // four slices, four rows: thread (slice, h) finishes row `slice`
+  if (m0 + r < M && h < Hd)
+    epi(m0 + r, h, (red[0][r][h] + red[1][r][h]) + (red[2][r][h] + red[3][r][h]));
+  if (CSUM && h == 0 && m0 + r < M)
+    csum(m0 + r, (redc[0][r] + redc[1][r]) + (redc[2][r] + redc[3][r]));
+}
+
+struct NoCsum {
+  AX_D void operator()(int, float) const {}
+};
+// H = act(sum + b1)
+struct EpiHidden {
+  float *H;
+  const float *b1;
+  int Hd, sym;
+  AX_D void operator()(int b, int h, float a) const {
+    const float v = a + b1[h];
+    H[(size_t)b * Hd + h] = sym ? v : tanhf(v);
+  }
+};
+// dP = sum (1 - H^2) (the symmetric form is linear)
+struct EpiBack {
+  float *dP;
+  const float *H;
+  int Hd, sym;
+  AX_D void operator()(int b, int h, float a) const {
+    const size_t q = (size_t)b * Hd + h;
+    const float hv = H[q];
+    dP[q] = sym ? a : a * (1.f - hv * hv);
+  }
+};
+// row-major [m][h] (W1's gradient; row N is b1's)
+struct EpiRows {
+  float *g;
+  int Hd;
+  AX_D void operator()(int m, int h, float a) const { g[(size_t)m * Hd + h] = a; }
+};
+// transposed [h][m] (W2's gradient), and its bias
+struct EpiCols {
+  float *g;
+  int N;
+  AX_D void operator()(int m, int h, float a) const { g[(size_t)h * N + m] = a; }
+};
+struct CsumBias {
+  float *g;
+  AX_D void operator()(int m, float a) const { g[m] = a; }
+};
+
+// Y(b, o) = sum_h H[b][h] W2[h][o] + b2[o] for kRows rows and 256 outputs a
+// block; fin(b, o, y) receives each.
+template <class Fin>
+AX_D void out_rows(const float *__restrict__ H, const float *__restrict__ theta, int B, int N,
+                   int Hd, Fin fin) {
+  __shared__ float4 Hs[64];
+  const int b0 = blockIdx.x * kRows, o = blockIdx.y * kThreads + threadIdx.x;
+  const float *W2 = theta + (size_t)N * Hd + Hd, *b2 = W2 + (size_t)Hd * N;
+  if (threadIdx.x < Hd * kRows) {
+    const int r = threadIdx.x / Hd, h = threadIdx.x % Hd;
+    reinterpret_cast<float *>(Hs)[h * kRows + r] =
+        b0 + r < B ? H[(size_t)(b0 + r) * Hd + h] : 0.f;
+  }
+  __syncthreads();
+  if (o >= N) return;
+  float acc[kRows] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+  for (int h = 0; h < Hd; ++h) {
+    const float w = __ldg(W2 + (size_t)h * N + o);
+    const float4 v = Hs[h];
+    acc[0] = fmaf(v.x, w, acc[0]);
+    acc[1] = fmaf(v.y, w, acc[1]);
+    acc[2] = fmaf(v.z, w, acc[2]);
+    acc[3] = fmaf(v.w, w, acc[3]);
+  }
+  const float bo = b2[o];
+#pragma unroll
+  for (int r = 0; r < kRows; ++r)
+    if (b0 + r < B) fin(b0 + r, o, acc[r] + bo);
 }
 
 // Y = H W2 + b2; dY = 2 (Y - T) / (B N); per-block partial of sum (Y-T)^2
-__global__ void fwd_out_loss_kernel(float *__restrict__ Y, float *__restrict__ dY,
-                                    const float *__restrict__ H, const float *__restrict__ Tt,
-                                    const float *__restrict__ theta, int B, int N, int Hd,
-                                    double *__restrict__ partials) {
+__global__ void __launch_bounds__(kThreads)
+fwd_out_loss_kernel(float *__restrict__ Y, float *__restrict__ dY, const float *__restrict__ H,
+                    const float *__restrict__ Tt, const float *__restrict__ theta, int B, int N,
+                    int Hd, double *__restrict__ partials) {
   __shared__ double sh[kThreads / 32];
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double l = 0.0;
-  if (q < (int64_t)B * N) {
-    const int b = (int)(q / N), o = (int)(q % N);
-    const float *W2 = theta + (size_t)N * Hd + Hd, *b2 = W2 + (size_t)Hd * N;
-    float a = 0.f;
-    for (int h = 0; h < Hd; ++h) a = fmaf(H[(size_t)b * Hd + h], W2[(size_t)h * N + o], a);
-    const float y = a + b2[o];
+  out_rows(H, theta, B, N, Hd, [&](int b, int o, float y) {
+    const size_t q = (size_t)b * N + o;
     Y[q] = y;
     const float res = y - Tt[q];
     dY[q] = 2.f * res / ((float)B * (float)N);
-    l = (double)res * (double)res;
-  }
+    l += (double)res * (double)res;
+  });
   double v[1] = {l};
   ax::block_sum<1>(v, sh);
-  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
+  if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = v[0];
 }
 
-// Y = H W2 + b2 (training forward without a target)
-__global__ void fwd_out_kernel(float *__restrict__ Y, const float *__restrict__ H,
-                               const float *__restrict__ theta, int B, int N, int Hd) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= (int64_t)B * N) return;
-  const int b = (int)(q / N), o = (int)(q % N);
-  const float *W2 = theta + (size_t)N * Hd + Hd, *b2 = W2 + (size_t)Hd * N;
-  float a = 0.f;
-  for (int h = 0; h < Hd; ++h) a = fmaf(H[(size_t)b * Hd + h], W2[(size_t)h * N + o], a);
-  Y[q] = a + b2[o];
-}
-
-// gW2[h][o] = sum_b H[b][h] dY[b][o]; gb2[o] = sum_b dY[b][o]
-__global__ void grad_w2_kernel(float *__restrict__ grad, const float *__restrict__ H,
-                               const float *__restrict__ dY, int B, int N, int Hd) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float *gW2 = grad + (size_t)N * Hd + Hd, *gb2 = gW2 + (size_t)Hd * N;
-  if (q < (int64_t)Hd * N) {
-    const int h = (int)(q / N), o = (int)(q % N);
-    float a = 0.f;
-    for (int b = 0; b < B; ++b) a = fmaf(H[(size_t)b * Hd + h], dY[(size_t)b * N + o], a);
-    gW2[q] = a;
-  } else if (q < (int64_t)Hd * N + N) {
-    const int o = (int)(q - (int64_t)Hd * N);
-    float a = 0.f;
-    for (int b = 0; b < B; ++b) a += dY[(size_t)b * N + o];
-    gb2[o] = a;
-  }
-}
-
-// dP[b][h] = (sum_o dY[b][o] W2[h][o]) (1 - H[b][h]^2)
-__global__ void back_hidden_kernel(float *__restrict__ dP, const float *__restrict__ dY,
-                                   const float *__restrict__ H, const float *__restrict__ theta,
-                                   int B, int N, int Hd, int sym) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= (int64_t)B * Hd) return;
-  const int b = (int)(q / Hd), h = (int)(q % Hd);
-  const float *W2 = theta + (size_t)N * Hd + Hd;
-  float a = 0.f;
-  for (int o = 0; o < N; ++o) a = fmaf(dY[(size_t)b * N + o], W2[(size_t)h * N + o], a);
-  const float hv = H[q];
-  dP[q] = sym ? a : a * (1.f - hv * hv);
-}
-
-// gW1[k][h] = sum_b X[b][k] dP[b][h]; gb1[h] = sum_b dP[b][h]
-__global__ void grad_w1_kernel(float *__restrict__ grad, const float *__restrict__ X,
-                               const float *__restrict__ dP, int B, int N, int Hd) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float *gb1 = grad + (size_t)N * Hd;
-  if (q < (int64_t)N * Hd) {
-    const int k = (int)(q / Hd), h = (int)(q % Hd);
-    float a = 0.f;
-    for (int b = 0; b < B; ++b) a = fmaf(X[(size_t)b * N + k], dP[(size_t)b * Hd + h], a);
-    grad[q] = a;
-  } else if (q < (int64_t)N * Hd + Hd) {
-    const int h = (int)(q - (int64_t)N * Hd);
-    float a = 0.f;
-    for (int b = 0; b < B; ++b) a += dP[(size_t)b * Hd + h];
-    gb1[h] = a;
-  }
+// The energy-norm training's forward: corr = osc[q] s_b Y(b, o) (fp64), the
+// element's scaled output before assembly
+__global__ void __launch_bounds__(kThreads)
+fwd_out_corr_kernel(double *__restrict__ corr, const float *__restrict__ H,
+                    const float *__restrict__ theta, const double *__restrict__ osc,
+                    const double *__restrict__ s, int B, int N, int Hd) {
+  out_rows(H, theta, B, N, Hd, [&](int b, int o, float y) {
+    const size_t q = (size_t)b * N + o;
+    corr[q] = osc[q] * s[b] * (double)y;
+  });
 }
 
 __global__ void adam_kernel(float *__restrict__ theta, float *__restrict__ m,
@@ -501,6 +639,23 @@ __global__ void adam_kernel(float *__restrict__ theta, float *__restrict__ m,
   m[q] = mq;
   v[q] = vq;
   theta[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
+}
+
+// Adam of the symmetric form: the free parameters are W1 (W2 = W1^T, zero
+// biases); each thread updates one and writes its mirror image
+__global__ void adam_sym_kernel(float *__restrict__ theta, float *__restrict__ m,
+                                float *__restrict__ v, const float *__restrict__ g, int N, int Hd,
+                                float lr, float b1, float b2, float eps, float c1, float c2) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (int64_t)N * Hd) return;
+  const float gq = g[q];
+  const float mq = b1 * m[q] + (1.f - b1) * gq;
+  const float vq = b2 * v[q] + (1.f - b2) * gq * gq;
+  m[q] = mq;
+  v[q] = vq;
+  const float t = theta[q] - lr * (mq / c1) / (sqrtf(vq / c2) + eps);
+  theta[q] = t;
+  theta[(size_t)N * Hd + Hd + (size_t)(q % Hd) * N + q / Hd] = t;
 }
 
 // bf16 inference copy: W1T [HP][NP], b1 [HP] (fp32), W2T [NP][HP], b2 [NP] (fp32)
@@ -553,6 +708,12 @@ int refresh_bf16(ax_mlp *M, cudaStream_t st) {
   return ax::launch_status();
 }
 
+inline unsigned blocks_of(int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads); }
+inline dim3 out_grid(int B, int N) {
+  return dim3((unsigned)((B + kRows - 1) / kRows), (unsigned)((N + kThreads - 1) / kThreads));
+}
+inline unsigned row_blocks(int M) { return (unsigned)((M + kRows - 1) / kRows); }
+
 int ensure_capacity(ax_mlp *M, int B) {
   if (B <= M->cap) return AX_OK;
   cudaFree(M->X);
@@ -562,12 +723,15 @@ int ensure_capacity(ax_mlp *M, int B) {
   cudaFree(M->dY);
   cudaFree(M->dP);
   cudaFree(M->partials);
+  cudaFree(M->es);
   M->cap = 0;
   const size_t bn = (size_t)B * M->n_in, bh = (size_t)B * M->n_hid;
-  const size_t nblk = (bn + kThreads - 1) / kThreads;
+  const dim3 og = out_grid(B, M->n_in);
+  const size_t nblk = (size_t)og.x * og.y;
   if (cudaMalloc(&M->X, bn * 4) != cudaSuccess || cudaMalloc(&M->T, bn * 4) != cudaSuccess ||
       cudaMalloc(&M->Y, bn * 4) != cudaSuccess || cudaMalloc(&M->dY, bn * 4) != cudaSuccess ||
       cudaMalloc(&M->H, bh * 4) != cudaSuccess || cudaMalloc(&M->dP, bh * 4) != cudaSuccess ||
+      cudaMalloc(&M->es, (size_t)B * 8) != cudaSuccess ||
       cudaMalloc(&M->partials, nblk * 8) != cudaSuccess) {
     (void)cudaGetLastError();
     return AX_ENOMEM;
@@ -576,22 +740,6 @@ int ensure_capacity(ax_mlp *M, int B) {
   return AX_OK;
 }
 
-// tied weights: gW1[k][h] += gW2[h][k]; gb1 = 0
-__global__ void tie_grad_kernel(float *__restrict__ grad, int N, int Hd) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const float *gW2 = grad + (size_t)N * Hd + Hd;
-  if (q < (int64_t)N * Hd) {
-    const int k = (int)(q / Hd), h = (int)(q % Hd);
-    grad[q] += gW2[(size_t)h * N + k];
-  } else if (q < (int64_t)N * Hd + Hd) {
-    grad[q] = 0.f;
-  }
-}
-// zero the W2 and b2 gradients (after tie_grad_kernel has read them)
-__global__ void zero_tail_kernel(float *__restrict__ grad, int64_t from, int64_t n) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < n - from) grad[from + q] = 0.f;
-}
 // W2 = W1^T, b1 = b2 = 0
 __global__ void tie_params_kernel(float *__restrict__ theta, int N, int Hd) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -619,30 +767,63 @@ __global__ void sum_partials_kernel2(const double *__restrict__ p, int n, double
   ax::warp_sum_partials<1>(p, n, out);
 }
 
-// forward + loss + full gradient on M->X / M->T (B samples)
+// H = act(X W1 + b1)
+void launch_hidden(ax_mlp *M, int B, cudaStream_t st) {
+  const int N = M->n_in, Hd = M->n_hid;
+  skinny_kernel<false, false, false, false><<<row_blocks(B), kThreads, 0, st>>>(
+      M->X, M->theta, nullptr, nullptr, B, N, Hd, N, Hd,
+      EpiHidden{M->H, M->theta + (size_t)N * Hd, Hd, M->arch == AX_MLP_SYM}, NoCsum{});
+}
+
+// Gradient from M->X, M->H, M->dY.  Tanh form: all four blocks.  Symmetric
+// form: the gradient of the free parameters W1 (W2's folded in: both are
+// [N][Hd] sums over the rows, X^T dP + dY^T H); the rest of M->grad is zero
+// from the start and stays so.
+void launch_backward(ax_mlp *M, int B, cudaStream_t st) {
+  const int N = M->n_in, Hd = M->n_hid;
+  const float *W2 = M->theta + (size_t)N * Hd + Hd;
+  if (M->arch == AX_MLP_SYM) {
+    // W2 = W1^T, so the back product reads W1's coalesced rows
+    skinny_kernel<false, false, false, false><<<row_blocks(B), kThreads, 0, st>>>(
+        M->dY, M->theta, nullptr, nullptr, B, N, Hd, N, Hd, EpiBack{M->dP, M->H, Hd, 1},
+        NoCsum{});
+    skinny_kernel<true, false, false, false><<<row_blocks(N), kThreads, 0, st>>>(
+        M->X, M->dP, M->dY, M->H, N, B, Hd, N, Hd, EpiRows{M->grad, Hd}, NoCsum{});
+    return;
+  }
+  float *gW2 = M->grad + (size_t)N * Hd + Hd;
+  skinny_kernel<true, false, false, true><<<row_blocks(N), kThreads, 0, st>>>(
+      M->dY, M->H, nullptr, nullptr, N, B, Hd, N, Hd, EpiCols{gW2, N},
+      CsumBias{gW2 + (size_t)Hd * N});
+  skinny_kernel<false, true, false, false><<<row_blocks(B), kThreads, 0, st>>>(
+      M->dY, W2, nullptr, nullptr, B, N, Hd, N, N, EpiBack{M->dP, M->H, Hd, 0}, NoCsum{});
+  skinny_kernel<true, false, true, false><<<row_blocks(N + 1), kThreads, 0, st>>>(
+      M->X, M->dP, nullptr, nullptr, N + 1, B, Hd, N, Hd, EpiRows{M->grad, Hd}, NoCsum{});
+}
+
+// forward + loss + gradient on M->X / M->T (B samples)
 int loss_grad_dev(ax_mlp *M, int B, cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
-  auto blocks = [](int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads); };
-  const int64_t bn = (int64_t)B * N, bh = (int64_t)B * Hd;
-  fwd_hidden_kernel<<<blocks(bh), kThreads, 0, st>>>(M->H, M->X, M->theta, B, N, Hd, M->arch);
-  fwd_out_loss_kernel<<<blocks(bn), kThreads, 0, st>>>(M->Y, M->dY, M->H, M->T, M->theta, B, N,
-                                                       Hd, M->partials);
-  sum_partials_kernel2<<<1, 32, 0, st>>>(M->partials, (int)blocks(bn), M->loss_dev);
-  grad_w2_kernel<<<blocks((int64_t)Hd * N + N), kThreads, 0, st>>>(M->grad, M->H, M->dY, B, N,
-                                                                    Hd);
-  back_hidden_kernel<<<blocks(bh), kThreads, 0, st>>>(M->dP, M->dY, M->H, M->theta, B, N, Hd,
-                                                     M->arch);
-  grad_w1_kernel<<<blocks((int64_t)N * Hd + Hd), kThreads, 0, st>>>(M->grad, M->X, M->dP, B, N,
-                                                                    Hd);
+  launch_hidden(M, B, st);
+  const dim3 og = out_grid(B, N);
+  fwd_out_loss_kernel<<<og, kThreads, 0, st>>>(M->Y, M->dY, M->H, M->T, M->theta, B, N, Hd,
+                                               M->partials);
+  sum_partials_kernel2<<<1, 32, 0, st>>>(M->partials, (int)(og.x * og.y), M->loss_dev);
+  launch_backward(M, B, st);
   return ax::launch_status();
 }
 
+// Adam on M->grad (symmetric form: the tied parameters together)
 int adam_dev(ax_mlp *M, float lr, float b1, float b2, float eps, cudaStream_t st) {
   M->adam_step += 1;
   const float c1 = 1.f - powf(b1, (float)M->adam_step);
   const float c2 = 1.f - powf(b2, (float)M->adam_step);
-  adam_kernel<<<(unsigned)((M->nparam + 255) / 256), 256, 0, st>>>(
-      M->theta, M->m, M->v, M->grad, M->nparam, lr, b1, b2, eps, c1, c2);
+  if (M->arch == AX_MLP_SYM)
+    adam_sym_kernel<<<blocks_of((int64_t)M->n_in * M->n_hid), kThreads, 0, st>>>(
+        M->theta, M->m, M->v, M->grad, M->n_in, M->n_hid, lr, b1, b2, eps, c1, c2);
+  else
+    adam_kernel<<<blocks_of(M->nparam), kThreads, 0, st>>>(M->theta, M->m, M->v, M->grad,
+                                                           M->nparam, lr, b1, b2, eps, c1, c2);
   return ax::launch_status();
 }
 
@@ -650,28 +831,33 @@ int adam_dev(ax_mlp *M, float lr, float b1, float b2, float eps, cudaStream_t st
 
 namespace ax {
 
-int mlp_reserve(ax_mlp *M, int B) { return ensure_capacity(M, B); }
+int mlp_reserve(ax_mlp *M, int B, int pairs) {
+  if (int rc = ensure_capacity(M, B)) return rc;
+  if (pairs <= M->kcap) return AX_OK;
+  cudaFree(M->ek);
+  M->ek = nullptr;
+  M->kcap = 0;
+  if (cudaMalloc(&M->ek, (2 + ax::kRedBlocks) * (size_t)pairs * sizeof(double)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return AX_ENOMEM;
+  }
+  M->kcap = pairs;
+  return AX_OK;
+}
 
-// H, Y from M->X for B rows (fp32 training forward)
-int mlp_train_forward(ax_mlp *M, int B, cudaStream_t st) {
+// M->X -> H, then corr = osc s_b Y in fp64 (B rows)
+int mlp_train_forward_corr(ax_mlp *M, int B, double *corr, const double *osc, const double *s,
+                           cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
-  auto blocks = [](int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads); };
-  fwd_hidden_kernel<<<blocks((int64_t)B * Hd), kThreads, 0, st>>>(M->H, M->X, M->theta, B, N,
-                                                                  Hd, M->arch);
-  fwd_out_kernel<<<blocks((int64_t)B * N), kThreads, 0, st>>>(M->Y, M->H, M->theta, B, N, Hd);
+  launch_hidden(M, B, st);
+  fwd_out_corr_kernel<<<out_grid(B, N), kThreads, 0, st>>>(corr, M->H, M->theta, osc, s, B, N,
+                                                           Hd);
   return launch_status();
 }
 
 // gradient from M->X, M->H and the output gradient M->dY (B rows)
 int mlp_train_backward(ax_mlp *M, int B, cudaStream_t st) {
-  const int N = M->n_in, Hd = M->n_hid;
-  auto blocks = [](int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads); };
-  grad_w2_kernel<<<blocks((int64_t)Hd * N + N), kThreads, 0, st>>>(M->grad, M->H, M->dY, B, N,
-                                                                    Hd);
-  back_hidden_kernel<<<blocks((int64_t)B * Hd), kThreads, 0, st>>>(M->dP, M->dY, M->H, M->theta,
-                                                                   B, N, Hd, M->arch);
-  grad_w1_kernel<<<blocks((int64_t)N * Hd + Hd), kThreads, 0, st>>>(M->grad, M->X, M->dP, B, N,
-                                                                    Hd);
+  launch_backward(M, B, st);
   return launch_status();
 }
 
@@ -680,15 +866,6 @@ int mlp_adam_step(ax_mlp *M, float lr, cudaStream_t st) {
 }
 
 int mlp_refresh(ax_mlp *M, cudaStream_t st) { return refresh_bf16(M, st); }
-
-int mlp_tie_grad(ax_mlp *M, cudaStream_t st) {
-  const int N = M->n_in, Hd = M->n_hid;
-  const int64_t n1 = (int64_t)N * Hd + Hd;
-  tie_grad_kernel<<<(unsigned)((n1 + 255) / 256), 256, 0, st>>>(M->grad, N, Hd);
-  const int64_t rest = M->nparam - n1;
-  zero_tail_kernel<<<(unsigned)((rest + 255) / 256), 256, 0, st>>>(M->grad, n1, M->nparam);
-  return launch_status();
-}
 
 int mlp_tie_params(ax_mlp *M, cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
@@ -751,6 +928,8 @@ int ax_mlp_destroy(ax_mlp *M) {
   for (float *p : f) cudaFree(p);
   cudaFree(M->theta_bf);
   cudaFree(M->partials);
+  cudaFree(M->es);
+  cudaFree(M->ek);
   cudaFree(M->loss_dev);
   delete M;
   return AX_OK;
@@ -832,7 +1011,6 @@ int ax_mlp_loss_grad(ax_mlp *M, const float *X, const float *T, int B, double *l
       cudaMemcpyAsync(M->T, T, bn, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return AX_ELAUNCH;
   if ((rc = loss_grad_dev(M, B, st))) return rc;
-  if (M->arch == AX_MLP_SYM && (rc = ax::mlp_tie_grad(M, st))) return rc;
   double l = 0.0;
   if (cudaMemcpyAsync(&l, M->loss_dev, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return AX_ELAUNCH;
@@ -849,7 +1027,6 @@ int ax_mlp_adam(ax_mlp *M, float lr, float beta1, float beta2, float eps, void *
   cudaStream_t st = (cudaStream_t)stream;
   int rc = adam_dev(M, lr, beta1, beta2, eps, st);
   if (rc) return rc;
-  if (M->arch == AX_MLP_SYM && (rc = ax::mlp_tie_params(M, st))) return rc;
   return refresh_bf16(M, st);
 }
 
@@ -874,9 +1051,7 @@ int ax_mlp_train(ax_mlp *M, const float *X_all, const float *T_all, int nsamples
       gather_rows_kernel<<<batch, kThreads, 0, st>>>(M->X, M->T, X_all, T_all,
                                                      perm + (size_t)ep * nsamples + s0, M->n_in);
       if ((rc = loss_grad_dev(M, batch, st))) return rc;
-      if (M->arch == AX_MLP_SYM && (rc = ax::mlp_tie_grad(M, st))) return rc;
       if ((rc = adam_dev(M, lr, 0.9f, 0.999f, 1e-8f, st))) return rc;
-      if (M->arch == AX_MLP_SYM && (rc = ax::mlp_tie_params(M, st))) return rc;
     }
   }
   if ((rc = refresh_bf16(M, st))) return rc;

@@ -19,6 +19,9 @@ struct ax_mlp {
   int cap = 0;
   float *X = nullptr, *T = nullptr, *H = nullptr, *Y = nullptr, *dY = nullptr, *dP = nullptr;
   double *partials = nullptr;
+  double *es = nullptr;  // energy training: each row's scale s_e (cap of them)
+  double *ek = nullptr;  // energy training, kcap pairs: ||e||_A^2, losses, their partials
+  int kcap = 0;
   double *loss_dev = nullptr;
 };
 
@@ -30,15 +33,15 @@ inline int64_t mlp_off_w2(const ax_mlp *M) { return mlp_off_b1(M) + M->n_hid; }
 inline int64_t mlp_off_b2(const ax_mlp *M) { return mlp_off_w2(M) + (int64_t)M->n_hid * M->n_in; }
 
 // Training internals (fp32, on the workspace of ax_mlp):
-int mlp_reserve(ax_mlp *M, int B);                          // workspace for B rows
-int mlp_train_forward(ax_mlp *M, int B, cudaStream_t st);   // X -> H, Y
-int mlp_train_backward(ax_mlp *M, int B, cudaStream_t st);  // X, H, dY -> grad
+int mlp_reserve(ax_mlp *M, int B, int pairs);               // workspace for B rows
+// X -> H, corr = osc .* s_b .* Y (fp64)
+int mlp_train_forward_corr(ax_mlp *M, int B, double *corr, const double *osc, const double *s,
+                           cudaStream_t st);
+// X, H, dY -> grad (symmetric form: of the tied parameters, in W1's place)
+int mlp_train_backward(ax_mlp *M, int B, cudaStream_t st);
 int mlp_adam_step(ax_mlp *M, float lr, cudaStream_t st);    // theta -= Adam(grad)
 int mlp_refresh(ax_mlp *M, cudaStream_t st);                // bf16 inference copy
-// Symmetric form: fold the W2 gradient into W1 (tied weights), zero the rest;
-// and re-tie the parameters (W2 = W1^T, zero biases) after an update.
-int mlp_tie_grad(ax_mlp *M, cudaStream_t st);
-int mlp_tie_params(ax_mlp *M, cudaStream_t st);
+int mlp_tie_params(ax_mlp *M, cudaStream_t st);             // W2 = W1^T, zero biases
 
 // corr[q] = mask[q] * c[q] * s_e * y_e[q - e*n] for every element e, where
 // y_e = MLP(x_e), x_e = (minv .* r)_e / s_e, s_e = ||(minv .* r)_e||_2
