@@ -68,20 +68,19 @@ int eop_launch_t(const EopArgs &a, cudaStream_t st) {
   m.dx = a.dx;
   m.dxt = a.dxt;
   m.drop = a.drop;
-  eop::EopUpd up{a.pw, a.r, a.minv, a.corr, 0.0, false};
+  eop::EopUpd up{a.pw, a.r, a.minv, a.corr, a.x, 0.0, 0.0, false};
   if constexpr (!DOT && !PUPD) {
     if (a.drop >= 0) {  // testing aid: same grid, its own instantiation
       cudaFuncSetAttribute(eop::ax_eop_kernel<LX, false, false, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
       eop::ax_eop_kernel<LX, false, false, true><<<grid, C::NTB, C::SMEM, st>>>(
-          m, (long long)a.nelv, a.err, a.dotp, eop::EopUpd{a.pw, a.r, a.minv, a.corr, 0.0, false},
-          a.beta, a.use_corr);
+          m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr, a.alpha);
       return launch_status();
     }
   }
   eop::ax_eop_kernel<LX, DOT, PUPD><<<grid, C::NTB, C::SMEM, st>>>(m, (long long)a.nelv, a.err,
                                                                   a.dotp, up, a.beta,
-                                                                  a.use_corr);
+                                                                  a.use_corr, a.alpha);
   return launch_status();
 }
 
@@ -187,7 +186,7 @@ int eopr_launch(int lx, double *w, const double *u, const double *dx, const doub
 
 int eop_launch(int lx, const EopArgs &a, cudaStream_t st) {
   if (a.pw && !(a.dotp && a.r && a.minv && a.beta)) return AX_EINVAL;
-  if (a.corr && !a.use_corr) return AX_EINVAL;
+  if ((a.corr && !a.use_corr) || (a.x && !a.alpha)) return AX_EINVAL;
   switch (lx) {
     case 6: return eop_launch_lx<6>(a, st);
     case 8: return eop_launch_lx<8>(a, st);

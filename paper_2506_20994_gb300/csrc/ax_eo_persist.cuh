@@ -179,11 +179,15 @@ struct EopMesh {
 };
 
 // Solver operands of the fused direction update (PUPD): pw = minv .* r
-// (+ corr when use_corr) + beta pw, formed in place in front of the apply.
+// (+ corr when use_corr) + beta pw, formed in place in front of the apply;
+// x (may be null) += alpha pw with the old pw: the previous step's solution
+// update, whose read of pw is this one's (at 56 % of HBM the apply has the
+// bandwidth to spare that the solver's vector kernels lack).
 struct EopUpd {
   double *pw;
   const double *r, *minv, *corr;
-  double beta;
+  double *x;
+  double alpha, beta;
   bool use_corr;
 };
 
@@ -422,6 +426,15 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     // lines of the three directions; the next element's inputs start loading
     double ucur[2][2];
     unsigned uk = 0u;
+    double xv[2][2];
+    if constexpr (PUPD) {
+      if (real && up.x) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+          for (int a = 0; a < 2; ++a) xv[b][a] = up.x[eb + pidx(b, a)];
+      }
+    }
 #pragma unroll
     for (int b = 0; b < 2; ++b)
 #pragma unroll
@@ -441,6 +454,15 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     for (int b = 0; b < 2; ++b)
 #pragma unroll
       for (int a = 0; a < 2; ++a) v[b][a] = split(ucur[b][a]);
+    if constexpr (PUPD) {
+      if (real && up.x) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+          for (int a = 0; a < 2; ++a)
+            up.x[eb + pidx(b, a)] = __fma_rn(up.alpha, pv[b][a], xv[b][a]);
+      }
+    }
     if (real && more) load_in(nxp);
     uk = __reduce_max_sync(0xffffffffu, real ? uk : 0u);
     if ((tid & 31) == 0) kslot[tid >> 5] = uk;
@@ -533,6 +555,9 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     if (tid == 0 && more) {
       fence_async_smem();
       issue_geo(nxp);
+      if constexpr (PUPD) {
+        if (up.x) prefetch_l2(up.x + (size_t)seq.elem(nxp) * N3, N3 * 8);
+      }
     }
     unsigned uke = 0u;
 #pragma unroll
@@ -597,12 +622,14 @@ template <int LX, bool DOT, bool PUPD, bool DROP = false>
 __global__ void __launch_bounds__(Cfg<LX>::NTB, Cfg<LX>::MINB)
 ax_eop_kernel(const EopMesh mesh, long long nelv, int *__restrict__ err,
               double *__restrict__ dotp, const EopUpd up0,
-              const double *__restrict__ beta_p, const int *__restrict__ use_corr_p) {
+              const double *__restrict__ beta_p, const int *__restrict__ use_corr_p,
+              const double *__restrict__ alpha_p) {
   using C = Cfg<LX>;
   extern __shared__ __align__(128) unsigned char sm[];
   EopUpd up = up0;
   if constexpr (PUPD) {  // solver scalars live on the device
     up.beta = *beta_p;
+    if (up.x) up.alpha = *alpha_p;
     up.use_corr = up.corr != nullptr && *use_corr_p != 0;
   }
   const SeqOne seq{mesh, nelv};
@@ -631,7 +658,7 @@ ax_eopr_kernel(const EopMesh mesh, long long nelv) {
   extern __shared__ __align__(128) unsigned char sm[];
   const SeqOne seq{mesh, nelv};
   double dsum = 0.0;
-  const EopUpd none{nullptr, nullptr, nullptr, nullptr, 0.0, false};
+  const EopUpd none{};
   eop_run<LX, false, false, true>(
       sm, (int)threadIdx.x, seq, [] { __syncthreads(); },
       [](bool p) { return __syncthreads_and(p) != 0; }, nullptr, none, dsum);

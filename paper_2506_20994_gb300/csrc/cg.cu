@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "dispatch.h"
+#include "gs.h"
 #include "op.h"
 #include "mlp.cuh"
 #include "reduce.cuh"
@@ -37,13 +38,7 @@ namespace {
 using ax::kRedBlocks;
 using ax::kRedThreads;
 
-// Device-side scalars of one CG run.
-struct CgScalars {
-  double rz, rz_new, rr, rr0, pap, alpha, beta;
-  int status;     // 0 ok, 1 breakdown (p.Ap <= 0 or non-finite)
-  int use_corr;   // flexible CG: 1 if the learned correction is in z
-  int fallbacks;  // flexible CG: steps that fell back to Jacobi
-};
+using ax::CgScalars;
 
 // ---------------------------------------------------------------- kernels
 template <typename... P>
@@ -96,12 +91,13 @@ __global__ void sqrt_minv_kernel(float *__restrict__ sqm, const double *__restri
     sqm[q] = sqrtf(ax::df::split(minv[q]).hi);
 }
 
-// r = b (masked), p = minv r; partials: rz = sum cm r^2, rr = sum c r^2
+// r = b (masked), p = minv r; rz = sum cm r^2, rr = rr0 = sum c r^2
 template <typename T>
 __global__ void cg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ p,
                                const T *__restrict__ b, const T *__restrict__ mask,
                                const T *__restrict__ minv, const T *__restrict__ c,
-                               double *__restrict__ partials, int64_t n) {
+                               CgScalars *__restrict__ s, double *__restrict__ partials,
+                               int64_t n) {
   __shared__ double sh[2 * kRedThreads / 32];
   T a_rz = 0, a_rr = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
@@ -117,17 +113,21 @@ __global__ void cg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restri
   }
   double v[2] = {(double)a_rz, (double)a_rr};
   ax::block_sum<2>(v, sh);
-  if (threadIdx.x == 0) {
-    partials[blockIdx.x] = v[0];
-    partials[gridDim.x + blockIdx.x] = v[1];
-  }
+  ax::finish_sums<2>(v, partials, &s->ticket, [s](const double *t) {
+    s->rz = t[0];
+    s->rr = t[1];
+    s->rr0 = t[1];
+    s->beta = 0.0;
+    s->status = 0;
+  });
 }
 
-// w = mask .* w; partial sum of c p w
+// w = mask .* w; partial sums of c p w; s, if given: alpha from them
 template <typename T>
 __global__ void mask_dot_kernel(T *__restrict__ w, const T *__restrict__ p,
                                 const T *__restrict__ mask, const T *__restrict__ c,
-                                double *__restrict__ partials, int64_t n) {
+                                double *__restrict__ partials, int64_t n,
+                                CgScalars *__restrict__ s = nullptr) {
   __shared__ double sh[kRedThreads / 32];
   T a = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
@@ -138,50 +138,27 @@ __global__ void mask_dot_kernel(T *__restrict__ w, const T *__restrict__ p,
   }
   double v[1] = {(double)a};
   ax::block_sum<1>(v, sh);
-  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
+  if (s)  // kernel-uniform
+    ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) { ax::cg_set_alpha(s, t[0]); });
+  else if (threadIdx.x == 0)
+    partials[blockIdx.x] = v[0];
 }
 
-// alpha = rz / <p, Ap> from the partials (one warp for the fixed-grid
-// partials; a whole block for the per-element-block partials of the fused
-// apply)
-__global__ void cg_alpha_kernel(const double *__restrict__ partials, int nblk,
-                                CgScalars *__restrict__ s) {
-  __shared__ double t[32];
-  double pap_all;
-  if (blockDim.x == 32) {
-    ax::warp_sum_partials<1>(partials, nblk, t);
-    __syncthreads();
-    pap_all = t[0];
-  } else {
-    pap_all = ax::block_sum_partials(partials, nblk, t);
-  }
-  if (threadIdx.x == 0) {
-    const double pap = pap_all;
-    s->pap = pap;
-    if (!(pap > 0.0) || !isfinite(pap) || !isfinite(s->rz)) {
-      s->status = 1;
-      s->alpha = 0.0;
-    } else {
-      s->alpha = s->rz / pap;
-    }
-  }
-}
-
-// x += alpha p; r -= alpha w; partials rz' = sum cm r^2, rr' = sum c r^2
-// MASKW: w is not masked yet (fused apply); the Dirichlet rows, where
-// cm = c * minv is 0, keep r = 0.  RR: also the rr partials; rr only feeds
-// the host's convergence test, so iterations it does not check skip that sum
-// and the read of c (their rr partials are written as 0).
-template <typename T, bool MASKW = false, bool RR = true>
+// x += alpha p; r -= alpha w; rz' = sum cm r^2, beta = rz' / rz and (RR)
+// rr' = sum c r^2.  XUP: x is updated here (else by the next apply, which
+// reads p anyway; x and p are then not touched).  MASKW: w is not masked yet (fused apply); the Dirichlet rows, where
+// cm = c * minv is 0, keep r = 0.  RR: rr only feeds the host's convergence
+// test, so iterations it does not check skip that sum and the read of c.
+template <typename T, bool MASKW = false, bool RR = true, bool XUP = true>
 __global__ void cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
                                  const T *__restrict__ w, const T *__restrict__ cm,
-                                 const T *__restrict__ c, const CgScalars *__restrict__ s,
+                                 const T *__restrict__ c, CgScalars *__restrict__ s,
                                  double *__restrict__ partials, int64_t n) {
   __shared__ double sh[2 * kRedThreads / 32];
   const T alpha = (T)s->alpha;
   T a_rz = 0, a_rr = 0;
   auto point = [&](T &xq, T &rq, T pq, T wq, T cmq, T cq) {
-    xq += alpha * pq;
+    if constexpr (XUP) xq += alpha * pq;
     const T rv = (MASKW && cmq == T(0)) ? rq : rq - alpha * wq;
     rq = rv;
     const T r2 = rv * rv;
@@ -195,15 +172,16 @@ __global__ void cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *
       const int64_t n4 = n / 4;
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
            v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = reinterpret_cast<V *>(x)[v], rv = reinterpret_cast<V *>(r)[v];
-        const V pv = reinterpret_cast<const V *>(p)[v], wv = reinterpret_cast<const V *>(w)[v];
+        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v];
+        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
+        const V wv = reinterpret_cast<const V *>(w)[v];
         const V mv = reinterpret_cast<const V *>(cm)[v];
         const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.f, 0.f, 0.f, 0.f};
         point(xv.x, rv.x, pv.x, wv.x, mv.x, cv.x);
         point(xv.y, rv.y, pv.y, wv.y, mv.y, cv.y);
         point(xv.z, rv.z, pv.z, wv.z, mv.z, cv.z);
         point(xv.w, rv.w, pv.w, wv.w, mv.w, cv.w);
-        reinterpret_cast<V *>(x)[v] = xv;
+        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
         reinterpret_cast<V *>(r)[v] = rv;
       }
       q0 = n4 * 4;
@@ -216,49 +194,42 @@ __global__ void cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *
       const int64_t n2 = n / 2;
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n2;
            v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = reinterpret_cast<V *>(x)[v], rv = reinterpret_cast<V *>(r)[v];
-        const V pv = reinterpret_cast<const V *>(p)[v], wv = reinterpret_cast<const V *>(w)[v];
+        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v];
+        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
+        const V wv = reinterpret_cast<const V *>(w)[v];
         const V mv = reinterpret_cast<const V *>(cm)[v];
         const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.0, 0.0};
         point(xv.x, rv.x, pv.x, wv.x, mv.x, cv.x);
         point(xv.y, rv.y, pv.y, wv.y, mv.y, cv.y);
-        reinterpret_cast<V *>(x)[v] = xv;
+        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
         reinterpret_cast<V *>(r)[v] = rv;
       }
       q0 = n2 * 2;
     }
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * blockDim.x)
-    point(x[q], r[q], p[q], w[q], cm[q], RR ? c[q] : T(0));
+       q += (int64_t)gridDim.x * blockDim.x) {
+    T xq = XUP ? x[q] : T(0);
+    point(xq, r[q], XUP ? p[q] : T(0), w[q], cm[q], RR ? c[q] : T(0));
+    if constexpr (XUP) x[q] = xq;
+  }
   double v[2] = {(double)a_rz, (double)a_rr};
   ax::block_sum<2>(v, sh);
-  if (threadIdx.x == 0) {
-    partials[blockIdx.x] = v[0];
-    partials[gridDim.x + blockIdx.x] = v[1];
-  }
+  ax::finish_sums<2>(v, partials, &s->ticket, [s](const double *t) {
+    s->beta = (s->rz != 0.0) ? t[0] / s->rz : 0.0;
+    s->rz = t[0];
+    s->rr = t[1];
+    if (!isfinite(t[0]) || !isfinite(t[1])) s->status = 1;
+  });
 }
 
-// first=1: rz = partial sums, rr0 = rr.  Otherwise beta = rz'/rz.
-__global__ void cg_beta_kernel(const double *__restrict__ partials, int nblk,
-                               CgScalars *__restrict__ s, int first) {
-  __shared__ double t[2];
-  ax::warp_sum_partials<2>(partials, nblk, t);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (first) {
-      s->rz = t[0];
-      s->rr = t[1];
-      s->rr0 = t[1];
-      s->beta = 0.0;
-      s->status = 0;
-    } else {
-      s->beta = (s->rz != 0.0) ? t[0] / s->rz : 0.0;
-      s->rz = t[0];
-      s->rr = t[1];
-      if (!isfinite(t[0]) || !isfinite(t[1])) s->status = 1;
-    }
-  }
+// x += alpha p (the last step's, when the applies carry the x update)
+__global__ void cg_x_kernel(double *__restrict__ x, const double *__restrict__ p,
+                            const CgScalars *__restrict__ s, int64_t n) {
+  const double alpha = s->alpha;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
+       q += (int64_t)gridDim.x * blockDim.x)
+    x[q] += alpha * p[q];
 }
 
 // p = minv r + beta p
@@ -413,8 +384,10 @@ int apply_f64(ax_poisson *P, double *w, const double *u, cudaStream_t st) {
 
 // dotp: also the per-block partials of u . Ax (P->ndot32 of them)
 // up: the fused direction update (even-odd fp32 kernel only; u = up->pw)
+// alpha: the fused loops' alpha, set by the gather-scatter
 int apply_lowp(ax_poisson *P, float *w, const float *u, cudaStream_t st,
-               double *dotp = nullptr, const ax::E32Upd *up = nullptr) {
+               double *dotp = nullptr, const ax::E32Upd *up = nullptr,
+               const ax::AlphaJob *alpha = nullptr) {
   int rc;
   if (up && !P->lowp_eo32) return AX_EINVAL;
   if (P->lowp_eo32 && P->lowp_mode == 2) {
@@ -444,12 +417,13 @@ int apply_lowp(ax_poisson *P, float *w, const float *u, cudaStream_t st,
   if (rc == AX_OK && P->hb32)  // the mass term's partials follow the kernel's
     rc = ax::mass_add<float>(w, P->hb32, u, P->n, dotp ? dotp + P->ndot32 : nullptr, st);
   if (rc) return rc;
-  return ax_gs_sum_f32(P->gs, w, st);
+  return alpha ? ax::gs_sum_alpha(P->gs, w, *alpha, st) : ax_gs_sum_f32(P->gs, w, st);
 }
 
-// The fused apply of a solver loop: w = gs(Ax(u)) (unmasked) and the
-// partials of u . Ax in P->dotp; returns the number of partials, or 0 when
-// this precision has no fused form (the caller masks and dots separately).
+// The fused apply of a solver loop: w = gs(Ax(u)) (unmasked), the partials of
+// u . Ax in P->dotp and alpha from them; fused_parts returns the number of
+// partials, or 0 when this precision has no fused form (the caller masks and
+// dots separately).
 // (With a mass term its kRedBlocks partials follow the operator's.)
 int fused_parts(const ax_poisson *P, const double *) {
   return P->dotp && P->ndot ? P->ndot + (P->hb ? kRedBlocks : 0) : 0;
@@ -460,37 +434,45 @@ int fused_parts(const ax_poisson *P, const float *) {
 int mass_fused(ax_poisson *P, double *w, const double *u, cudaStream_t st) {
   return P->hb ? ax::mass_add<double>(w, P->hb, u, P->n, P->dotp + P->ndot, st) : AX_OK;
 }
+template <typename T>
+ax::AlphaJob alpha_job(const ax_poisson *P) {
+  return ax::AlphaJob{P->dotp, fused_parts(P, (const T *)nullptr), P->scal};
+}
 int apply_fused(ax_poisson *P, double *w, const double *u, cudaStream_t st) {
   int rc = ax::op_apply_dot(P->op, w, u, P->dotp, st);
   if (rc == AX_OK) rc = mass_fused(P, w, u, st);
-  return rc ? rc : ax_gs_sum(P->gs, w, st);
+  return rc ? rc : ax::gs_sum_alpha(P->gs, w, alpha_job<double>(P), st);
 }
 int apply_fused(ax_poisson *P, float *w, const float *u, cudaStream_t st) {
-  return apply_lowp(P, w, u, st, P->dotp);
+  const ax::AlphaJob job = alpha_job<float>(P);
+  return apply_lowp(P, w, u, st, P->dotp, nullptr, &job);
 }
 // The direction update p = minv r + beta p folded into the apply that reads
 // p next (fp64 with prepared geometry); false where no such kernel exists.
 bool fuses_update(const ax_poisson *P, const double *) { return P->dotp && P->ndot > 0; }
 bool fuses_update(const ax_poisson *P, const float *) { return P->dotp && P->lowp_eo32; }
+// fp64: the previous step's x += alpha p as well, from the old p it reads
 int apply_fused_update(ax_poisson *P, double *w, double *p, const double *r,
-                       const double *minv, const double *beta, cudaStream_t st,
-                       const double *corr = nullptr, const int *use_corr = nullptr) {
-  int rc = ax::op_update_apply_dot(P->op, w, p, r, minv, beta, P->dotp, st, corr, use_corr);
+                       const double *minv, double *x, cudaStream_t st,
+                       const double *corr = nullptr) {
+  const ax::OpUpdate up{p, r, minv, corr, x, &P->scal->alpha, &P->scal->beta,
+                        corr ? &P->scal->use_corr : nullptr};
+  int rc = ax::op_update_apply_dot(P->op, w, up, P->dotp, st);
   if (rc == AX_OK) rc = mass_fused(P, w, p, st);
-  return rc ? rc : ax_gs_sum(P->gs, w, st);
+  return rc ? rc : ax::gs_sum_alpha(P->gs, w, alpha_job<double>(P), st);
 }
 // fp32 vectors (the refinement's inner CG, even-odd fp32 kernel): the same
-// fusion, p = minv .* r + beta p in fp32 inside the apply
+// fusion without x, p = minv .* r + beta p in fp32 inside the apply
 int apply_fused_update(ax_poisson *P, float *w, float *p, const float *r, const float *minv,
-                       const double *beta, cudaStream_t st, const float *corr = nullptr,
-                       const int * = nullptr) {
+                       float *, cudaStream_t st, const float *corr = nullptr) {
   if (corr) return AX_EINVAL;  // the flexible loop keeps its own direction kernel
   ax::E32Upd up;
   up.pw = p;
   up.r = r;
   up.minv = minv;
-  up.beta = beta;
-  return apply_lowp(P, w, p, st, P->dotp, &up);
+  up.beta = &P->scal->beta;
+  const ax::AlphaJob job = alpha_job<float>(P);
+  return apply_lowp(P, w, p, st, P->dotp, &up, &job);
 }
 
 // Generic PCG loop on vectors of type T (fp64 with the fp64 operator, or
@@ -502,8 +484,8 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
              double *relres, cudaStream_t st) {
   const int64_t n = P->n;
   const unsigned nb = kRedBlocks;
-  cg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, p, b, mask, minv, c, P->partials, n);
-  cg_beta_kernel<<<1, 64, 0, st>>>(P->partials, nb, P->scal, 1);
+  cg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, p, b, mask, minv, c, P->scal, P->partials,
+                                               n);
   if (ax::launch_status()) return AX_ELAUNCH;
   if (cudaMemcpyAsync(P->scal_host, P->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost, st) !=
           cudaSuccess ||
@@ -523,35 +505,30 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
   // of p . A_e p), and the mask moves into the update
   const int nparts = fused_parts(P, (const T *)nullptr);
   const bool fused = nparts > 0;
-  // after the first iteration the next direction is formed inside the apply
+  // after the first iteration the next direction is formed inside the apply,
+  // in fp64 together with the x update of the step before
   const bool fused_p = fused && fuses_update(P, (const T *)nullptr);
+  const bool fused_x = fused_p && std::is_same_v<T, double>;
   while (it < maxit) {
     int rc;
     if (fused) {
-      // device address of the beta field (P->scal lives on the device)
-      const double *beta_dev = reinterpret_cast<const double *>(
-          reinterpret_cast<const char *>(P->scal) + offsetof(CgScalars, beta));
-      rc = (fused_p && it > 0) ? apply_fused_update(P, w, p, r, minv, beta_dev, st)
+      rc = (fused_p && it > 0) ? apply_fused_update(P, w, p, r, minv, x, st)
                                : apply_fused(P, w, p, st);
       if (rc) return rc;
-      cg_alpha_kernel<<<1, 1024, 0, st>>>(P->dotp, nparts, P->scal);
       // rr only where the host will test it (after this iteration)
       const bool checked = (it + 1) % P->check_every == 0 || it + 1 == maxit;
-      if (checked)
-        cg_update_kernel<T, true, true><<<nb, kRedThreads, 0, st>>>(x, r, p, w, cm, c, P->scal,
-                                                                    P->partials, n);
-      else
-        cg_update_kernel<T, true, false><<<nb, kRedThreads, 0, st>>>(x, r, p, w, cm, c,
-                                                                     P->scal, P->partials, n);
+      auto update = fused_x ? (checked ? cg_update_kernel<T, true, true, !std::is_same_v<T, double>>
+                                       : cg_update_kernel<T, true, false, !std::is_same_v<T, double>>)
+                            : (checked ? cg_update_kernel<T, true, true, true>
+                                       : cg_update_kernel<T, true, false, true>);
+      update<<<nb, kRedThreads, 0, st>>>(x, r, p, w, cm, c, P->scal, P->partials, n);
     } else {
       rc = apply(w, p, st);
       if (rc) return rc;
-      mask_dot_kernel<T><<<nb, kRedThreads, 0, st>>>(w, p, mask, c, P->partials, n);
-      cg_alpha_kernel<<<1, 32, 0, st>>>(P->partials, nb, P->scal);
+      mask_dot_kernel<T><<<nb, kRedThreads, 0, st>>>(w, p, mask, c, P->partials, n, P->scal);
       cg_update_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, p, w, cm, c, P->scal, P->partials,
                                                       n);
     }
-    cg_beta_kernel<<<1, 64, 0, st>>>(P->partials, nb, P->scal, 0);
     ++it;
     if (it % P->check_every == 0 || it == maxit) {
       if (cudaMemcpyAsync(P->scal_host, P->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost,
@@ -570,6 +547,8 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
     }
     if (!fused_p) cg_p_kernel<T><<<nb, kRedThreads, 0, st>>>(p, r, minv, P->scal, n);
   }
+  if constexpr (std::is_same_v<T, double>)
+    if (fused_x && it > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
   if (ax::launch_status()) return AX_ELAUNCH;
   if (iters) *iters = it;
   if (relres) *relres = rel;
@@ -703,6 +682,7 @@ int ax_poisson_create(ax_poisson **out, int lx, int nelv, const double *dx, cons
     ax_poisson_destroy(P);
     return AX_ENOMEM;
   }
+  cudaMemsetAsync(P->scal, 0, sizeof(CgScalars), st);  // the reductions' ticket starts at zero
   // exact Jacobi diagonal, assembled, then the masked inverse
   jacobi_diag_kernel<<<blocks_for(n, 256), 256, 0, st>>>(P->w, dx, h1, g11, g22, g33, g12, g13,
                                                          g23, lx, n);
@@ -1004,21 +984,21 @@ extern "C" int ax_jacobi_noalloc(double *minv, const double *dx, const double *h
 // ---------------------------------------------------------------------------
 namespace {
 
-// x += alpha p; r_old = r; r -= alpha w; partial rr = sum c r^2.  MASKW: w is
-// not masked yet (fused apply); rows where cm = c * minv is 0 keep r = 0.
-// RR: the rr partials (read by the host's convergence test only); without
-// it the kernel neither reads c nor reduces.
-template <typename T, bool MASKW = false, bool RR = true>
+// x += alpha p (XUP, as in cg_update_kernel); r_old = r; r -= alpha w; rr = sum
+// c r^2.  MASKW: w is not masked yet (fused apply); rows where cm = c * minv
+// is 0 keep r = 0.  RR: rr (read by the host's convergence test only);
+// without it the kernel neither reads c nor reduces.
+template <typename T, bool MASKW = false, bool RR = true, bool XUP = true>
 __global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
                                   const T *__restrict__ p, const T *__restrict__ w,
                                   const T *__restrict__ c, const T *__restrict__ cm,
-                                  const CgScalars *__restrict__ s,
+                                  CgScalars *__restrict__ s,
                                   double *__restrict__ partials, int64_t n) {
   __shared__ double sh[kRedThreads / 32];
   const T alpha = (T)s->alpha;
   T a_rr = 0;
   auto point = [&](T &xq, T &rq, T &roq, T pq, T wq, T cq, T cmq) {
-    xq += alpha * pq;
+    if constexpr (XUP) xq += alpha * pq;
     roq = rq;
     rq = (MASKW && cmq == T(0)) ? rq : rq - alpha * wq;
     if constexpr (RR) a_rr += cq * rq * rq;
@@ -1030,15 +1010,16 @@ __global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__res
       const int64_t n4 = n / 4;
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
            v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = reinterpret_cast<V *>(x)[v], rv = reinterpret_cast<V *>(r)[v], ov;
-        const V pv = reinterpret_cast<const V *>(p)[v], wv = reinterpret_cast<const V *>(w)[v];
+        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v], ov;
+        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
+        const V wv = reinterpret_cast<const V *>(w)[v];
         const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.f, 0.f, 0.f, 0.f};
         const V mv = MASKW ? reinterpret_cast<const V *>(cm)[v] : V{1.f, 1.f, 1.f, 1.f};
         point(xv.x, rv.x, ov.x, pv.x, wv.x, cv.x, mv.x);
         point(xv.y, rv.y, ov.y, pv.y, wv.y, cv.y, mv.y);
         point(xv.z, rv.z, ov.z, pv.z, wv.z, cv.z, mv.z);
         point(xv.w, rv.w, ov.w, pv.w, wv.w, cv.w, mv.w);
-        reinterpret_cast<V *>(x)[v] = xv;
+        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
         reinterpret_cast<V *>(r)[v] = rv;
         reinterpret_cast<V *>(r_old)[v] = ov;
       }
@@ -1050,13 +1031,14 @@ __global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__res
       const int64_t n2 = n / 2;
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n2;
            v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = reinterpret_cast<V *>(x)[v], rv = reinterpret_cast<V *>(r)[v], ov;
-        const V pv = reinterpret_cast<const V *>(p)[v], wv = reinterpret_cast<const V *>(w)[v];
+        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v], ov;
+        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
+        const V wv = reinterpret_cast<const V *>(w)[v];
         const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.0, 0.0};
         const V mv = MASKW ? reinterpret_cast<const V *>(cm)[v] : V{1.0, 1.0};
         point(xv.x, rv.x, ov.x, pv.x, wv.x, cv.x, mv.x);
         point(xv.y, rv.y, ov.y, pv.y, wv.y, cv.y, mv.y);
-        reinterpret_cast<V *>(x)[v] = xv;
+        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
         reinterpret_cast<V *>(r)[v] = rv;
         reinterpret_cast<V *>(r_old)[v] = ov;
       }
@@ -1064,50 +1046,65 @@ __global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__res
     }
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * blockDim.x)
-    point(x[q], r[q], r_old[q], p[q], w[q], RR ? c[q] : T(0), MASKW ? cm[q] : T(1));
+       q += (int64_t)gridDim.x * blockDim.x) {
+    T xq = XUP ? x[q] : T(0);
+    point(xq, r[q], r_old[q], XUP ? p[q] : T(0), w[q], RR ? c[q] : T(0), MASKW ? cm[q] : T(1));
+    if constexpr (XUP) x[q] = xq;
+  }
   if constexpr (RR) {
     double v[1] = {(double)a_rr};
     ax::block_sum<1>(v, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
+    ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) { s->rr = t[0]; });
   }
 }
 
-// partials of <zj, r>, <corr, r>, <zj, r_old>, <corr, r_old> (zj = minv r),
-// weighted by c; with cm = c * minv the Jacobi pair costs 3 multiply-adds and
-// the correction pair 3 more (the fp64 pipe, not memory, bounds this kernel)
+// <zj, r>, <corr, r>, <zj, r_old>, <corr, r_old> (zj = minv r), weighted by c;
+// with cm = c * minv the Jacobi pair costs 3 multiply-adds and the correction
+// pair 3 more (in fp64 the narrow pipe, not memory, bounds this kernel).  From
+// them rz (first: of <z0, r0>, else with Notay's beta) and the choice between
+// the learned and the Jacobi step.  fp32: 16-byte accesses.
 template <typename T>
 __global__ void fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
                                 const T *__restrict__ corr, const T *__restrict__ cm,
-                                const T *__restrict__ c, int have_corr,
-                                double *__restrict__ partials, int64_t n) {
+                                const T *__restrict__ c, int have_corr, int first,
+                                CgScalars *__restrict__ s, double *__restrict__ partials,
+                                int64_t n) {
   __shared__ double sh[4 * kRedThreads / 32];
   T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const T rv = r[q], ro = r_old[q];
-    const T a = cm[q] * rv;
+  auto point = [&](T rv, T ro, T cmv, T cv, T ev) {
+    const T a = cmv * rv;
     d0 += a * rv;
     d2 += a * ro;
     if (have_corr) {
-      const T e = c[q] * corr[q];
+      const T e = cv * ev;
       d1 += e * rv;
       d3 += e * ro;
     }
+  };
+  int64_t q0 = 0;
+  if constexpr (sizeof(T) == 4) {
+    if (aligned16(r, r_old, corr, cm, c)) {
+      using V = float4;
+      const int64_t n4 = n / 4;
+      for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
+           v += (int64_t)gridDim.x * blockDim.x) {
+        auto at = [v](const T *p) { return reinterpret_cast<const V *>(p)[v]; };
+        const V rv = at(r), ro = at(r_old), mv = at(cm);
+        const V cv = have_corr ? at(c) : V{}, ev = have_corr ? at(corr) : V{};
+        point(rv.x, ro.x, mv.x, cv.x, ev.x);
+        point(rv.y, ro.y, mv.y, cv.y, ev.y);
+        point(rv.z, ro.z, mv.z, cv.z, ev.z);
+        point(rv.w, ro.w, mv.w, cv.w, ev.w);
+      }
+      q0 = n4 * 4;
+    }
   }
+  for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
+       q += (int64_t)gridDim.x * blockDim.x)
+    point(r[q], r_old[q], cm[q], have_corr ? c[q] : T(0), have_corr ? corr[q] : T(0));
   double v[4] = {(double)d0, (double)d1, (double)d2, (double)d3};
   ax::block_sum<4>(v, sh);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 4; ++k) partials[k * gridDim.x + blockIdx.x] = v[k];
-}
-
-// first: rz from <z0, r0>; otherwise Notay's beta; choose learned or Jacobi
-__global__ void fcg_beta_kernel(const double *__restrict__ partials, int nblk,
-                                CgScalars *__restrict__ s, int first, int have_corr) {
-  __shared__ double t[4];
-  ax::warp_sum_partials<4>(partials, nblk, t);
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  ax::finish_sums<4>(v, partials, &s->ticket, [s, have_corr, first](const double *t) {
     const double rz_l = t[0] + t[1], rz_j = t[0];
     const double num_l = rz_l - (t[2] + t[3]), num_j = t[0] - t[2];
     const bool ok_l = have_corr && rz_l > 0.0 && isfinite(rz_l) && isfinite(num_l);
@@ -1122,7 +1119,7 @@ __global__ void fcg_beta_kernel(const double *__restrict__ partials, int nblk,
     }
     s->rz = rz;
     if (!isfinite(rz)) s->status = 1;
-  }
+  });
 }
 
 // p = minv r + use_corr * corr + beta p   (first: p = z)
@@ -1166,12 +1163,12 @@ __global__ void fcg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
   }
 }
 
-// init: x = 0, r = mask b, partial rr
+// init: x = 0, r = mask b, rr = rr0
 template <typename T>
 __global__ void fcg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
                                 const T *__restrict__ b, const T *__restrict__ mask,
-                                const T *__restrict__ c, double *__restrict__ partials,
-                                int64_t n) {
+                                const T *__restrict__ c, CgScalars *__restrict__ s,
+                                double *__restrict__ partials, int64_t n) {
   __shared__ double sh[kRedThreads / 32];
   T a = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
@@ -1184,23 +1181,13 @@ __global__ void fcg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restr
   }
   double v[1] = {(double)a};
   ax::block_sum<1>(v, sh);
-  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
-}
-
-__global__ void fcg_rr_kernel(const double *__restrict__ partials, int nblk,
-                              CgScalars *__restrict__ s, int first) {
-  __shared__ double t[1];
-  ax::warp_sum_partials<1>(partials, nblk, t);
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) {
     s->rr = t[0];
-    if (first) {
-      s->rr0 = t[0];
-      s->status = 0;
-      s->fallbacks = 0;
-      s->use_corr = 0;
-    }
-  }
+    s->rr0 = t[0];
+    s->status = 0;
+    s->fallbacks = 0;
+    s->use_corr = 0;
+  });
 }
 
 template <typename T>
@@ -1235,17 +1222,12 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
       if (rc) return rc;
       if ((rc = gs_sum_t<T>(P->gs, corr, st))) return rc;
     }
-    fcg_dots_kernel<T><<<nb, kRedThreads, 0, st>>>(r, r_old, corr, cm, c, have, P->partials,
-                                                   n);
-    fcg_beta_kernel<<<1, 128, 0, st>>>(P->partials, nb, P->scal, first, have);
+    fcg_dots_kernel<T><<<nb, kRedThreads, 0, st>>>(r, r_old, corr, cm, c, have, first, P->scal,
+                                                   P->partials, n);
     if (first || !fused_p)
       fcg_p_kernel<T><<<nb, kRedThreads, 0, st>>>(p, r, minv, corr, P->scal, first, n);
     return ax::launch_status();
   };
-  const char *scal_bytes = reinterpret_cast<const char *>(P->scal);
-  const double *beta_dev =
-      reinterpret_cast<const double *>(scal_bytes + offsetof(CgScalars, beta));
-  const int *use_corr_dev = reinterpret_cast<const int *>(scal_bytes + offsetof(CgScalars, use_corr));
   auto read_scalars = [&]() -> int {
     if (cudaMemcpyAsync(P->scal_host, P->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost, st) !=
             cudaSuccess ||
@@ -1253,8 +1235,7 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
       return AX_ELAUNCH;
     return AX_OK;
   };
-  fcg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, r_old, b, mask, c, P->partials, n);
-  fcg_rr_kernel<<<1, 32, 0, st>>>(P->partials, nb, P->scal, 1);
+  fcg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, r_old, b, mask, c, P->scal, P->partials, n);
   int rc = precondition(1);
   if (rc) return rc;
   if ((rc = read_scalars())) return rc;
@@ -1269,27 +1250,25 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
   while (status != AX_OK && it < maxit) {
     const bool checked = (it + 1) % P->check_every == 0 || it + 1 == maxit;
     if (fused) {
-      rc = (fused_p && applied > 0)
-               ? apply_fused_update(P, w, p, r, minv, beta_dev, st, corr, use_corr_dev)
-               : apply_fused(P, w, p, st);
+      if constexpr (std::is_same_v<T, double>)
+        rc = (fused_p && applied > 0) ? apply_fused_update(P, w, p, r, minv, x, st, corr)
+                                      : apply_fused(P, w, p, st);
+      else
+        rc = apply_fused(P, w, p, st);
       ++applied;
       if (rc) return rc;
-      cg_alpha_kernel<<<1, 1024, 0, st>>>(P->dotp, nparts, P->scal);
       // rr only where the host will test it (after this iteration)
-      if (checked)
-        fcg_update_kernel<T, true, true><<<nb, kRedThreads, 0, st>>>(x, r, r_old, p, w, c, cm,
-                                                                     P->scal, P->partials, n);
-      else
-        fcg_update_kernel<T, true, false><<<nb, kRedThreads, 0, st>>>(x, r, r_old, p, w, c, cm,
-                                                                      P->scal, P->partials, n);
+      auto update = checked ? (fused_p ? fcg_update_kernel<T, true, true, !std::is_same_v<T, double>>
+                                       : fcg_update_kernel<T, true, true, true>)
+                            : (fused_p ? fcg_update_kernel<T, true, false, !std::is_same_v<T, double>>
+                                       : fcg_update_kernel<T, true, false, true>);
+      update<<<nb, kRedThreads, 0, st>>>(x, r, r_old, p, w, c, cm, P->scal, P->partials, n);
     } else {
       if ((rc = apply(w, p, st))) return rc;
-      mask_dot_kernel<T><<<nb, kRedThreads, 0, st>>>(w, p, mask, c, P->partials, n);
-      cg_alpha_kernel<<<1, 32, 0, st>>>(P->partials, nb, P->scal);
+      mask_dot_kernel<T><<<nb, kRedThreads, 0, st>>>(w, p, mask, c, P->partials, n, P->scal);
       fcg_update_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, r_old, p, w, c, cm, P->scal,
                                                        P->partials, n);
     }
-    if (checked || !fused) fcg_rr_kernel<<<1, 32, 0, st>>>(P->partials, nb, P->scal, 0);
     ++it;
     if (it % P->check_every == 0 || it == maxit) {
       if ((rc = read_scalars())) return rc;
@@ -1305,6 +1284,8 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
     }
     if ((rc = precondition(0))) return rc;
   }
+  if constexpr (std::is_same_v<T, double>)
+    if (fused_p && applied > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
   if ((rc = read_scalars())) return rc;
   if (iters) *iters = it;
   if (relres) *relres = rel;

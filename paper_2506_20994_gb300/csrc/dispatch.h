@@ -108,7 +108,8 @@ inline bool df64eo_supported(int lx) { return lx >= 4 && lx <= 12 && lx % 2 == 0
 // (eop_coef_bytes, device); dfield: its matrices' exponent field.  dotp:
 // one partial of u . w per CTA, eop_blocks(lx, nelv, true) of them; pw, r,
 // minv, beta (+ corr, use_corr): the fused direction update, pw = minv .* r
-// (+ corr when *use_corr) + (*beta) pw formed in place before the apply.  err: device word set to 1 if a staged copy never
+// (+ corr when *use_corr) + (*beta) pw formed in place before the apply; x,
+// alpha: with it, x += (*alpha) pw first (the old pw).  err: device word set to 1 if a staged copy never
 // arrived (may be null).
 struct EopArgs {
   double *w = nullptr;
@@ -118,8 +119,9 @@ struct EopArgs {
   const double *dx = nullptr, *dxt = nullptr;
   int dfield = 0, nelv = 0;
   int *err = nullptr;
-  double *dotp = nullptr, *pw = nullptr;
+  double *dotp = nullptr, *pw = nullptr, *x = nullptr;
   const double *r = nullptr, *minv = nullptr, *beta = nullptr, *corr = nullptr;
+  const double *alpha = nullptr;
   const int *use_corr = nullptr;
   long long drop = -1;  // testing aid: element whose geometry copy is not issued
 };

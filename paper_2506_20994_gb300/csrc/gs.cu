@@ -18,6 +18,8 @@
 #include <vector>
 
 #include "common.cuh"
+#include "cg_scalars.cuh"
+#include "gs.h"
 
 struct ax_gs {
   int64_t n_local = 0;
@@ -34,12 +36,44 @@ struct ax_gs {
 
 namespace {
 
-// threads [0, n_pairs): two-copy nodes; then one thread per other node
-template <typename T>
+constexpr int kGsThreads = 256;
+
+// Block 0 of a launch with an alpha job: the partials in the order of a
+// 1024-thread block (virtual thread t adds t, t + 1024, ...; shuffle tree per
+// 32; the 32 sums in order), four virtual threads to each of this block's.
+__device__ __noinline__ void alpha_block(const ax::AlphaJob &job) {
+  __shared__ double sh[32];
+#pragma unroll
+  for (int v = 0; v < 1024 / kGsThreads; ++v) {
+    const int vt = (int)threadIdx.x + v * kGsThreads;
+    double a = 0.0;
+    for (int b = vt; b < job.n; b += 1024) a += __ldg(job.partials + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if ((vt & 31) == 0) sh[vt >> 5] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int k = 0; k < 32; ++k) t += sh[k];
+    ax::cg_set_alpha(job.s, t);
+  }
+}
+
+// threads [0, n_pairs): two-copy nodes; then one thread per other node.
+// ALPHA: block 0 sets the solver's alpha instead (first, so that its chain of
+// sums hides behind the copies; as a launch of its own it cost 3-4 us of each
+// iteration).
+template <typename T, bool ALPHA>
 __global__ void gs_sum_kernel(T *__restrict__ v, const int2 *__restrict__ pairs,
                               int64_t n_pairs, const int *__restrict__ off,
-                              const int *__restrict__ idx, int64_t n_multi) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                              const int *__restrict__ idx, int64_t n_multi,
+                              const ax::AlphaJob job) {
+  if (ALPHA && blockIdx.x == 0) {
+    alpha_block(job);
+    return;
+  }
+  const int64_t s = (int64_t)(blockIdx.x - (ALPHA ? 1 : 0)) * blockDim.x + threadIdx.x;
   if (s < n_pairs) {
     const int2 q = __ldg(pairs + s);
     const T acc = v[q.x] + v[q.y];
@@ -56,18 +90,30 @@ __global__ void gs_sum_kernel(T *__restrict__ v, const int2 *__restrict__ pairs,
 }
 
 template <typename T>
-int gs_sum_launch(ax_gs *g, T *v, cudaStream_t st) {
+int gs_sum_launch(ax_gs *g, T *v, const ax::AlphaJob *job, cudaStream_t st) {
   if (!g) return AX_EINVAL;
-  if (g->n_shared == 0) return AX_OK;
-  if (!v) return AX_EINVAL;
-  const int threads = 256;
-  const unsigned grid = (unsigned)((g->n_shared + threads - 1) / threads);
-  gs_sum_kernel<T><<<grid, threads, 0, st>>>(v, g->d_pairs, g->n_pairs, g->d_off, g->d_idx,
-                                             g->n_multi);
+  if (g->n_shared == 0 && !job) return AX_OK;
+  if (g->n_shared > 0 && !v) return AX_EINVAL;
+  const unsigned grid = (unsigned)((g->n_shared + kGsThreads - 1) / kGsThreads);
+  if (job)
+    gs_sum_kernel<T, true><<<grid + 1, kGsThreads, 0, st>>>(v, g->d_pairs, g->n_pairs, g->d_off,
+                                                            g->d_idx, g->n_multi, *job);
+  else
+    gs_sum_kernel<T, false><<<grid, kGsThreads, 0, st>>>(v, g->d_pairs, g->n_pairs, g->d_off,
+                                                         g->d_idx, g->n_multi, ax::AlphaJob{});
   return ax::launch_status();
 }
 
 }  // namespace
+
+namespace ax {
+int gs_sum_alpha(ax_gs *g, double *v, const AlphaJob &job, cudaStream_t st) {
+  return gs_sum_launch<double>(g, v, &job, st);
+}
+int gs_sum_alpha(ax_gs *g, float *v, const AlphaJob &job, cudaStream_t st) {
+  return gs_sum_launch<float>(g, v, &job, st);
+}
+}  // namespace ax
 
 extern "C" {
 
@@ -180,11 +226,11 @@ int ax_gs_setup(ax_gs **out, const int64_t *glob, int64_t n_local, void *stream)
 }
 
 int ax_gs_sum(ax_gs *g, double *v, void *stream) {
-  return gs_sum_launch<double>(g, v, (cudaStream_t)stream);
+  return gs_sum_launch<double>(g, v, nullptr, (cudaStream_t)stream);
 }
 
 int ax_gs_sum_f32(ax_gs *g, float *v, void *stream) {
-  return gs_sum_launch<float>(g, v, (cudaStream_t)stream);
+  return gs_sum_launch<float>(g, v, nullptr, (cudaStream_t)stream);
 }
 
 int ax_gs_info(const ax_gs *g, int64_t *n_local, int64_t *n_shared, int64_t *n_copies) {

@@ -185,18 +185,21 @@ int op_apply_dot(ax_op *op, double *w, const double *u, double *partials, cudaSt
   return eop_launch(op->lx, a, st);
 }
 
-int op_update_apply_dot(ax_op *op, double *w, double *p, const double *r, const double *minv,
-                        const double *beta, double *partials, cudaStream_t st,
-                        const double *corr, const int *use_corr) {
-  if (!op || !op->gp || !partials || !p || !r || !minv || !beta) return AX_EINVAL;
+int op_update_apply_dot(ax_op *op, double *w, const OpUpdate &up, double *partials,
+                        cudaStream_t st) {
+  if (!op || !op->gp || !partials || !up.p || !up.r || !up.minv || !up.beta ||
+      (up.x && !up.alpha))
+    return AX_EINVAL;
   EopArgs a = eop_args(op, w, nullptr);
   a.dotp = partials;
-  a.pw = p;
-  a.r = r;
-  a.minv = minv;
-  a.beta = beta;
-  a.corr = corr;
-  a.use_corr = use_corr;
+  a.pw = up.p;
+  a.r = up.r;
+  a.minv = up.minv;
+  a.beta = up.beta;
+  a.corr = up.corr;
+  a.use_corr = up.use_corr;
+  a.x = up.x;
+  a.alpha = up.alpha;
   return eop_launch(op->lx, a, st);
 }
 

@@ -67,4 +67,38 @@ AX_D double block_sum_partials(const double *__restrict__ partials, int nblk, do
   return t;
 }
 
+// The second pass inside the first one's kernel: every block stores its NV
+// sums (v, valid in thread 0) as partials[q * gridDim.x + blockIdx.x]; the
+// block that arrives last adds them in index order (one warp per quantity, as
+// warp_sum_partials) and its thread 0 calls f(sums).  `ticket` is zero before
+// the launch and left zero.  A launch of its own for one block costs a kernel
+// boundary and 2 us, in the loops of the solvers once or twice an iteration.
+template <int NV, class F>
+AX_D void finish_sums(double (&v)[NV], double *partials, unsigned *ticket, F f) {
+  __shared__ double t[NV];
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) partials[(size_t)q * gridDim.x + blockIdx.x] = v[q];
+    __threadfence();  // the partials before the ticket
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;  // block-uniform
+  __threadfence();  // the ticket before the other blocks' partials
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q < NV) {
+    double s = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(partials + (size_t)q * gridDim.x + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) t[q] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *ticket = 0u;
+    f(t);
+  }
+}
+
 }  // namespace ax
