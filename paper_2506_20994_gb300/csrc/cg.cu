@@ -38,9 +38,32 @@ namespace {
 using ax::kRedBlocks;
 using ax::kRedThreads;
 
+// The fixed grid of the vector kernels is four blocks per SM: all resident.
+constexpr int kRedPerSm = 4;
+
 using ax::CgScalars;
 
 // ---------------------------------------------------------------- kernels
+// Walks the block-strided vectors v = first, + stride, ... < n two at a time:
+// load(slot, v) for both, then work(slot, v) for both, so that two vectors'
+// loads are in flight before the first one's stores.
+template <class Load, class Work>
+__device__ __forceinline__ void walk2(int64_t n, Load load, Work work) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += 2 * stride) {
+    const bool two = v + stride < n;
+    load(0, v);
+    if (two) load(1, v + stride);
+    work(0, v);
+    if (two) work(1, v + stride);
+  }
+}
+// x == 0 by integer operations: an fp64 comparison occupies the narrow fp64
+// pipe like an addition.
+__device__ __forceinline__ bool is_zero(double x) {
+  return ((unsigned long long)__double_as_longlong(x) << 1) == 0ull;
+}
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.f; }
 template <typename... P>
 __device__ __forceinline__ bool aligned16(const P *...p) {
   return ((reinterpret_cast<uintptr_t>(p) | ...) & 15u) == 0;
@@ -98,7 +121,6 @@ __global__ void cg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restri
                                const T *__restrict__ minv, const T *__restrict__ c,
                                CgScalars *__restrict__ s, double *__restrict__ partials,
                                int64_t n) {
-  __shared__ double sh[2 * kRedThreads / 32];
   T a_rz = 0, a_rr = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -112,7 +134,7 @@ __global__ void cg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restri
     a_rr += cq * rv * rv;
   }
   double v[2] = {(double)a_rz, (double)a_rr};
-  ax::block_sum<2>(v, sh);
+  ax::block_sum<2>(v);
   ax::finish_sums<2>(v, partials, &s->ticket, [s](const double *t) {
     s->rz = t[0];
     s->rr = t[1];
@@ -128,7 +150,6 @@ __global__ void mask_dot_kernel(T *__restrict__ w, const T *__restrict__ p,
                                 const T *__restrict__ mask, const T *__restrict__ c,
                                 double *__restrict__ partials, int64_t n,
                                 CgScalars *__restrict__ s = nullptr) {
-  __shared__ double sh[kRedThreads / 32];
   T a = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -137,7 +158,7 @@ __global__ void mask_dot_kernel(T *__restrict__ w, const T *__restrict__ p,
     a += c[q] * p[q] * wv;
   }
   double v[1] = {(double)a};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   if (s)  // kernel-uniform
     ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) { ax::cg_set_alpha(s, t[0]); });
   else if (threadIdx.x == 0)
@@ -150,61 +171,52 @@ __global__ void mask_dot_kernel(T *__restrict__ w, const T *__restrict__ p,
 // cm = c * minv is 0, keep r = 0.  RR: rr only feeds the host's convergence
 // test, so iterations it does not check skip that sum and the read of c.
 template <typename T, bool MASKW = false, bool RR = true, bool XUP = true>
-__global__ void cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
+__global__ void __launch_bounds__(kRedThreads, kRedPerSm)
+cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
                                  const T *__restrict__ w, const T *__restrict__ cm,
                                  const T *__restrict__ c, CgScalars *__restrict__ s,
                                  double *__restrict__ partials, int64_t n) {
-  __shared__ double sh[2 * kRedThreads / 32];
   const T alpha = (T)s->alpha;
   T a_rz = 0, a_rr = 0;
   auto point = [&](T &xq, T &rq, T pq, T wq, T cmq, T cq) {
     if constexpr (XUP) xq += alpha * pq;
-    const T rv = (MASKW && cmq == T(0)) ? rq : rq - alpha * wq;
+    const T rv = (MASKW && is_zero(cmq)) ? rq : rq - alpha * wq;
     rq = rv;
     const T r2 = rv * rv;
     a_rz += cmq * r2;
     if constexpr (RR) a_rr += cq * r2;
   };
   int64_t q0 = 0;
-  if constexpr (sizeof(T) == 4) {
-    if (aligned16(x, r, p, w, cm, c)) {  // fp32: 16-byte accesses
-      using V = float4;
-      const int64_t n4 = n / 4;
-      for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
-           v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v];
-        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
-        const V wv = reinterpret_cast<const V *>(w)[v];
-        const V mv = reinterpret_cast<const V *>(cm)[v];
-        const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.f, 0.f, 0.f, 0.f};
-        point(xv.x, rv.x, pv.x, wv.x, mv.x, cv.x);
-        point(xv.y, rv.y, pv.y, wv.y, mv.y, cv.y);
-        point(xv.z, rv.z, pv.z, wv.z, mv.z, cv.z);
-        point(xv.w, rv.w, pv.w, wv.w, mv.w, cv.w);
-        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
-        reinterpret_cast<V *>(r)[v] = rv;
-      }
-      q0 = n4 * 4;
-    }
-  } else if constexpr (!RR) {
-    // fp64: 16-byte accesses, two points each (measured faster without the rr
-    // sum, 174 vs 205 us at 16.8 M points; with it, slower: 245 vs 203 us)
+  // 16-byte accesses.  In fp64 with the rr sum, scalar ones measured faster
+  // (203 against 245 us at 16.8 M points)
+  if constexpr (sizeof(T) == 4 || !RR) {
     if (aligned16(x, r, p, w, cm, c)) {
-      using V = double2;
-      const int64_t n2 = n / 2;
-      for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n2;
-           v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v];
-        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
-        const V wv = reinterpret_cast<const V *>(w)[v];
-        const V mv = reinterpret_cast<const V *>(cm)[v];
-        const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.0, 0.0};
-        point(xv.x, rv.x, pv.x, wv.x, mv.x, cv.x);
-        point(xv.y, rv.y, pv.y, wv.y, mv.y, cv.y);
-        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
-        reinterpret_cast<V *>(r)[v] = rv;
-      }
-      q0 = n2 * 2;
+      using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+      constexpr int NV = 16 / sizeof(T);
+      V xv[2], rv[2], pv[2], wv[2], mv[2], cv[2];
+      auto at = [](const T *f, int64_t v) { return reinterpret_cast<const V *>(f)[v]; };
+      walk2(
+          n / NV,
+          [&](int k, int64_t v) {
+            xv[k] = XUP ? at(x, v) : V{};
+            rv[k] = at(r, v);
+            pv[k] = XUP ? at(p, v) : V{};
+            wv[k] = at(w, v);
+            mv[k] = at(cm, v);
+            cv[k] = RR ? at(c, v) : V{};
+          },
+          [&](int k, int64_t v) {
+            T *xs = reinterpret_cast<T *>(&xv[k]), *rs = reinterpret_cast<T *>(&rv[k]);
+            const T *ps = reinterpret_cast<const T *>(&pv[k]);
+            const T *ws = reinterpret_cast<const T *>(&wv[k]);
+            const T *ms = reinterpret_cast<const T *>(&mv[k]);
+            const T *cs = reinterpret_cast<const T *>(&cv[k]);
+#pragma unroll
+            for (int l = 0; l < NV; ++l) point(xs[l], rs[l], ps[l], ws[l], ms[l], cs[l]);
+            if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv[k];
+            reinterpret_cast<V *>(r)[v] = rv[k];
+          });
+      q0 = n / NV * NV;
     }
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
@@ -213,13 +225,16 @@ __global__ void cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *
     point(xq, r[q], XUP ? p[q] : T(0), w[q], cm[q], RR ? c[q] : T(0));
     if constexpr (XUP) x[q] = xq;
   }
-  double v[2] = {(double)a_rz, (double)a_rr};
-  ax::block_sum<2>(v, sh);
-  ax::finish_sums<2>(v, partials, &s->ticket, [s](const double *t) {
+  constexpr int NS = RR ? 2 : 1;
+  double v[NS];
+  v[0] = (double)a_rz;
+  if constexpr (RR) v[1] = (double)a_rr;
+  ax::block_sum<NS>(v);
+  ax::finish_sums<NS>(v, partials, &s->ticket, [s](const double *t) {
     s->beta = (s->rz != 0.0) ? t[0] / s->rz : 0.0;
     s->rz = t[0];
-    s->rr = t[1];
-    if (!isfinite(t[0]) || !isfinite(t[1])) s->status = 1;
+    if constexpr (RR) s->rr = t[1];
+    if (!isfinite(t[0]) || (RR && !isfinite(t[NS - 1]))) s->status = 1;
   });
 }
 
@@ -297,7 +312,6 @@ __global__ void residual_kernel(double *__restrict__ r, float *__restrict__ r32,
                                 const double *__restrict__ b, const double *__restrict__ w,
                                 const double *__restrict__ mask, const double *__restrict__ c,
                                 double *__restrict__ partials, int64_t n) {
-  __shared__ double sh[kRedThreads / 32];
   double a = 0.0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -307,7 +321,7 @@ __global__ void residual_kernel(double *__restrict__ r, float *__restrict__ r32,
     a += c[q] * rv * rv;
   }
   double v[1] = {a};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
 }
 __global__ void sum_partials_kernel(const double *__restrict__ partials, int nblk,
@@ -989,61 +1003,52 @@ namespace {
 // is 0 keep r = 0.  RR: rr (read by the host's convergence test only);
 // without it the kernel neither reads c nor reduces.
 template <typename T, bool MASKW = false, bool RR = true, bool XUP = true>
-__global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
+__global__ void __launch_bounds__(kRedThreads, kRedPerSm)
+fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
                                   const T *__restrict__ p, const T *__restrict__ w,
                                   const T *__restrict__ c, const T *__restrict__ cm,
                                   CgScalars *__restrict__ s,
                                   double *__restrict__ partials, int64_t n) {
-  __shared__ double sh[kRedThreads / 32];
   const T alpha = (T)s->alpha;
   T a_rr = 0;
   auto point = [&](T &xq, T &rq, T &roq, T pq, T wq, T cq, T cmq) {
     if constexpr (XUP) xq += alpha * pq;
     roq = rq;
-    rq = (MASKW && cmq == T(0)) ? rq : rq - alpha * wq;
+    rq = (MASKW && is_zero(cmq)) ? rq : rq - alpha * wq;
     if constexpr (RR) a_rr += cq * rq * rq;
   };
   int64_t q0 = 0;
-  if constexpr (sizeof(T) == 4) {
-    if (aligned16(x, r, r_old, p, w, c, cm)) {  // fp32: 16-byte accesses
-      using V = float4;
-      const int64_t n4 = n / 4;
-      for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
-           v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v], ov;
-        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
-        const V wv = reinterpret_cast<const V *>(w)[v];
-        const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.f, 0.f, 0.f, 0.f};
-        const V mv = MASKW ? reinterpret_cast<const V *>(cm)[v] : V{1.f, 1.f, 1.f, 1.f};
-        point(xv.x, rv.x, ov.x, pv.x, wv.x, cv.x, mv.x);
-        point(xv.y, rv.y, ov.y, pv.y, wv.y, cv.y, mv.y);
-        point(xv.z, rv.z, ov.z, pv.z, wv.z, cv.z, mv.z);
-        point(xv.w, rv.w, ov.w, pv.w, wv.w, cv.w, mv.w);
-        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
-        reinterpret_cast<V *>(r)[v] = rv;
-        reinterpret_cast<V *>(r_old)[v] = ov;
-      }
-      q0 = n4 * 4;
-    }
-  } else {
-    if (aligned16(x, r, r_old, p, w, c, cm)) {  // fp64: 16-byte accesses, two points each
-      using V = double2;
-      const int64_t n2 = n / 2;
-      for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n2;
-           v += (int64_t)gridDim.x * blockDim.x) {
-        V xv = XUP ? reinterpret_cast<V *>(x)[v] : V{}, rv = reinterpret_cast<V *>(r)[v], ov;
-        const V pv = XUP ? reinterpret_cast<const V *>(p)[v] : V{};
-        const V wv = reinterpret_cast<const V *>(w)[v];
-        const V cv = RR ? reinterpret_cast<const V *>(c)[v] : V{0.0, 0.0};
-        const V mv = MASKW ? reinterpret_cast<const V *>(cm)[v] : V{1.0, 1.0};
-        point(xv.x, rv.x, ov.x, pv.x, wv.x, cv.x, mv.x);
-        point(xv.y, rv.y, ov.y, pv.y, wv.y, cv.y, mv.y);
-        if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv;
-        reinterpret_cast<V *>(r)[v] = rv;
-        reinterpret_cast<V *>(r_old)[v] = ov;
-      }
-      q0 = n2 * 2;
-    }
+  if (aligned16(x, r, r_old, p, w, c, cm)) {  // 16-byte accesses
+    using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+    constexpr int NV = 16 / sizeof(T);
+    V xv[2], rv[2], pv[2], wv[2], mv[2], cv[2];
+    auto at = [](const T *f, int64_t v) { return reinterpret_cast<const V *>(f)[v]; };
+    walk2(
+        n / NV,
+        [&](int k, int64_t v) {
+          xv[k] = XUP ? at(x, v) : V{};
+          rv[k] = at(r, v);
+          pv[k] = XUP ? at(p, v) : V{};
+          wv[k] = at(w, v);
+          mv[k] = MASKW ? at(cm, v) : V{};
+          cv[k] = RR ? at(c, v) : V{};
+        },
+        [&](int k, int64_t v) {
+          reinterpret_cast<V *>(r_old)[v] = rv[k];
+          T *xs = reinterpret_cast<T *>(&xv[k]), *rs = reinterpret_cast<T *>(&rv[k]);
+          const T *ps = reinterpret_cast<const T *>(&pv[k]);
+          const T *ws = reinterpret_cast<const T *>(&wv[k]);
+          const T *ms = reinterpret_cast<const T *>(&mv[k]);
+          const T *cs = reinterpret_cast<const T *>(&cv[k]);
+#pragma unroll
+          for (int l = 0; l < NV; ++l) {
+            T old;
+            point(xs[l], rs[l], old, ps[l], ws[l], cs[l], MASKW ? ms[l] : T(1));
+          }
+          if constexpr (XUP) reinterpret_cast<V *>(x)[v] = xv[k];
+          reinterpret_cast<V *>(r)[v] = rv[k];
+        });
+    q0 = n / NV * NV;
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -1053,7 +1058,7 @@ __global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__res
   }
   if constexpr (RR) {
     double v[1] = {(double)a_rr};
-    ax::block_sum<1>(v, sh);
+    ax::block_sum<1>(v);
     ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) { s->rr = t[0]; });
   }
 }
@@ -1064,12 +1069,12 @@ __global__ void fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__res
 // them rz (first: of <z0, r0>, else with Notay's beta) and the choice between
 // the learned and the Jacobi step.  fp32: 16-byte accesses.
 template <typename T>
-__global__ void fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
+__global__ void __launch_bounds__(kRedThreads, kRedPerSm)
+fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
                                 const T *__restrict__ corr, const T *__restrict__ cm,
                                 const T *__restrict__ c, int have_corr, int first,
                                 CgScalars *__restrict__ s, double *__restrict__ partials,
                                 int64_t n) {
-  __shared__ double sh[4 * kRedThreads / 32];
   T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
   auto point = [&](T rv, T ro, T cmv, T cv, T ev) {
     const T a = cmv * rv;
@@ -1086,6 +1091,7 @@ __global__ void fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r
     if (aligned16(r, r_old, corr, cm, c)) {
       using V = float4;
       const int64_t n4 = n / 4;
+#pragma unroll 2
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
            v += (int64_t)gridDim.x * blockDim.x) {
         auto at = [v](const T *p) { return reinterpret_cast<const V *>(p)[v]; };
@@ -1103,7 +1109,7 @@ __global__ void fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r
        q += (int64_t)gridDim.x * blockDim.x)
     point(r[q], r_old[q], cm[q], have_corr ? c[q] : T(0), have_corr ? corr[q] : T(0));
   double v[4] = {(double)d0, (double)d1, (double)d2, (double)d3};
-  ax::block_sum<4>(v, sh);
+  ax::block_sum<4>(v);
   ax::finish_sums<4>(v, partials, &s->ticket, [s, have_corr, first](const double *t) {
     const double rz_l = t[0] + t[1], rz_j = t[0];
     const double num_l = rz_l - (t[2] + t[3]), num_j = t[0] - t[2];
@@ -1169,7 +1175,6 @@ __global__ void fcg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restr
                                 const T *__restrict__ b, const T *__restrict__ mask,
                                 const T *__restrict__ c, CgScalars *__restrict__ s,
                                 double *__restrict__ partials, int64_t n) {
-  __shared__ double sh[kRedThreads / 32];
   T a = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -1180,7 +1185,7 @@ __global__ void fcg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restr
     a += c[q] * rv * rv;
   }
   double v[1] = {(double)a};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) {
     s->rr = t[0];
     s->rr0 = t[0];
@@ -1462,7 +1467,6 @@ __global__ void energy_features_kernel(float *__restrict__ X, double *__restrict
                                        const double *__restrict__ r,
                                        const double *__restrict__ isc, int N) {
   constexpr int KEEP = 4;
-  __shared__ double sh[kRedThreads / 32];
   __shared__ double inv_b;
   const size_t base = (size_t)blockIdx.x * N;
   double ss = 0.0, z[KEEP];
@@ -1477,7 +1481,7 @@ __global__ void energy_features_kernel(float *__restrict__ X, double *__restrict
     ss += y * y;
   }
   double v[1] = {ss};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   if (threadIdx.x == 0) {  // one root and one division a block: the fp64 pipe is narrow
     const double s = sqrt(v[0]);
     s_out[blockIdx.x] = s;
@@ -1512,7 +1516,6 @@ __global__ void energy_dot_dy_kernel(float *__restrict__ dY, const double *__res
                                      const double *__restrict__ osc,
                                      const double *__restrict__ s, const double *__restrict__ eA,
                                      int N, int nelv, double *__restrict__ partials) {
-  __shared__ double sh[kRedThreads / 32];
   __shared__ double scale_b;
   if (threadIdx.x == 0) scale_b = eA[0] > 0.0 ? -2.0 / eA[0] : 0.0;
   __syncthreads();
@@ -1529,7 +1532,7 @@ __global__ void energy_dot_dy_kernel(float *__restrict__ dY, const double *__res
     }
   }
   double v[1] = {a};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
 }
 

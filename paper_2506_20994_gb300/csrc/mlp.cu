@@ -254,13 +254,17 @@ mlp_apply_kernel(T *__restrict__ corr, const T *__restrict__ r, const T *__restr
 }
 
 // Symmetric form with its scale precomputed (sc = sqrt(minv), fp32) and an
-// even number of points per element: one warp streams 16 elements through
-// both layers with no shared memory and no block barrier.  Layer 1 loads the
-// mma A-fragments straight from r and sc (rows g, g+8, columns k+2t4 and
-// k+2t4+8: 16-byte and 8-byte pairs, full sectors), one k-step ahead;
-// its accumulators are re-packed in registers as the A-fragments of
-// layer 2 (n-tiles 2q, 2q+1 of layer 1 are k-step q of layer 2); the
-// epilogue stores corr = sc * y as pairs.  Weights come through L1/L2.
+// even number of points per element: a block takes 16 elements (the rows of
+// the mma tiles) through both layers.  All four warps load and scale the rows
+// together (every load of a row in flight at once) into shared memory as
+// bf16; the warps then share layer 1's hidden n-tiles and, from the hidden
+// layer in shared memory, layer 2's output tiles.  Weights come through L1/L2.
+// Rows of shared memory are padded by 8 values, so that the fragment loads
+// (8 rows x 4 words) touch every bank once.
+// With one warp streaming 16 elements by itself, 4096 elements were 256 warps
+// on 152 SMs, each a chain of 32 load latencies: 42 us, against NEW_US here
+// (fp32, lx = 8, 48 hidden units).  Sums keep their order (k ascending in each
+// tile), so the results are the same bits.
 constexpr int kSymWarps = 4;  // warps per block
 
 template <typename T>
@@ -274,71 +278,96 @@ struct Pair<float> {
   using V = float2;
 };
 
+template <int NT1>
+inline size_t sym_smem(int NP) {
+  return (size_t)16 * (NP + 8) * 2 + (size_t)16 * (NT1 * 8 + 8) * 2;
+}
+
 template <typename T, int NT1>  // NT1 = HP / 8 hidden n-tiles
 __global__ void __launch_bounds__(kSymWarps * 32)
 mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
                      const float *__restrict__ sc, const __nv_bfloat16 *__restrict__ W1T,
                      const __nv_bfloat16 *__restrict__ W2T, int N, int NP, int nelv) {
   using V = typename Pair<T>::V;
-  constexpr int HP = NT1 * 8;
-  const int lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-  const long long ew = ((long long)blockIdx.x * kSymWarps + (threadIdx.x >> 5)) * 16;
-  if (ew >= nelv) return;  // warp-uniform
-  const bool ok0 = ew + g < nelv, ok1 = ew + g + 8 < nelv;
-  const size_t row0 = (size_t)(ok0 ? ew + g : 0) * N, row1 = (size_t)(ok1 ? ew + g + 8 : 0) * N;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int HP = NT1 * 8, HS = HP + 8;
+  const int XS = NP + 8;
+  __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(smem_raw);
+  __nv_bfloat16 *hs = xs + 16 * XS;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
+  const long long e0 = (long long)blockIdx.x * 16;
+  const int nel = (int)min(16ll, (long long)nelv - e0);
 
-  // A-fragment inputs of one k-step: x at (row, k + 2 t4 + {0, 1, 8, 9})
-  struct In {
-    V r[4];
-    float2 s[4];
-  };
-  auto load = [&](int ks, In &in) {
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int k = ks + 2 * t4 + ((h & 2) ? 8 : 0);
-      const bool okr = (h & 1) ? ok1 : ok0;
-      const size_t q = ((h & 1) ? row1 : row0) + k;
-      if (okr && k < N) {  // N even: the pair (k, k + 1) is inside the element
-        in.r[h] = *reinterpret_cast<const V *>(r + q);
-        in.s[h] = *reinterpret_cast<const float2 *>(sc + q);
-      } else {
-        in.r[h] = V{};
-        in.s[h] = make_float2(0.f, 0.f);
+  // the scaled rows, warp w rows w, w + 4, ... (N even: pairs stay in a row)
+  for (int row = wp; row < 16; row += kSymWarps) {
+    const size_t base = (size_t)(e0 + (row < nel ? row : 0)) * N;
+#pragma unroll 8
+    for (int k = 2 * lane; k < NP; k += 64) {
+      uint32_t x = 0u;
+      if (row < nel && k < N) {
+        const V rv = *reinterpret_cast<const V *>(r + base + k);
+        const float2 sv = *reinterpret_cast<const float2 *>(sc + base + k);
+        x = pack_bf16(sv.x * to_f32(rv.x), sv.y * to_f32(rv.y));
       }
-    }
-  };
-  float acc1[NT1][4];
-#pragma unroll
-  for (int j = 0; j < NT1; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc1[j][q] = 0.f;
-  In cur, nxt;
-  load(0, nxt);
-  for (int ks = 0; ks < NP; ks += 16) {
-    cur = nxt;
-    if (ks + 16 < NP) load(ks + 16, nxt);
-    uint32_t a[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h)  // fragment order: (g, k), (g+8, k), (g, k+8), (g+8, k+8)
-      a[h] = pack_bf16(cur.s[h].x * to_f32(cur.r[h].x), cur.s[h].y * to_f32(cur.r[h].y));
-#pragma unroll
-    for (int j = 0; j < NT1; ++j) {
-      const __nv_bfloat16 *w = W1T + (size_t)(j * 8 + g) * NP + ks + 2 * t4;
-      mma_bf16(acc1[j], a, __ldg(reinterpret_cast<const unsigned int *>(w)),
-               __ldg(reinterpret_cast<const unsigned int *>(w + 8)));
+      *reinterpret_cast<uint32_t *>(xs + row * XS + k) = x;
     }
   }
-  // layer-1 accumulators (rows g, g+8; hidden 8j + 2t4 + {0, 1}) as layer-2
-  // A-fragments: k-step q takes n-tiles 2q (k) and 2q + 1 (k + 8)
+  __syncthreads();
+
+  // layer 1: hidden n-tiles wp, wp + 4
+  const __nv_bfloat16 *x0 = xs + g * XS + 2 * t4, *x1 = x0 + 8 * XS;
+  constexpr int TW = (NT1 + kSymWarps - 1) / kSymWarps;
+  float acc[TW][4];
+#pragma unroll
+  for (int j = 0; j < TW; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+#pragma unroll 4
+  for (int ks = 0; ks < NP; ks += 16) {
+    const uint32_t a[4] = {*reinterpret_cast<const uint32_t *>(x0 + ks),
+                           *reinterpret_cast<const uint32_t *>(x1 + ks),
+                           *reinterpret_cast<const uint32_t *>(x0 + ks + 8),
+                           *reinterpret_cast<const uint32_t *>(x1 + ks + 8)};
+#pragma unroll
+    for (int j = 0; j < TW; ++j) {
+      const int nt = wp + j * kSymWarps;
+      if (nt < NT1) {  // warp-uniform
+        const __nv_bfloat16 *w = W1T + (size_t)(nt * 8 + g) * NP + ks + 2 * t4;
+        mma_bf16(acc[j], a, __ldg(reinterpret_cast<const unsigned int *>(w)),
+                 __ldg(reinterpret_cast<const unsigned int *>(w + 8)));
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < TW; ++j) {
+    const int nt = wp + j * kSymWarps;
+    if (nt < NT1) {
+      *reinterpret_cast<uint32_t *>(hs + g * HS + nt * 8 + 2 * t4) = pack_bf16(acc[j][0], acc[j][1]);
+      *reinterpret_cast<uint32_t *>(hs + (g + 8) * HS + nt * 8 + 2 * t4) =
+          pack_bf16(acc[j][2], acc[j][3]);
+    }
+  }
+  __syncthreads();
+
+  // layer 2: output tiles wp, wp + 4, ...; corr = sc * y
   uint32_t a2[NT1 / 2][4];
 #pragma unroll
   for (int q = 0; q < NT1 / 2; ++q) {
-    a2[q][0] = pack_bf16(acc1[2 * q][0], acc1[2 * q][1]);
-    a2[q][1] = pack_bf16(acc1[2 * q][2], acc1[2 * q][3]);
-    a2[q][2] = pack_bf16(acc1[2 * q + 1][0], acc1[2 * q + 1][1]);
-    a2[q][3] = pack_bf16(acc1[2 * q + 1][2], acc1[2 * q + 1][3]);
+    const __nv_bfloat16 *h0 = hs + g * HS + 16 * q + 2 * t4, *h1 = h0 + 8 * HS;
+    a2[q][0] = *reinterpret_cast<const uint32_t *>(h0);
+    a2[q][1] = *reinterpret_cast<const uint32_t *>(h1);
+    a2[q][2] = *reinterpret_cast<const uint32_t *>(h0 + 8);
+    a2[q][3] = *reinterpret_cast<const uint32_t *>(h1 + 8);
   }
-  for (int nt = 0; nt < NP / 8; ++nt) {
+  const bool ok0 = g < nel, ok1 = g + 8 < nel;
+  const size_t row0 = (size_t)(e0 + (ok0 ? g : 0)) * N, row1 = (size_t)(e0 + (ok1 ? g + 8 : 0)) * N;
+#pragma unroll 4
+  for (int nt = wp; nt < NP / 8; nt += kSymWarps) {
+    const int col = nt * 8 + 2 * t4;
+    const bool in = col < N;
+    const float2 zero = make_float2(0.f, 0.f);
+    const float2 s0 = in && ok0 ? *reinterpret_cast<const float2 *>(sc + row0 + col) : zero;
+    const float2 s1 = in && ok1 ? *reinterpret_cast<const float2 *>(sc + row1 + col) : zero;
     float acc2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int q = 0; q < NT1 / 2; ++q) {
@@ -346,24 +375,31 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
       mma_bf16(acc2, a2[q], __ldg(reinterpret_cast<const unsigned int *>(w)),
                __ldg(reinterpret_cast<const unsigned int *>(w + 8)));
     }
-    const int col = nt * 8 + 2 * t4;
-    if (col < N) {
-      if (ok0) {
-        const float2 sv = *reinterpret_cast<const float2 *>(sc + row0 + col);
-        V o;
-        o.x = from_f32<T>(sv.x * acc2[0]);
-        o.y = from_f32<T>(sv.y * acc2[1]);
-        *reinterpret_cast<V *>(corr + row0 + col) = o;
-      }
-      if (ok1) {
-        const float2 sv = *reinterpret_cast<const float2 *>(sc + row1 + col);
-        V o;
-        o.x = from_f32<T>(sv.x * acc2[2]);
-        o.y = from_f32<T>(sv.y * acc2[3]);
-        *reinterpret_cast<V *>(corr + row1 + col) = o;
-      }
+    if (in && ok0) {
+      V o;
+      o.x = from_f32<T>(s0.x * acc2[0]);
+      o.y = from_f32<T>(s0.y * acc2[1]);
+      *reinterpret_cast<V *>(corr + row0 + col) = o;
+    }
+    if (in && ok1) {
+      V o;
+      o.x = from_f32<T>(s1.x * acc2[2]);
+      o.y = from_f32<T>(s1.y * acc2[3]);
+      *reinterpret_cast<V *>(corr + row1 + col) = o;
     }
   }
+}
+
+template <typename T, int NT1>
+int sym_apply(T *corr, const T *r, const float *sc, const __nv_bfloat16 *w1,
+              const __nv_bfloat16 *w2, int N, int NP, int nelv, cudaStream_t st) {
+  auto kern = mlp_sym_apply_kernel<T, NT1>;
+  const size_t smem = sym_smem<NT1>(NP);
+  static std::atomic<size_t> granted[ax::kMaxDevices];
+  if (!ax::grant_smem(kern, smem, granted)) return AX_EINVAL;
+  kern<<<(unsigned)((nelv + 15) / 16), kSymWarps * 32, smem, st>>>(corr, r, sc, w1, w2, N, NP,
+                                                                  nelv);
+  return ax::launch_status();
 }
 
 // ---------------------------------------------------------------- training
@@ -372,7 +408,6 @@ __global__ void gather_pairs_kernel(float *__restrict__ X, float *__restrict__ T
                                     const double *__restrict__ r, const double *__restrict__ err,
                                     const double *__restrict__ minv, const int *__restrict__ idx,
                                     int N) {
-  __shared__ double sh[kThreads / 32];
   const int b = blockIdx.x;
   const size_t base = (size_t)idx[b] * N;
   double ss = 0.0;
@@ -381,7 +416,7 @@ __global__ void gather_pairs_kernel(float *__restrict__ X, float *__restrict__ T
     ss += z * z;
   }
   double v[1] = {ss};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   __shared__ double s_b;
   if (threadIdx.x == 0) s_b = sqrt(v[0]);
   __syncthreads();
@@ -602,7 +637,6 @@ __global__ void __launch_bounds__(kThreads)
 fwd_out_loss_kernel(float *__restrict__ Y, float *__restrict__ dY, const float *__restrict__ H,
                     const float *__restrict__ Tt, const float *__restrict__ theta, int B, int N,
                     int Hd, double *__restrict__ partials) {
-  __shared__ double sh[kThreads / 32];
   double l = 0.0;
   out_rows(H, theta, B, N, Hd, [&](int b, int o, float y) {
     const size_t q = (size_t)b * N + o;
@@ -612,7 +646,7 @@ fwd_out_loss_kernel(float *__restrict__ Y, float *__restrict__ dY, const float *
     l += (double)res * (double)res;
   });
   double v[1] = {l};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = v[0];
 }
 
@@ -884,15 +918,12 @@ int mlp_correction(const ax_mlp *M, T *corr, const T *r, const T *minv, const T 
                                                           L.HP == 48 || L.HP == 64)) {
     auto w1 = reinterpret_cast<const __nv_bfloat16 *>(base + L.w1t);
     auto w2 = reinterpret_cast<const __nv_bfloat16 *>(base + L.w2t);
-    const unsigned grid = (unsigned)((nelv + 16 * kSymWarps - 1) / (16 * kSymWarps));
-    const int th = kSymWarps * 32;
     switch (L.HP) {
-      case 16: mlp_sym_apply_kernel<T, 2><<<grid, th, 0, st>>>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv); break;
-      case 32: mlp_sym_apply_kernel<T, 4><<<grid, th, 0, st>>>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv); break;
-      case 48: mlp_sym_apply_kernel<T, 6><<<grid, th, 0, st>>>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv); break;
-      default: mlp_sym_apply_kernel<T, 8><<<grid, th, 0, st>>>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv); break;
+      case 16: return sym_apply<T, 2>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv, st);
+      case 32: return sym_apply<T, 4>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv, st);
+      case 48: return sym_apply<T, 6>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv, st);
+      default: return sym_apply<T, 8>(corr, r, sc, w1, w2, M->n_in, L.NP, nelv, st);
     }
-    return launch_status();
   }
   const size_t smem = apply_smem(L.HP);
   auto kern = M->arch == AX_MLP_SYM ? mlp_apply_kernel<T, true> : mlp_apply_kernel<T, false>;

@@ -15,24 +15,33 @@ namespace ax {
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 152 * 4;  // 4 blocks per SM of the 152-SM part
 
-// Sum of v over the block; valid in thread 0.  Deterministic order.
+// Sum of v over the block (kRedThreads threads); valid in thread 0.
+// Deterministic order: lane l of quantity q's warp adds threads l, l + 32, ...
+// in order, then a fixed shuffle tree.  Through shared memory, because the
+// fp64 pipe takes about 19 cycles an SM for each warp-wide addition whatever
+// lanes are active: 13 of them a block and quantity, where a shuffle tree in
+// each of the eight warps and a serial sum need 48 (at 608 blocks 3 us of the
+// update kernel's time per quantity).
 template <int NV>
-AX_D void block_sum(double (&v)[NV], double *sh /* [NV][kRedThreads/32] */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+AX_D void block_sum(double (&v)[NV]) {
+  __shared__ double buf[NV][kRedThreads];
+  __shared__ double tot[NV];
 #pragma unroll
-  for (int q = 0; q < NV; ++q) {
+  for (int q = 0; q < NV; ++q) buf[q][threadIdx.x] = v[q];
+  __syncthreads();
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q < NV) {
+    double s = buf[q][lane];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
-    if (lane == 0) sh[q * (kRedThreads / 32) + wid] = v[q];
+    for (int k = 1; k < kRedThreads / 32; ++k) s += buf[q][lane + 32 * k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) tot[q] = s;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      double s = 0.0;
-      for (int k = 0; k < kRedThreads / 32; ++k) s += sh[q * (kRedThreads / 32) + k];
-      v[q] = s;
-    }
+    for (int k = 0; k < NV; ++k) v[k] = tot[k];
   }
 }
 

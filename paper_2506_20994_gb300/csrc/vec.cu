@@ -10,13 +10,12 @@ namespace {
 __global__ void wdot_kernel(const double *__restrict__ a, const double *__restrict__ b,
                             const double *__restrict__ wgt, double *__restrict__ partials,
                             int64_t n) {
-  __shared__ double sh[ax::kRedThreads / 32];
   double s = 0.0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x)
     s += wgt[q] * a[q] * b[q];
   double v[1] = {s};
-  ax::block_sum<1>(v, sh);
+  ax::block_sum<1>(v);
   if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
 }
 
@@ -45,7 +44,6 @@ template <typename T>
 __global__ void mass_add_kernel(T *__restrict__ w, const T *__restrict__ hb,
                                 const T *__restrict__ u, int64_t n,
                                 double *__restrict__ partials) {
-  __shared__ double sh[ax::kRedThreads / 32];
   T acc = T(0);
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -55,7 +53,7 @@ __global__ void mass_add_kernel(T *__restrict__ w, const T *__restrict__ hb,
   }
   if (partials) {  // kernel-uniform
     double v[1] = {(double)acc};
-    ax::block_sum<1>(v, sh);
+    ax::block_sum<1>(v);
     if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
   }
 }
