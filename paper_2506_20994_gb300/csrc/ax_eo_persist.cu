@@ -12,14 +12,9 @@ namespace ax {
 
 namespace {
 
-template <int LX, bool DOT, bool PUPD>
-auto eop_kernel() {
-  return eop::ax_eop_kernel<LX, DOT, PUPD>;
-}
-
 // Resident CTAs of one kernel variant on the current device times its SMs
 // (cached per device; the shared-memory limit is raised on first use).
-template <int LX, bool DOT, bool PUPD>
+template <int LX, bool DOT, bool PUPD, bool HB = false>
 int eop_grid() {
   using C = eop::Cfg<LX>;
   static std::atomic<int> grid[kMaxDevices];
@@ -30,7 +25,7 @@ int eop_grid() {
   }
   int g = grid[dev].load(std::memory_order_acquire);
   if (g > 0) return g;
-  auto kern = eop_kernel<LX, DOT, PUPD>();
+  auto kern = eop::ax_eop_kernel<LX, DOT, PUPD, false, HB>;
   int sms = 0, bps = 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) !=
           cudaSuccess ||
@@ -68,12 +63,23 @@ int eop_launch_t(const EopArgs &a, cudaStream_t st) {
   m.dx = a.dx;
   m.dxt = a.dxt;
   m.drop = a.drop;
+  m.hb = a.hb;
   eop::EopUpd up{a.pw, a.r, a.minv, a.corr, a.x, 0.0, 0.0, false};
   if constexpr (!DOT && !PUPD) {
     if (a.drop >= 0) {  // testing aid: same grid, its own instantiation
       cudaFuncSetAttribute(eop::ax_eop_kernel<LX, false, false, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
       eop::ax_eop_kernel<LX, false, false, true><<<grid, C::NTB, C::SMEM, st>>>(
+          m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr, a.alpha);
+      return launch_status();
+    }
+  }
+  if constexpr (!DOT && !PUPD) {
+    if (a.hb) {
+      const int gh = eop_grid<LX, false, false, true>();
+      if (gh <= 0) return AX_ELAUNCH;
+      const unsigned nb = (unsigned)std::min<long long>(gh, std::max(a.nelv, 1));
+      eop::ax_eop_kernel<LX, false, false, false, true><<<nb, C::NTB, C::SMEM, st>>>(
           m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr, a.alpha);
       return launch_status();
     }
@@ -186,7 +192,7 @@ int eopr_launch(int lx, double *w, const double *u, const double *dx, const doub
 
 int eop_launch(int lx, const EopArgs &a, cudaStream_t st) {
   if (a.pw && !(a.dotp && a.r && a.minv && a.beta)) return AX_EINVAL;
-  if ((a.corr && !a.use_corr) || (a.x && !a.alpha)) return AX_EINVAL;
+  if ((a.corr && !a.use_corr) || (a.x && !a.alpha) || (a.hb && a.dotp)) return AX_EINVAL;
   switch (lx) {
     case 6: return eop_launch_lx<6>(a, st);
     case 8: return eop_launch_lx<8>(a, st);

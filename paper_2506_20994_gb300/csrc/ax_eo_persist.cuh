@@ -173,6 +173,8 @@ struct EopMesh {
   const uint2 *urange = nullptr;
   guard::RawGeo raw{};
   const double *dx = nullptr, *dxt = nullptr;
+  // HB: h2 .* B of the Helmholtz form, w = Ax(u) + hb .* u
+  const double *hb = nullptr;
   // testing aid (ax_op_inject_copy_loss): this element's geometry copy is
   // never issued, so its wait runs out; -1: none
   long long drop = -1;
@@ -231,11 +233,15 @@ struct SeqOne {
 // matrices' exponent field and symmetry are formed here from M.dx, M.dxt,
 // and each element's exponent window is checked from its own values; M.gp,
 // M.coef and M.urange are not used.  (ax_helm on fp64 arrays.)
-template <int LX, bool DOT, bool PUPD, bool RAW = false, bool DROP = false, class Seq,
-          class Sync, class SyncAnd>
+// HB: the Helmholtz mass term, w += M.hb .* u with fp64 units as w is stored.
+// As a pass of its own it moved 32 bytes a point more (4096 elements, lx = 10:
+// 134.9 us a call, now 118.5).
+template <int LX, bool DOT, bool PUPD, bool RAW = false, bool DROP = false, bool HB = false,
+          class Seq, class Sync, class SyncAnd>
 AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd sync_and,
                   int *err, const EopUpd &up, double &dsum) {
   static_assert(!RAW || (!DOT && !PUPD), "the raw-array form is the plain apply");
+  static_assert(!HB || (!DOT && !PUPD && !RAW), "the mass term joins the handle's plain apply");
   using namespace df;
   using C = Cfg<LX>;
   constexpr int H = C::H, N = C::N, H2 = C::H2, NT = C::NT, NW = C::NW, N3 = C::N3;
@@ -558,6 +564,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       if constexpr (PUPD) {
         if (up.x) prefetch_l2(up.x + (size_t)seq.elem(nxp) * N3, N3 * 8);
       }
+      if constexpr (HB) prefetch_l2(M.hb + (size_t)seq.elem(nxp) * N3, N3 * 8);
     }
     unsigned uke = 0u;
 #pragma unroll
@@ -582,6 +589,15 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 
     // ---- phase 5: transposed contractions, summed, stored
     contract_all(Lb, tf, tn, gr, gs, gt);
+    double hv[2][2];
+    if constexpr (HB) {
+      if (real) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+          for (int a = 0; a < 2; ++a) hv[b][a] = __ldg(M.hb + eb + pidx(b, a));
+      }
+    }
     if (real && !bad) {
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
@@ -589,7 +605,11 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
                         dd2{pk(gs[b][0].hi, gs[b][1].hi), pk(gs[b][0].lo, gs[b][1].lo)});
         acc = dsum2(acc, dd2{pk(gt[b][0].hi, gt[b][1].hi), pk(gt[b][0].lo, gt[b][1].lo)});
         const df2 w0 = norm(lx_(acc.hi), lx_(acc.lo)), w1 = norm(ly_(acc.hi), ly_(acc.lo));
-        const double wd0 = join(w0.hi, w0.lo), wd1 = join(w1.hi, w1.lo);
+        double wd0 = join(w0.hi, w0.lo), wd1 = join(w1.hi, w1.lo);
+        if constexpr (HB) {
+          wd0 = __fma_rn(hv[b][0], ucur[b][0], wd0);
+          wd1 = __fma_rn(hv[b][1], ucur[b][1], wd1);
+        }
         M.w[eb + pidx(b, 0)] = wd0;
         M.w[eb + pidx(b, 1)] = wd1;
         if constexpr (DOT) {
@@ -604,6 +624,17 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
                              M.dxt, M.raw.h1, M.raw.g11, M.raw.g22, M.raw.g33, M.raw.g12,
                              M.raw.g13, M.raw.g23, eb, reinterpret_cast<double *>(Lb), tid, NT,
                              sync, DOT ? &dsum : nullptr);
+      if constexpr (HB) {  // every thread's own points, after the barrier inside
+        if (real) {
+#pragma unroll
+          for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+              const size_t q = eb + pidx(b, a);
+              M.w[q] = __fma_rn(hv[b][a], ucur[b][a], M.w[q]);
+            }
+        }
+      }
     }
     sync();  // the lines and key slots are free for the next element
     pos = nxp;
@@ -617,8 +648,9 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 
 // The operator handle's kernel: one mesh, elements blockIdx.x + k gridDim.x.
 // DOT: one partial of u . w per CTA (fixed order) in dotp[blockIdx.x].
-// DROP: the testing aid of ax_op_inject_copy_loss (plain applies only).
-template <int LX, bool DOT, bool PUPD, bool DROP = false>
+// DROP: the testing aid of ax_op_inject_copy_loss (plain applies only).  HB:
+// with the mass term (plain applies only).
+template <int LX, bool DOT, bool PUPD, bool DROP = false, bool HB = false>
 __global__ void __launch_bounds__(Cfg<LX>::NTB, Cfg<LX>::MINB)
 ax_eop_kernel(const EopMesh mesh, long long nelv, int *__restrict__ err,
               double *__restrict__ dotp, const EopUpd up0,
@@ -634,7 +666,7 @@ ax_eop_kernel(const EopMesh mesh, long long nelv, int *__restrict__ err,
   }
   const SeqOne seq{mesh, nelv};
   double dsum = 0.0;
-  eop_run<LX, DOT, PUPD, false, DROP>(
+  eop_run<LX, DOT, PUPD, false, DROP, HB>(
       sm, (int)threadIdx.x, seq, [] { __syncthreads(); },
       [](bool p) { return __syncthreads_and(p) != 0; }, err, up, dsum);
   if constexpr (DOT) {  // one partial per CTA: fixed shuffle tree, warps in order

