@@ -80,28 +80,35 @@ DF_HD float fma(float a, float b, float c) { return __builtin_fmaf(a, b, c); }
 DF_HD int f2i_rn(float a) { return (int)__builtin_nearbyintf(a); }
 #endif
 
+// max(a + b, c), one instruction on the device
+DF_HD int addmax(int a, int b, int c) {
+#ifdef __CUDA_ARCH__
+  return __viaddmax_s32(a, b, c);
+#else
+  return a + b > c ? a + b : c;
+#endif
+}
+
 // --- fp64 -> double-float split, integer ops only ---------------------------
 // hi = x truncated to 24 significant bits; lo = the next 23 bits of x, so
-// |x - (hi + lo)| < 2^-46 |x| for 2^-80 <= |x| < 2^128.  Smaller magnitudes
-// keep an absolute error below 2^-100 (hi flushes toward zero below 2^-126).
+// |x - (hi + lo)| < 2^-46 |x| for 2^-103 <= |x| < 2^128.  Smaller magnitudes
+// keep an absolute error below 2^-125 (hi flushes toward zero below 2^-126).
+// Nine integer instructions and one subtraction: lo is the difference of two
+// fp32 numbers of its sign and of exponent(hi) - 23, one with the 23 bits as
+// its mantissa and one with none (exact); the exponent is clamped at zero,
+// where both are subnormal.  (Scaling the 23 bits by a power of two chosen by
+// a compare took sixteen.)
 DF_HD df2 split(double x) {
   const uint64_t b = d2u(x);
   const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
   const uint32_t sgn = hw & 0x80000000u;
-  uint32_t mag = hw & 0x7FFFFFFFu;            // exponent(11) | mantissa-high(20)
-  const uint32_t bias = 896u << 20;           // 1023 - 127
-  mag = mag < bias ? bias : mag;              // flush below the fp32 normal range
-  // ((mag - bias) << 3) | (lw >> 29): fp32 exponent(8) | 23 mantissa bits
-  const uint32_t fh = (((mag - bias) << 3) | (lw >> 29)) | sgn;
-  // remaining 29 bits r of the mantissa, value r * 2^(e-1075); keep the top 23
-  const uint32_t r23 = (lw >> 6) & 0x7FFFFFu;
-  const float rf = sub(u2f(0x4B000000u | r23), 8388608.0f);  // exact integer r >> 6
-  const uint32_t e = (hw >> 20) & 0x7FFu;
-  // +-2^(e-1069), or zero (lo dropped) below |x| = 2^-80
-  const uint32_t sc = e >= 943u ? (((e - 942u) << 23) | sgn) : 0u;
+  // exponent(11) | mantissa-high(20), rebased and flushed below the fp32 range
+  const uint32_t mag = (uint32_t)addmax((int)(hw & 0x7FFFFFFFu), -(896 << 20), 0);
+  const uint32_t fm = (mag << 3) | (lw >> 29);  // fp32 exponent(8) | 23 mantissa bits
+  const uint32_t base = (uint32_t)addmax((int)(fm & 0x7F800000u), -(23 << 23), 0) | sgn;
   df2 o;
-  o.hi = u2f(fh);
-  o.lo = mul(rf, u2f(sc));
+  o.hi = u2f(fm | sgn);
+  o.lo = sub(u2f(base | ((lw >> 6) & 0x7FFFFFu)), u2f(base));
   return o;
 }
 
