@@ -119,38 +119,61 @@ def df64_roundtrip(x: np.ndarray):
 # ---------------------------------------------------------------------------
 # device calls (torch CUDA tensors in and out)
 # ---------------------------------------------------------------------------
-def _stream():
+_torch = None
+_raw_stream = _get_device = None
+
+
+def _load_torch():
+    """torch, imported once; with it the raw-handle queries of the current
+    stream and device (torch.cuda.current_stream() builds a Stream object on
+    every call: 2.8 us of a 12 us call on the GB300 host, against 0.1 us)."""
+    global _torch, _raw_stream, _get_device
     import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    dev = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None:
+        _raw_stream, _get_device = raw, dev
+    _torch = torch
+    return torch
+
+
+def _stream():
+    torch = _torch or _load_torch()
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(_get_device())
     return torch.cuda.current_stream().cuda_stream
 
 
 def _dev_args(lx, w, tensors, dtypes, d_tensors, d_dtype):
-    import torch
+    torch = _torch or _load_torch()
+    Tensor = torch.Tensor
     n = None
     for t, dt in zip([w] + list(tensors), dtypes):
-        if not isinstance(t, torch.Tensor) or not t.is_cuda:
+        if not isinstance(t, Tensor) or not t.is_cuda:
             raise TypeError("expected CUDA tensors")
-        if t.dtype != dt:
+        if t.dtype is not dt:
             raise TypeError(f"expected {dt}, got {t.dtype}")
         if not t.is_contiguous():
             raise ValueError("tensors must be contiguous")
+        m = t.numel()
         if n is None:
-            n = t.numel()
-        elif t.numel() != n:
+            n = m
+        elif m != n:
             raise ValueError("all element fields must have the same size")
+    l2 = lx * lx
     for t in d_tensors:
-        if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == d_dtype
-                and t.is_contiguous() and t.numel() == lx * lx):
+        if not (isinstance(t, Tensor) and t.is_cuda and t.dtype is d_dtype
+                and t.is_contiguous() and t.numel() == l2):
             raise ValueError(f"dx/dxt must be contiguous {d_dtype} CUDA tensors of lx*lx values")
-    if n % (lx ** 3):
+    if n % (l2 * lx):
         raise ValueError("field size is not a multiple of lx^3")
-    return n // (lx ** 3)
+    return n // (l2 * lx)
 
 
 def ax_helm(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, lx: int,
             variant: int = AX_VARIANT_AUTO, elems_per_block: int = 0) -> None:
     """w <- element-local stiffness apply of u, fp64 (ax_helm_variant)."""
-    import torch
+    torch = _torch or _load_torch()
     f = torch.float64
     nel = _dev_args(lx, w, [u, h1, g11, g22, g33, g12, g13, g23], [f] * 9, [dx, dxt], f)
     rc = lib().ax_helm_variant(variant, w.data_ptr(), u.data_ptr(), dx.data_ptr(),
@@ -164,7 +187,7 @@ def ax_helm_xyz(w, u, dx, dy, dz, dxt, dyt, dzt, h1, g11, g22, g33, g12, g13, g2
                 lx: int) -> None:
     """w <- element-local stiffness apply of u with one matrix per direction
     (the full argument list of Listings 1-2), fp64 (ax_helm_xyz)."""
-    import torch
+    torch = _torch or _load_torch()
     f = torch.float64
     nel = _dev_args(lx, w, [u, h1, g11, g22, g33, g12, g13, g23], [f] * 9,
                     [dx, dy, dz, dxt, dyt, dzt], f)
@@ -176,7 +199,7 @@ def ax_helm_trilinear_f32(w, u, dx, dxt, h1, corners, xi, wq, lx: int) -> None:
     """fp32 operator with G computed from each element's corner vertices
     (ax_helm_trilinear_f32).  w, u, dx, dxt, h1: fp32 CUDA tensors (h1 may
     be None: h1 = 1); corners (E*24), xi, wq (lx): fp64 CUDA tensors."""
-    import torch
+    torch = _torch or _load_torch()
     f = torch.float32
     fields = [u] if h1 is None else [u, h1]
     nel = _dev_args(lx, w, fields, [f] * (len(fields) + 1), [dx, dxt], f)
@@ -213,7 +236,7 @@ def ax_helm_h2(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, h2, B, lx: int) 
 
 def ax_helm_f32(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, lx: int) -> None:
     """fp32 storage and arithmetic (ax_helm_f32)."""
-    import torch
+    torch = _torch or _load_torch()
     f = torch.float32
     nel = _dev_args(lx, w, [u, h1, g11, g22, g33, g12, g13, g23], [f] * 9, [dx, dxt], f)
     rc = lib().ax_helm_f32(w.data_ptr(), u.data_ptr(), dx.data_ptr(), dxt.data_ptr(),
@@ -224,7 +247,7 @@ def ax_helm_f32(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, lx: int) -> Non
 
 def ax_helm_bf16(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, lx: int) -> None:
     """bf16 storage of u, h1, G; fp32 D, arithmetic and w (ax_helm_bf16)."""
-    import torch
+    torch = _torch or _load_torch()
     b = torch.bfloat16
     nel = _dev_args(lx, w, [u, h1, g11, g22, g33, g12, g13, g23],
                     [torch.float32] + [b] * 8, [dx, dxt], torch.float32)
