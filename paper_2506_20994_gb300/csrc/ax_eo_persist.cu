@@ -79,15 +79,13 @@ int eop_launch_t(const EopArgs &a, cudaStream_t st) {
       const int gh = eop_grid<LX, false, false, true>();
       if (gh <= 0) return AX_ELAUNCH;
       const unsigned nb = (unsigned)std::min<long long>(gh, std::max(a.nelv, 1));
-      eop::ax_eop_kernel<LX, false, false, false, true><<<nb, C::NTB, C::SMEM, st>>>(
-          m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr, a.alpha);
-      return launch_status();
+      return launch_chained(a.chained, eop::ax_eop_kernel<LX, false, false, false, true>, nb,
+                            C::NTB, C::SMEM, st, m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr,
+                            a.alpha);
     }
   }
-  eop::ax_eop_kernel<LX, DOT, PUPD><<<grid, C::NTB, C::SMEM, st>>>(m, (long long)a.nelv, a.err,
-                                                                  a.dotp, up, a.beta,
-                                                                  a.use_corr, a.alpha);
-  return launch_status();
+  return launch_chained(a.chained, eop::ax_eop_kernel<LX, DOT, PUPD>, grid, C::NTB, C::SMEM, st,
+                        m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr, a.alpha);
 }
 
 template <int LX>
@@ -131,8 +129,7 @@ int eopr_launch_lx(double *w, const double *u, const double *dx, const double *d
   m.dx = dx;
   m.dxt = dxt;
   const unsigned nb = (unsigned)std::min<long long>(g, std::max(nelv, 1));
-  eop::ax_eopr_kernel<LX><<<nb, C::NTB, C::SMEM, st>>>(m, (long long)nelv);
-  return launch_status();
+  return launch_chained(true, eop::ax_eopr_kernel<LX>, nb, C::NTB, C::SMEM, st, m, (long long)nelv);
 }
 
 template <int LX>

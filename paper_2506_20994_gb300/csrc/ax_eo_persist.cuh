@@ -236,10 +236,13 @@ struct SeqOne {
 // HB: the Helmholtz mass term, w += M.hb .* u with fp64 units as w is stored.
 // As a pass of its own it moved 32 bytes a point more (4096 elements, lx = 10:
 // 134.9 us a call, now 118.5).
+// ready(): called once, after the set-up that needs no other kernel's results
+// (the first element's prepared geometry and the coefficients, both the
+// handle's own) and before everything else; RAW calls it first.
 template <int LX, bool DOT, bool PUPD, bool RAW = false, bool DROP = false, bool HB = false,
-          class Seq, class Sync, class SyncAnd>
+          class Seq, class Sync, class SyncAnd, class Ready>
 AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd sync_and,
-                  int *err, const EopUpd &up, double &dsum) {
+                  int *err, EopUpd &up, double &dsum, Ready ready) {
   static_assert(!RAW || (!DOT && !PUPD), "the raw-array form is the plain apply");
   static_assert(!HB || (!DOT && !PUPD && !RAW), "the mass term joins the handle's plain apply");
   using namespace df;
@@ -336,7 +339,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 #pragma unroll
         for (int tr = 0; tr < 2; ++tr) {
           const double *m = tr ? M.dxt : M.dx;
-          const double a = __ldg(m + q), mir = __ldg(m + (N - l) * LX + (N - i));
+          const double a = __ldcg(m + q), mir = __ldcg(m + (N - l) * LX + (N - i));
           atomicMax(&drec[0], guard::abs_bits(a));
           atomicMax(&drec[1], guard::abs_bits(__dadd_rn(a, mir)));
         }
@@ -344,7 +347,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       for (int q = tid; q < 2 * H2; q += C::NTB) {
         const int tr = q / H2, i = (q / H) % H, l = q % H;
         const double *m = tr ? M.dxt : M.dx;
-        const double a = __ldg(m + l * LX + i), b = __ldg(m + (N - l) * LX + i);
+        const double a = __ldcg(m + l * LX + i), b = __ldcg(m + (N - l) * LX + i);
         const df2 P = split_rn(__dmul_rn(0.5, __dadd_rn(a, b)));
         const df2 Q = split_rn(__dmul_rn(0.5, __dsub_rn(a, b)));
         cf[(tr * H + i) * CS + l] = dd2{pk(P.hi, Q.hi), pk(P.lo, Q.lo)};
@@ -389,8 +392,17 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   EopPos pos;
   bool have = seq.first(pos);
   int cmesh = -1;  // mesh whose coefficients are staged
+  if constexpr (RAW) ready();
   sync();  // the barrier is initialised before anyone waits on it
   if (tid == 0 && have) issue_geo(pos);
+  bool staged = false;  // the first run's coefficients are
+  if constexpr (!RAW) {
+    if (have) {
+      load_coef(seq.mesh(seq.mesh_of(pos)));
+      staged = true;
+    }
+    ready();
+  }
 
   double uv[2][2] = {{0.0, 0.0}, {0.0, 0.0}};      // u (or r) of the element in turn
   double mv[2][2], pv[2][2], qv[2][2];             // PUPD: minv, old direction, corr
@@ -403,12 +415,12 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       for (int a = 0; a < 2; ++a) {
         const size_t q = eb + pidx(b, a);
         if constexpr (PUPD) {
-          uv[b][a] = __ldg(up.r + q);
-          mv[b][a] = __ldg(up.minv + q);
-          pv[b][a] = up.pw[q];
-          qv[b][a] = up.corr ? __ldg(up.corr + q) : 0.0;
+          uv[b][a] = __ldcg(up.r + q);
+          mv[b][a] = __ldcg(up.minv + q);
+          pv[b][a] = __ldcg(up.pw + q);
+          qv[b][a] = up.corr ? __ldcg(up.corr + q) : 0.0;
         } else {
-          uv[b][a] = __ldg(M.u + q);
+          uv[b][a] = __ldcg(M.u + q);
         }
       }
   };
@@ -420,7 +432,8 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   // behind a test that is false after the first element, cost 6 %)
   while (have) {
     cmesh = seq.mesh_of(pos);
-    load_coef(seq.mesh(cmesh));  // the previous element's last barrier freed them
+    if (!staged) load_coef(seq.mesh(cmesh));  // the previous element's last barrier freed them
+    staged = false;
   for (; have && seq.mesh_of(pos) == cmesh; parity ^= 1u) {
     EopPos nxp;
     const bool more = seq.advance(pos, nxp);
@@ -438,7 +451,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
-          for (int a = 0; a < 2; ++a) xv[b][a] = up.x[eb + pidx(b, a)];
+          for (int a = 0; a < 2; ++a) xv[b][a] = __ldcg(up.x + eb + pidx(b, a));
       }
     }
 #pragma unroll
@@ -595,7 +608,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
-          for (int a = 0; a < 2; ++a) hv[b][a] = __ldg(M.hb + eb + pidx(b, a));
+          for (int a = 0; a < 2; ++a) hv[b][a] = __ldcg(M.hb + eb + pidx(b, a));
       }
     }
     if (real && !bad) {
@@ -659,16 +672,20 @@ ax_eop_kernel(const EopMesh mesh, long long nelv, int *__restrict__ err,
   using C = Cfg<LX>;
   extern __shared__ __align__(128) unsigned char sm[];
   EopUpd up = up0;
-  if constexpr (PUPD) {  // solver scalars live on the device
-    up.beta = *beta_p;
-    if (up.x) up.alpha = *alpha_p;
-    up.use_corr = up.corr != nullptr && *use_corr_p != 0;
-  }
+  auto ready = [&] {
+    grid_wait();
+    grid_go();
+    if constexpr (PUPD) {  // solver scalars live on the device
+      up.beta = __ldcg(beta_p);
+      if (up.x) up.alpha = __ldcg(alpha_p);
+      up.use_corr = up.corr != nullptr && __ldcg(use_corr_p) != 0;
+    }
+  };
   const SeqOne seq{mesh, nelv};
   double dsum = 0.0;
   eop_run<LX, DOT, PUPD, false, DROP, HB>(
       sm, (int)threadIdx.x, seq, [] { __syncthreads(); },
-      [](bool p) { return __syncthreads_and(p) != 0; }, err, up, dsum);
+      [](bool p) { return __syncthreads_and(p) != 0; }, err, up, dsum, ready);
   if constexpr (DOT) {  // one partial per CTA: fixed shuffle tree, warps in order
     double *red = reinterpret_cast<double *>(sm + C::OFF_MISC + 16 + C::NW * 8);
 #pragma unroll
@@ -690,10 +707,13 @@ ax_eopr_kernel(const EopMesh mesh, long long nelv) {
   extern __shared__ __align__(128) unsigned char sm[];
   const SeqOne seq{mesh, nelv};
   double dsum = 0.0;
-  const EopUpd none{};
+  EopUpd none{};
   eop_run<LX, false, false, true>(
       sm, (int)threadIdx.x, seq, [] { __syncthreads(); },
-      [](bool p) { return __syncthreads_and(p) != 0; }, nullptr, none, dsum);
+      [](bool p) { return __syncthreads_and(p) != 0; }, nullptr, none, dsum, [] {
+        grid_wait();
+        grid_go();
+      });
 }
 
 // Prepared geometry of this kernel: per element, entry (b * 7 + f) * NT + tid

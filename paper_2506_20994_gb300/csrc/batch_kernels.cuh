@@ -123,9 +123,9 @@ __device__ __noinline__ void batch_run_eo(const BatchGroup &G, const BatchItem *
     return r != 0u;
   };
   double dsum = 0.0;
-  const eop::EopUpd up{};
+  eop::EopUpd up{};
   eop::eop_run<LX, false, false>(sm + (size_t)slot * batch_eo_slot_bytes<LX>(), tid, seq, sync,
-                                 sync_and, err, up, dsum);
+                                 sync_and, err, up, dsum, [] {});
 }
 
 // fp32 meshes of these orders with 16-byte aligned arrays run the even-odd

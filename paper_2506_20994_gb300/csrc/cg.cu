@@ -176,7 +176,9 @@ cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
                                  const T *__restrict__ w, const T *__restrict__ cm,
                                  const T *__restrict__ c, CgScalars *__restrict__ s,
                                  double *__restrict__ partials, int64_t n) {
-  const T alpha = (T)s->alpha;
+  ax::grid_wait();
+  ax::grid_go();
+  const T alpha = (T)__ldcg(&s->alpha);
   T a_rz = 0, a_rr = 0;
   auto point = [&](T &xq, T &rq, T pq, T wq, T cmq, T cq) {
     if constexpr (XUP) xq += alpha * pq;
@@ -194,7 +196,7 @@ cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
       using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
       constexpr int NV = 16 / sizeof(T);
       V xv[2], rv[2], pv[2], wv[2], mv[2], cv[2];
-      auto at = [](const T *f, int64_t v) { return reinterpret_cast<const V *>(f)[v]; };
+      auto at = [](const T *f, int64_t v) { return __ldcg(reinterpret_cast<const V *>(f) + v); };
       walk2(
           n / NV,
           [&](int k, int64_t v) {
@@ -221,8 +223,10 @@ cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
-    T xq = XUP ? x[q] : T(0);
-    point(xq, r[q], XUP ? p[q] : T(0), w[q], cm[q], RR ? c[q] : T(0));
+    T xq = XUP ? __ldcg(x + q) : T(0), rq = __ldcg(r + q);
+    point(xq, rq, XUP ? __ldcg(p + q) : T(0), __ldcg(w + q), __ldcg(cm + q),
+          RR ? __ldcg(c + q) : T(0));
+    r[q] = rq;
     if constexpr (XUP) x[q] = xq;
   }
   constexpr int NS = RR ? 2 : 1;
@@ -231,7 +235,8 @@ cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
   if constexpr (RR) v[1] = (double)a_rr;
   ax::block_sum<NS>(v);
   ax::finish_sums<NS>(v, partials, &s->ticket, [s](const double *t) {
-    s->beta = (s->rz != 0.0) ? t[0] / s->rz : 0.0;
+    const double rz = __ldcg(&s->rz);
+    s->beta = (rz != 0.0) ? t[0] / rz : 0.0;
     s->rz = t[0];
     if constexpr (RR) s->rr = t[1];
     if (!isfinite(t[0]) || (RR && !isfinite(t[NS - 1]))) s->status = 1;
@@ -535,7 +540,9 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
                                        : cg_update_kernel<T, true, false, !std::is_same_v<T, double>>)
                             : (checked ? cg_update_kernel<T, true, true, true>
                                        : cg_update_kernel<T, true, false, true>);
-      update<<<nb, kRedThreads, 0, st>>>(x, r, p, w, cm, c, P->scal, P->partials, n);
+      if (ax::launch_chained(true, update, nb, kRedThreads, 0, st, x, r, p, w, cm, c, P->scal,
+                             P->partials, n))
+        return AX_ELAUNCH;
     } else {
       rc = apply(w, p, st);
       if (rc) return rc;

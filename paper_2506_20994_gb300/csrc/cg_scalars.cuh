@@ -16,12 +16,13 @@ struct CgScalars {
 
 // alpha = rz / <p, Ap>
 AX_D void cg_set_alpha(CgScalars *s, double pap) {
+  const double rz = __ldcg(&s->rz);
   s->pap = pap;
-  if (!(pap > 0.0) || !isfinite(pap) || !isfinite(s->rz)) {
+  if (!(pap > 0.0) || !isfinite(pap) || !isfinite(rz)) {
     s->status = 1;
     s->alpha = 0.0;
   } else {
-    s->alpha = s->rz / pap;
+    s->alpha = rz / pap;
   }
 }
 

@@ -77,6 +77,42 @@ inline bool grant_smem(K kernel, size_t bytes, std::atomic<size_t> (&granted)[kM
   return true;
 }
 
+// Launches that may begin while the kernel before them in the stream is still
+// running (programmatic dependent launch): what remains of a launch between
+// two kernels is then hidden, 2-3 us of a 10 us apply.  Such a kernel calls
+// grid_wait() before it reads or writes anything another kernel may touch;
+// the wait returns when every earlier kernel of the stream has finished and
+// its writes are visible (each of them has waited in turn).  Behind the wait
+// it calls grid_go(), which lets the next launch begin: so at most one kernel
+// waits behind the running one, and its blocks take only what is free.
+// Behind the wait, data that other kernels write is read past L1 (__ldcg, the
+// bulk-copy engine): L1 is emptied when a kernel is launched, which here is
+// before the kernel in front of it is done, and read-only loads (const
+// __restrict__, __ldg) would return lines that kernel's neighbours have
+// rewritten since.  In front of the wait stands only what no kernel of the
+// stream can be writing: see EopArgs::chained.
+AX_D void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+AX_D void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline int launch_chained(bool chained, void (*kern)(P...), unsigned grid, unsigned block, size_t smem,
+                          cudaStream_t st, A &&...args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;  // without: after everything before it in the stream
+  if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return AX_ELAUNCH;
+  }
+  return AX_OK;
+}
+
 // Asks the memory system to bring [p, p + bytes) into L2 (bulk copy engine).
 // No data is returned.  The bulk unit needs a 16-byte aligned address and
 // size; anything else (a caller's offset view) is skipped, since a prefetch

@@ -47,7 +47,7 @@ __device__ __noinline__ void alpha_block(const ax::AlphaJob &job) {
   for (int v = 0; v < 1024 / kGsThreads; ++v) {
     const int vt = (int)threadIdx.x + v * kGsThreads;
     double a = 0.0;
-    for (int b = vt; b < job.n; b += 1024) a += __ldg(job.partials + b);
+    for (int b = vt; b < job.n; b += 1024) a += __ldcg(job.partials + b);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
     if ((vt & 31) == 0) sh[vt >> 5] = a;
@@ -69,6 +69,8 @@ __global__ void gs_sum_kernel(T *__restrict__ v, const int2 *__restrict__ pairs,
                               int64_t n_pairs, const int *__restrict__ off,
                               const int *__restrict__ idx, int64_t n_multi,
                               const ax::AlphaJob job) {
+  ax::grid_wait();
+  ax::grid_go();
   if (ALPHA && blockIdx.x == 0) {
     alpha_block(job);
     return;
@@ -76,7 +78,7 @@ __global__ void gs_sum_kernel(T *__restrict__ v, const int2 *__restrict__ pairs,
   const int64_t s = (int64_t)(blockIdx.x - (ALPHA ? 1 : 0)) * blockDim.x + threadIdx.x;
   if (s < n_pairs) {
     const int2 q = __ldg(pairs + s);
-    const T acc = v[q.x] + v[q.y];
+    const T acc = __ldcg(v + q.x) + __ldcg(v + q.y);
     v[q.x] = acc;
     v[q.y] = acc;
     return;
@@ -84,8 +86,8 @@ __global__ void gs_sum_kernel(T *__restrict__ v, const int2 *__restrict__ pairs,
   const int64_t m = s - n_pairs;
   if (m >= n_multi) return;
   const int b = __ldg(off + m), e = __ldg(off + m + 1);
-  T acc = v[__ldg(idx + b)];
-  for (int k = b + 1; k < e; ++k) acc += v[__ldg(idx + k)];
+  T acc = __ldcg(v + __ldg(idx + b));
+  for (int k = b + 1; k < e; ++k) acc += __ldcg(v + __ldg(idx + k));
   for (int k = b; k < e; ++k) v[__ldg(idx + k)] = acc;
 }
 
@@ -96,12 +98,10 @@ int gs_sum_launch(ax_gs *g, T *v, const ax::AlphaJob *job, cudaStream_t st) {
   if (g->n_shared > 0 && !v) return AX_EINVAL;
   const unsigned grid = (unsigned)((g->n_shared + kGsThreads - 1) / kGsThreads);
   if (job)
-    gs_sum_kernel<T, true><<<grid + 1, kGsThreads, 0, st>>>(v, g->d_pairs, g->n_pairs, g->d_off,
-                                                            g->d_idx, g->n_multi, *job);
-  else
-    gs_sum_kernel<T, false><<<grid, kGsThreads, 0, st>>>(v, g->d_pairs, g->n_pairs, g->d_off,
-                                                         g->d_idx, g->n_multi, ax::AlphaJob{});
-  return ax::launch_status();
+    return ax::launch_chained(true, gs_sum_kernel<T, true>, grid + 1, kGsThreads, 0, st, v, g->d_pairs,
+                              g->n_pairs, g->d_off, g->d_idx, g->n_multi, *job);
+  return ax::launch_chained(true, gs_sum_kernel<T, false>, grid, kGsThreads, 0, st, v, g->d_pairs,
+                            g->n_pairs, g->d_off, g->d_idx, g->n_multi, ax::AlphaJob{});
 }
 
 }  // namespace

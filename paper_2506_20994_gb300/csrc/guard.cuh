@@ -147,14 +147,14 @@ __device__ __noinline__ void element_f64(bool on, double *__restrict__ w, const 
     double ur = 0.0, us = 0.0, ut = 0.0;
 #pragma unroll 4
     for (int l = 0; l < LX; ++l) {
-      ur = __fma_rn(__ldg(dx + l * LX + i), u[eb + (k * LX + j) * LX + l], ur);
-      us = __fma_rn(__ldg(dy + l * LX + j), u[eb + (k * LX + l) * LX + i], us);
-      ut = __fma_rn(__ldg(dz + l * LX + k), u[eb + (l * LX + j) * LX + i], ut);
+      ur = __fma_rn(__ldcg(dx + l * LX + i), u[eb + (k * LX + j) * LX + l], ur);
+      us = __fma_rn(__ldcg(dy + l * LX + j), u[eb + (k * LX + l) * LX + i], us);
+      ut = __fma_rn(__ldcg(dz + l * LX + k), u[eb + (l * LX + j) * LX + i], ut);
     }
     const size_t q = eb + p;
-    const double a11 = __ldg(g11 + q), a22 = __ldg(g22 + q), a33 = __ldg(g33 + q);
-    const double a12 = __ldg(g12 + q), a13 = __ldg(g13 + q), a23 = __ldg(g23 + q);
-    const double hh = __ldg(h1 + q);
+    const double a11 = __ldcg(g11 + q), a22 = __ldcg(g22 + q), a33 = __ldcg(g33 + q);
+    const double a12 = __ldcg(g12 + q), a13 = __ldcg(g13 + q), a23 = __ldcg(g23 + q);
+    const double hh = __ldcg(h1 + q);
     sr[p] = hh * (a11 * ur + a12 * us + a13 * ut);
     ss[p] = hh * (a12 * ur + a22 * us + a23 * ut);
     st[p] = hh * (a13 * ur + a23 * us + a33 * ut);
@@ -165,9 +165,9 @@ __device__ __noinline__ void element_f64(bool on, double *__restrict__ w, const 
     double acc = 0.0;
 #pragma unroll 4
     for (int l = 0; l < LX; ++l) {
-      acc = __fma_rn(__ldg(dxt + l * LX + i), sr[(k * LX + j) * LX + l], acc);
-      acc = __fma_rn(__ldg(dyt + l * LX + j), ss[(k * LX + l) * LX + i], acc);
-      acc = __fma_rn(__ldg(dzt + l * LX + k), st[(l * LX + j) * LX + i], acc);
+      acc = __fma_rn(__ldcg(dxt + l * LX + i), sr[(k * LX + j) * LX + l], acc);
+      acc = __fma_rn(__ldcg(dyt + l * LX + j), ss[(k * LX + l) * LX + i], acc);
+      acc = __fma_rn(__ldcg(dzt + l * LX + k), st[(l * LX + j) * LX + i], acc);
     }
     w[eb + p] = acc;
     if (dot) *dot = __fma_rn(u[eb + p], acc, *dot);

@@ -1,0 +1,117 @@
+"""Kernels that may be launched while the one before them still runs: long
+chains in which each call reads what the call before it wrote, and the buffers
+come round again, must give the bits of the same chain with a synchronisation
+after every call; also under graph capture and after the geometry is
+rewritten."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2506_20994_gb300 as ax  # noqa: E402
+from paper_2506_20994_gb300 import synth  # noqa: E402
+
+from _cases import GKEYS, operator_case  # noqa: E402
+
+
+def _t(a, dt=torch.float64):
+    return torch.as_tensor(np.ascontiguousarray(a), device="cuda").to(dt)
+
+
+def _scale(c, dt=torch.float64):
+    """Operands scaled so that repeated applies stay in range."""
+    d = {k: _t(c[k], dt) for k in ("u", "dx", "dxt", "h1") + GKEYS}
+    d["h1"] = d["h1"] * float(0.3 * np.linalg.norm(c["u"]) / np.linalg.norm(c["w"]))
+    return d
+
+
+def _same(step, bufs, n=24):
+    """step(out, in, k) over three buffers in turn, with and without waits."""
+    ref = [b.clone() for b in bufs]
+    for k in range(n):
+        step(ref[(k + 1) % 3], ref[k % 3], k)
+        torch.cuda.synchronize()
+    for _ in range(3):
+        got = [b.clone() for b in bufs]
+        torch.cuda.synchronize()
+        for k in range(n):
+            step(got[(k + 1) % 3], got[k % 3], k)
+        torch.cuda.synchronize()
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dims,lx", [((1, 1, 1), 8), ((5, 3, 2), 6), ((8, 8, 8), 8),
+                                     ((9, 9, 8), 10), ((17, 13, 11), 6)])
+def test_handle_raw_and_gather_scatter_chains(dims, lx):
+    c = operator_case(dims, lx, seed=600 + lx)
+    d = _scale(c)
+    G = [d[k] for k in GKEYS]
+    op = ax.Operator(lx, d["dx"], d["dxt"], d["h1"], *G)
+    gs = ax.GatherScatter(ax.box_numbering(*dims, lx))
+    bufs = [d["u"].clone(), torch.zeros_like(d["u"]), torch.zeros_like(d["u"])]
+    _same(lambda w, u, k: op.apply(w, u), bufs)
+    _same(lambda w, u, k: ax.ax_helm(w, u, d["dx"], d["dxt"], d["h1"], *G, lx), bufs)
+
+    def mixed(w, u, k):
+        if k % 2:
+            op.apply(w, u)
+        else:
+            ax.ax_helm(w, u, d["dx"], d["dxt"], d["h1"], *G, lx)
+        gs.sum(w)
+        if k % 5 == 4:
+            w.mul_(0.5)  # a kernel of another library in between
+    _same(mixed, bufs)
+
+
+def test_rewritten_geometry_and_capture():
+    lx = 8
+    c = operator_case((6, 5, 4), lx, seed=611)
+    d = _scale(c)
+    op = ax.Operator(lx, d["dx"], d["dxt"], d["h1"], *[d[k] for k in GKEYS])
+    h = [d["h1"], (d["h1"] * 1.25).contiguous()]
+    bufs = [d["u"].clone(), torch.zeros_like(d["u"]), torch.zeros_like(d["u"])]
+
+    def step(w, u, k):
+        if k % 3 == 0:
+            op.set_h1(h[(k // 3) % 2])
+        op.apply(w, u)
+    _same(step, bufs)
+    # a captured chain, replayed after the geometry changed outside the graph
+    a, b = torch.empty_like(d["u"]), torch.empty_like(d["u"])
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        op.set_h1(h[0])
+        op.apply(a, d["u"])
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            for _ in range(4):
+                op.apply(a, d["u"])
+                op.apply(b, a)
+        for q in (0, 1, 0):
+            op.set_h1(h[q])
+            g.replay()
+            s.synchronize()
+            got = b.clone()
+            op.apply(a, d["u"])
+            s.synchronize()
+            op.apply(b, a)
+            s.synchronize()
+            assert torch.equal(got, b)
+
+
+def test_solvers_repeat_bitwise():
+    P = ax.Poisson(synth.box_vertices(9, 8, 7, seed=4), 8)
+    P.set_check_every(8)
+    b = P.rhs(synth.poisson_source)
+    x0, n0 = P.cg(b, tol=1e-9)[:2]
+    r = P.residual(b, x0).reshape(-1)
+    cm = P.gs.inverse_multiplicity()
+    bb = b.reshape(-1)
+    assert float((cm * r * r).sum()) <= (1.5e-9) ** 2 * float((cm * bb * bb).sum())
+    for _ in range(4):
+        x, n = P.cg(b, tol=1e-9)[:2]
+        assert n == n0 and torch.equal(x, x0)
