@@ -76,13 +76,13 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
   __syncthreads();
 
   for (int t = threadIdx.x; t < N2; t += blockDim.x) {
-    const double a = __ldg(dx + t), at = __ldg(dxt + t);
+    const double a = __ldcg(dx + t), at = __ldcg(dxt + t);
     guard::note_d(rec, a);
     guard::note_d(rec, at);
     sdx[t] = split(a);
     sdxt[t] = split(at);
     if constexpr (XYZ) {
-      const double b = __ldg(dy + t), c = __ldg(dz + t), bt = __ldg(dyt + t), ct = __ldg(dzt + t);
+      const double b = __ldcg(dy + t), c = __ldcg(dz + t), bt = __ldcg(dyt + t), ct = __ldcg(dzt + t);
       guard::note_d(rec, b);
       guard::note_d(rec, c);
       guard::note_d(rec, bt);
@@ -107,7 +107,7 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
   if (own) {
 #pragma unroll
     for (int k = 0; k < LX; ++k) {
-      const double x = active ? __ldg(u + base + (size_t)k * N2) : 0.0;
+      const double x = active ? __ldcg(u + base + (size_t)k * N2) : 0.0;
       ukey = max(ukey, guard::key(x));
       uk[k] = split(x);
       su[k * N2 + p] = uk[k];
@@ -133,9 +133,9 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
       df2 wr{0.f, 0.f}, ws{0.f, 0.f}, wt{0.f, 0.f};
       if (active) {
         const size_t q = base + (size_t)k * N2;
-        const double v11 = __ldg(g11 + q), v22 = __ldg(g22 + q), v33 = __ldg(g33 + q);
-        const double v12 = __ldg(g12 + q), v13 = __ldg(g13 + q), v23 = __ldg(g23 + q);
-        const double vh = __ldg(h1 + q);
+        const double v11 = __ldcg(g11 + q), v22 = __ldcg(g22 + q), v33 = __ldcg(g33 + q);
+        const double v12 = __ldcg(g12 + q), v13 = __ldcg(g13 + q), v23 = __ldcg(g23 + q);
+        const double vh = __ldcg(h1 + q);
         gkey = max(gkey, max(max(guard::key(v11), guard::key(v22)),
                              max(max(guard::key(v33), guard::key(v12)),
                                  max(guard::key(v13), guard::key(v23)))));
@@ -208,6 +208,8 @@ ax_df64_kernel(double *__restrict__ w, const double *__restrict__ u,
                const double *__restrict__ g12, const double *__restrict__ g13,
                const double *__restrict__ g23, int nelv, int epb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_wait();
+  grid_go();
   const long long e0 = (long long)blockIdx.x * epb;
   const long long left = nelv - e0;
   const int nel = left < epb ? (int)left : epb;
@@ -226,9 +228,8 @@ int launch_df64(double *w, const double *u, const double *dx, const double *dxt,
   static std::atomic<size_t> granted[kMaxDevices];
   if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
-  kern<<<grid, epb * LX * LX, smem, stream>>>(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23,
-                                              nelv, epb);
-  return launch_status();
+  return launch_chained(true, kern, grid, epb * LX * LX, smem, stream, w, u, dx, dxt, h1, g11, g22,
+                        g33, g12, g13, g23, nelv, epb);
 }
 
 }  // namespace ax

@@ -105,9 +105,9 @@ __device__ __forceinline__ void df64eo_body(double *__restrict__ w, const double
 #pragma unroll
     for (int tr = 0; tr < 2; ++tr) {
       const double *m = tr ? dxt : dx;
-      const double da = __ldg(m + l * LX + i), db = __ldg(m + (N - l) * LX + i);
-      guard::note_pair(rec, da, __ldg(m + (N - l) * LX + (N - i)));
-      guard::note_pair(rec, db, __ldg(m + l * LX + (N - i)));
+      const double da = __ldcg(m + l * LX + i), db = __ldcg(m + (N - l) * LX + i);
+      guard::note_pair(rec, da, __ldcg(m + (N - l) * LX + (N - i)));
+      guard::note_pair(rec, db, __ldcg(m + l * LX + (N - i)));
       const df2 a = split(da), b = split(db);
       // lanes: x = (a + b)/2, y = (a - b)/2 (exact halving)
       dd2 s = dsum2(dd2{pk(a.hi, a.hi), pk(a.lo, a.lo)}, dd2{pk(b.hi, -b.hi), pk(b.lo, -b.lo)});
@@ -191,7 +191,7 @@ __device__ __forceinline__ void df64eo_body(double *__restrict__ w, const double
         for (int b = 0; b < 2; ++b)
 #pragma unroll
           for (int a = 0; a < 2; ++a) {
-            const double x = active ? __ldg(u + gidx(c, b, a)) : 0.0;
+            const double x = active ? __ldcg(u + gidx(c, b, a)) : 0.0;
             ukey = max(ukey, guard::key(x));
             gr[c][b][a] = split(x);
           }
@@ -206,7 +206,7 @@ __device__ __forceinline__ void df64eo_body(double *__restrict__ w, const double
     const size_t x = gidx((q >> 2) & 1, (q >> 1) & 1, q & 1);
     const double *fld[7] = {g11, g22, g33, g12, g13, g23, h1};
 #pragma unroll
-    for (int f = 0; f < 7; ++f) g.v[f] = __ldg(fld[f] + x);
+    for (int f = 0; f < 7; ++f) g.v[f] = __ldcg(fld[f] + x);
   };
   eo::GeoStage geo[2];
   if (active) load_geo(0, geo[0]);
@@ -367,6 +367,8 @@ ax_df64eo_kernel(double *__restrict__ w, const double *__restrict__ u,
                  const double *__restrict__ g12, const double *__restrict__ g13,
                  const double *__restrict__ g23, int nelv, int epb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_wait();
+  grid_go();
   const long long e0 = (long long)blockIdx.x * epb;
   const long long left = nelv - e0;
   const int nel = left < epb ? (int)left : epb;
@@ -386,9 +388,7 @@ int launch_df64eo(double *w, const double *u, const double *dx, const double *dx
   static std::atomic<size_t> granted[kMaxDevices];
   if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
-  kern<<<grid, epb * H3, smem, stream>>>(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, nelv,
-                                         epb);
-  return launch_status();
+  return launch_chained(true, kern, grid, epb * H3, smem, stream, w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, nelv, epb);
 }
 
 }  // namespace ax

@@ -326,8 +326,8 @@ AX_D void e32_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     for (int q = tid; q < 2 * H2; q += C::NTB) {
       const int m = q / H2, i = (q / H) % H, l = q % H;
       const float *D = m ? M.dxt : M.dx;  // M(i, l) = D[l * lx + i]
-      const float a = __ldg(D + l * LX + i), b = __ldg(D + (N - l) * LX + i);
-      const float a2 = __ldg(D + l * LX + N - i), b2 = __ldg(D + (N - l) * LX + N - i);
+      const float a = __ldcg(D + l * LX + i), b = __ldcg(D + (N - l) * LX + i);
+      const float a2 = __ldcg(D + l * LX + N - i), b2 = __ldcg(D + (N - l) * LX + N - i);
       const float A = __fmul_rn(0.5f, __fadd_rn(a, b)), B = __fmul_rn(0.5f, __fsub_rn(a, b));
       const float A2 = __fmul_rn(0.5f, __fadd_rn(a2, b2));
       const float B2 = __fmul_rn(0.5f, __fsub_rn(a2, b2));
@@ -385,7 +385,7 @@ AX_D void e32_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   sync();  // the barriers are initialised before anyone waits on them
   if (tid == 0 && have) issue(pos, 0);
 
-  const float beta = PUPD ? (float)*up.beta : 0.f;  // the solver's scalar, on the device
+  const float beta = PUPD ? (float)__ldcg(up.beta) : 0.f;  // the solver's scalar, on the device
   unsigned n = 0;  // elements done by this group
   while (have) {
     const int cmesh = seq.mesh_of(pos);
@@ -518,6 +518,8 @@ ax_eo32_kernel(const Mesh<SU, SG> mesh, long long nelv, int *__restrict__ err,
                double *__restrict__ dotp, const E32Upd up) {
   using C = Cfg<LX, SU, SG, PUPD>;
   extern __shared__ __align__(128) unsigned char sm[];
+  grid_wait();
+  grid_go();
   const SeqOne<SU, SG> seq{mesh, nelv};
   double dsum = 0.0;
   e32_run<LX, SU, SG, DOT, PUPD, kE32CoefRegs>(
@@ -602,19 +604,19 @@ int launch(float *w, const SU *u, const float *dx, const float *dxt, const SG *c
     if constexpr (std::is_same_v<SU, float>) {
       if (!dotp || !up->pw || !up->r || !up->minv || !up->beta) return AX_EINVAL;
       using C = Cfg<LX, SU, SG, true>;
-      ax_eo32_kernel<LX, SU, SG, true, true><<<nb, C::NTB, C::SMEM, st>>>(m, nelv, err, dotp,
-                                                                          *up);
+      return launch_chained(true, ax_eo32_kernel<LX, SU, SG, true, true>, nb, C::NTB, C::SMEM, st, m,
+                            nelv, err, dotp, *up);
     } else {
       return AX_EINVAL;
     }
   } else if (dotp) {
     using C = Cfg<LX, SU, SG>;
-    ax_eo32_kernel<LX, SU, SG, true><<<nb, C::NTB, C::SMEM, st>>>(m, nelv, err, dotp, none);
-  } else {
-    using C = Cfg<LX, SU, SG>;
-    ax_eo32_kernel<LX, SU, SG, false><<<nb, C::NTB, C::SMEM, st>>>(m, nelv, err, dotp, none);
+    return launch_chained(true, ax_eo32_kernel<LX, SU, SG, true>, nb, C::NTB, C::SMEM, st, m, nelv, err,
+                          dotp, none);
   }
-  return launch_status();
+  using C = Cfg<LX, SU, SG>;
+  return launch_chained(true, ax_eo32_kernel<LX, SU, SG, false>, nb, C::NTB, C::SMEM, st, m, nelv, err,
+                        dotp, none);
 }
 
 }  // namespace e32

@@ -92,13 +92,15 @@ ax_eo32w_kernel(const e32::Mesh<SU, SG> M, long long nelv, int *__restrict__ err
   const uint32_t barU = eop::smem_u32(sm + C::OFF_BAR + wp * 16), barG = barU + 8;
   double *red = reinterpret_cast<double *>(sm + C::OFF_BAR + kWarps * 16);
 
+  grid_wait();
+  grid_go();
   // even-odd coefficients of dx (m = 0) and dxt (m = 1): M(i, l) = D[l * 8 + i]
   bool ok = true;
   for (int q = threadIdx.x; q < 2 * H2; q += blockDim.x) {
     const int m = q / H2, i = (q / H) % H, l = q % H;
     const float *D = m ? M.dxt : M.dx;
-    const float a = __ldg(D + l * LX + i), b = __ldg(D + (N - l) * LX + i);
-    const float a2 = __ldg(D + l * LX + N - i), b2 = __ldg(D + (N - l) * LX + N - i);
+    const float a = __ldcg(D + l * LX + i), b = __ldcg(D + (N - l) * LX + i);
+    const float a2 = __ldcg(D + l * LX + N - i), b2 = __ldcg(D + (N - l) * LX + N - i);
     const float A = __fmul_rn(0.5f, __fadd_rn(a, b)), B = __fmul_rn(0.5f, __fsub_rn(a, b));
     const float A2 = __fmul_rn(0.5f, __fadd_rn(a2, b2));
     const float B2 = __fmul_rn(0.5f, __fsub_rn(a2, b2));
@@ -303,7 +305,7 @@ ax_eo32w_kernel(const e32::Mesh<SU, SG> M, long long nelv, int *__restrict__ err
   };
 
   double dsum = 0.0;
-  const float beta = PUPD ? (float)*up.beta : 0.f;  // the solver's scalar, on the device
+  const float beta = PUPD ? (float)__ldcg(up.beta) : 0.f;  // the solver's scalar, on the device
   // the element loop, compiled for both matrix forms (gen: CTA-uniform)
   auto run = [&](auto gen) __attribute__((always_inline)) {
     for (unsigned parity = 0u; e < nelv; e += nw, parity ^= 1u) {

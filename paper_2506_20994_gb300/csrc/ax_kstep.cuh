@@ -273,6 +273,8 @@ ax_kstep_kernel(W *__restrict__ w, const SU *__restrict__ u, const T *__restrict
                 const S *__restrict__ g33, const S *__restrict__ g12,
                 const S *__restrict__ g13, const S *__restrict__ g23, int nelv, int epb,
                 double *__restrict__ dotp) {
+  grid_wait();
+  grid_go();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long e0 = (long long)blockIdx.x * epb;
   const long long left = nelv - e0;
@@ -309,9 +311,8 @@ int launch_kstep(W *w, const SU *u, const T *dx, const T *dxt, const S *h1, cons
   static std::atomic<size_t> granted[2][kMaxDevices];  // per kernel
   if (!grant_smem(kern, smem, granted[dotp != nullptr])) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
-  kern<<<grid, epb * LX * LX, smem, stream>>>(w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23,
-                                              nelv, epb, dotp);
-  return launch_status();
+  return launch_chained(true, kern, grid, epb * LX * LX, smem, stream, w, u, dx, dxt, h1, g11, g22,
+                        g33, g12, g13, g23, nelv, epb, dotp);
 }
 
 }  // namespace ax

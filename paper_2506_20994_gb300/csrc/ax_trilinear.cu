@@ -81,17 +81,20 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
   const long long e = active ? e0 + le : 0;
   const size_t base = (size_t)e * N3 + p;
 
+  grid_wait();
+  grid_go();
   for (int t = threadIdx.x; t < N2; t += blockDim.x) {
     const int a = t / LX, b = t % LX;
-    Fd[b * RS + a] = dx[t];
-    Bd[b * RS + a] = dxt[t];
-    Td[a * RS + b] = dxt[t];
+    const float f = __ldcg(dx + t), g = __ldcg(dxt + t);
+    Fd[b * RS + a] = f;
+    Bd[b * RS + a] = g;
+    Td[a * RS + b] = g;
   }
   for (int t = threadIdx.x; t < LX; t += blockDim.x) {
-    const double x = xi[t];
+    const double x = __ldcg(xi + t);
     phi0[t] = (float)(0.5 * (1.0 - x));
     phi1[t] = (float)(0.5 * (1.0 + x));
-    swq[t] = (float)wq[t];
+    swq[t] = (float)__ldcg(wq + t);
   }
   // half edge vectors of the trilinear map, corner index ((c*2+b)*2+a)*3+coord
   for (int t = p; active && t < 36; t += N2) {  // lx < 6: fewer than 36 threads
@@ -108,14 +111,14 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
       c1 = c0 + 4;
     }
     const double *x = corners + (size_t)e * 24;
-    cf[t] = (float)(0.5 * (x[c1 * 3 + d] - x[c0 * 3 + d]));
+    cf[t] = 0.5f * (float)(__ldcg(x + c1 * 3 + d) - __ldcg(x + c0 * 3 + d));
   }
 
   float uk[LX];
   if (own) {
 #pragma unroll
     for (int k = 0; k < LX; ++k) {
-      uk[k] = active ? u[base + (size_t)k * N2] : 0.f;
+      uk[k] = active ? __ldcg(u + base + (size_t)k * N2) : 0.f;
       su[k * N2 + p] = uk[k];
     }
   }
@@ -192,7 +195,7 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
         const float A22 = __fmaf_rn(a, f, -b * d);
         const float det = __fmaf_rn(a, A00, __fmaf_rn(b, A10, c * A20));
         float s = __fdividef(wij * swq[k], det);  // fp32 operator: ~2 ulp is ample
-        if (H1) s *= h1[base + (size_t)k * N2];
+        if (H1) s *= __ldcg(h1 + base + (size_t)k * N2);
         const float g11 = s * __fmaf_rn(A00, A00, __fmaf_rn(A01, A01, A02 * A02));
         const float g22 = s * __fmaf_rn(A10, A10, __fmaf_rn(A11, A11, A12 * A12));
         const float g33 = s * __fmaf_rn(A20, A20, __fmaf_rn(A21, A21, A22 * A22));
@@ -263,8 +266,8 @@ int launch_tri(float *w, const float *u, const float *dx, const float *dxt, cons
   static std::atomic<size_t> granted[2][kMaxDevices];
   if (!grant_smem(kern, smem, granted[h1 != nullptr])) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
-  kern<<<grid, epb * LX * LX, smem, st>>>(w, u, dx, dxt, h1, corners, xi, wq, nelv, epb);
-  return launch_status();
+  return launch_chained(true, kern, grid, epb * LX * LX, smem, st, w, u, dx, dxt, h1, corners, xi,
+                        wq, nelv, epb);
 }
 
 }  // namespace

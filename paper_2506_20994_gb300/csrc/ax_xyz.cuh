@@ -23,6 +23,8 @@ namespace xyz {
 template <int LX>
 __global__ void __launch_bounds__(256) ax_df64_xyz_kernel(AX_XYZ_PARAMS) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_wait();
+  grid_go();
   const long long e0 = (long long)blockIdx.x * epb;
   const long long left = nelv - e0;
   const int nel = left < epb ? (int)left : epb;
@@ -33,6 +35,8 @@ __global__ void __launch_bounds__(256) ax_df64_xyz_kernel(AX_XYZ_PARAMS) {
 template <int LX>
 __global__ void __launch_bounds__(256) ax_kstep_xyz_kernel(AX_XYZ_PARAMS) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_wait();
+  grid_go();
   const long long e0 = (long long)blockIdx.x * epb;
   const long long left = nelv - e0;
   const int nel = left < epb ? (int)left : epb;
@@ -60,8 +64,7 @@ int launch_xyz(AX_XYZ_PARAMS, cudaStream_t st) {
   static std::atomic<size_t> granted[kMaxDevices];
   if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
-  kern<<<grid, epb * LX * LX, smem, st>>>(AX_XYZ_ARGS);
-  return launch_status();
+  return launch_chained(true, kern, grid, epb * LX * LX, smem, st, AX_XYZ_ARGS);
 }
 
 // per lx range (one translation unit each): a 2-7, b 8-10, c 11-12, d 13-16

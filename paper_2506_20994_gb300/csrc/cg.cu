@@ -150,12 +150,14 @@ __global__ void mask_dot_kernel(T *__restrict__ w, const T *__restrict__ p,
                                 const T *__restrict__ mask, const T *__restrict__ c,
                                 double *__restrict__ partials, int64_t n,
                                 CgScalars *__restrict__ s = nullptr) {
+  ax::grid_wait();
+  ax::grid_go();
   T a = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
-    const T wv = w[q] * mask[q];
+    const T wv = __ldcg(w + q) * __ldcg(mask + q);
     w[q] = wv;
-    a += c[q] * p[q] * wv;
+    a += __ldcg(c + q) * __ldcg(p + q) * wv;
   }
   double v[1] = {(double)a};
   ax::block_sum<1>(v);
@@ -257,7 +259,9 @@ template <typename T>
 __global__ void cg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
                             const T *__restrict__ minv, const CgScalars *__restrict__ s,
                             int64_t n) {
-  const T beta = (T)s->beta;
+  ax::grid_wait();
+  ax::grid_go();
+  const T beta = (T)__ldcg(&s->beta);
   int64_t q0 = 0;
   if constexpr (sizeof(T) == 4) {
     if (aligned16(p, r, minv)) {  // fp32: 16-byte accesses
@@ -265,8 +269,9 @@ __global__ void cg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
       const int64_t n4 = n / 4;
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
            v += (int64_t)gridDim.x * blockDim.x) {
-        V pv = reinterpret_cast<V *>(p)[v];
-        const V rv = reinterpret_cast<const V *>(r)[v], mv = reinterpret_cast<const V *>(minv)[v];
+        V pv = __ldcg(reinterpret_cast<const V *>(p) + v);
+        const V rv = __ldcg(reinterpret_cast<const V *>(r) + v);
+        const V mv = __ldcg(reinterpret_cast<const V *>(minv) + v);
         pv.x = mv.x * rv.x + beta * pv.x;
         pv.y = mv.y * rv.y + beta * pv.y;
         pv.z = mv.z * rv.z + beta * pv.z;
@@ -278,7 +283,7 @@ __global__ void cg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x)
-    p[q] = minv[q] * r[q] + beta * p[q];
+    p[q] = __ldcg(minv + q) * __ldcg(r + q) + beta * __ldcg(p + q);
 }
 
 // out = a .* b; out += a
@@ -546,9 +551,11 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
     } else {
       rc = apply(w, p, st);
       if (rc) return rc;
-      mask_dot_kernel<T><<<nb, kRedThreads, 0, st>>>(w, p, mask, c, P->partials, n, P->scal);
-      cg_update_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, p, w, cm, c, P->scal, P->partials,
-                                                      n);
+      rc = ax::launch_chained(true, mask_dot_kernel<T>, nb, kRedThreads, 0, st, w, p, mask, c,
+                              P->partials, n, P->scal) |
+           ax::launch_chained(true, cg_update_kernel<T>, nb, kRedThreads, 0, st, x, r, p, w, cm, c,
+                              P->scal, P->partials, n);
+      if (rc) return AX_ELAUNCH;
     }
     ++it;
     if (it % P->check_every == 0 || it == maxit) {
@@ -566,7 +573,9 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
         break;
       }
     }
-    if (!fused_p) cg_p_kernel<T><<<nb, kRedThreads, 0, st>>>(p, r, minv, P->scal, n);
+    if (!fused_p && ax::launch_chained(true, cg_p_kernel<T>, nb, kRedThreads, 0, st, p, r, minv,
+                                       P->scal, n))
+      return AX_ELAUNCH;
   }
   if constexpr (std::is_same_v<T, double>)
     if (fused_x && it > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
@@ -1016,7 +1025,9 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
                                   const T *__restrict__ c, const T *__restrict__ cm,
                                   CgScalars *__restrict__ s,
                                   double *__restrict__ partials, int64_t n) {
-  const T alpha = (T)s->alpha;
+  ax::grid_wait();
+  ax::grid_go();
+  const T alpha = (T)__ldcg(&s->alpha);
   T a_rr = 0;
   auto point = [&](T &xq, T &rq, T &roq, T pq, T wq, T cq, T cmq) {
     if constexpr (XUP) xq += alpha * pq;
@@ -1029,7 +1040,7 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
     using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
     constexpr int NV = 16 / sizeof(T);
     V xv[2], rv[2], pv[2], wv[2], mv[2], cv[2];
-    auto at = [](const T *f, int64_t v) { return reinterpret_cast<const V *>(f)[v]; };
+    auto at = [](const T *f, int64_t v) { return __ldcg(reinterpret_cast<const V *>(f) + v); };
     walk2(
         n / NV,
         [&](int k, int64_t v) {
@@ -1059,8 +1070,11 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
-    T xq = XUP ? x[q] : T(0);
-    point(xq, r[q], r_old[q], XUP ? p[q] : T(0), w[q], RR ? c[q] : T(0), MASKW ? cm[q] : T(1));
+    T xq = XUP ? __ldcg(x + q) : T(0), rq = __ldcg(r + q), old;
+    point(xq, rq, old, XUP ? __ldcg(p + q) : T(0), __ldcg(w + q), RR ? __ldcg(c + q) : T(0),
+          MASKW ? __ldcg(cm + q) : T(1));
+    r_old[q] = old;
+    r[q] = rq;
     if constexpr (XUP) x[q] = xq;
   }
   if constexpr (RR) {
@@ -1082,6 +1096,8 @@ fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
                                 const T *__restrict__ c, int have_corr, int first,
                                 CgScalars *__restrict__ s, double *__restrict__ partials,
                                 int64_t n) {
+  ax::grid_wait();
+  ax::grid_go();
   T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
   auto point = [&](T rv, T ro, T cmv, T cv, T ev) {
     const T a = cmv * rv;
@@ -1101,7 +1117,7 @@ fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
 #pragma unroll 2
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
            v += (int64_t)gridDim.x * blockDim.x) {
-        auto at = [v](const T *p) { return reinterpret_cast<const V *>(p)[v]; };
+        auto at = [v](const T *p) { return __ldcg(reinterpret_cast<const V *>(p) + v); };
         const V rv = at(r), ro = at(r_old), mv = at(cm);
         const V cv = have_corr ? at(c) : V{}, ev = have_corr ? at(corr) : V{};
         point(rv.x, ro.x, mv.x, cv.x, ev.x);
@@ -1114,22 +1130,20 @@ fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x)
-    point(r[q], r_old[q], cm[q], have_corr ? c[q] : T(0), have_corr ? corr[q] : T(0));
+    point(__ldcg(r + q), __ldcg(r_old + q), __ldcg(cm + q), have_corr ? __ldcg(c + q) : T(0),
+          have_corr ? __ldcg(corr + q) : T(0));
   double v[4] = {(double)d0, (double)d1, (double)d2, (double)d3};
   ax::block_sum<4>(v);
   ax::finish_sums<4>(v, partials, &s->ticket, [s, have_corr, first](const double *t) {
     const double rz_l = t[0] + t[1], rz_j = t[0];
     const double num_l = rz_l - (t[2] + t[3]), num_j = t[0] - t[2];
     const bool ok_l = have_corr && rz_l > 0.0 && isfinite(rz_l) && isfinite(num_l);
-    if (have_corr && !ok_l) s->fallbacks += 1;
+    if (have_corr && !ok_l) s->fallbacks = __ldcg(&s->fallbacks) + 1;
     const double rz = ok_l ? rz_l : rz_j;
     const double num = ok_l ? num_l : num_j;
     s->use_corr = ok_l ? 1 : 0;
-    if (first) {
-      s->beta = 0.0;
-    } else {
-      s->beta = (s->rz != 0.0) ? num / s->rz : 0.0;
-    }
+    const double old = __ldcg(&s->rz);
+    s->beta = (!first && old != 0.0) ? num / old : 0.0;
     s->rz = rz;
     if (!isfinite(rz)) s->status = 1;
   });
@@ -1140,8 +1154,10 @@ template <typename T>
 __global__ void fcg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
                              const T *__restrict__ minv, const T *__restrict__ corr,
                              const CgScalars *__restrict__ s, int first, int64_t n) {
-  const T beta = first ? T(0) : (T)s->beta;
-  const bool uc = s->use_corr != 0;
+  ax::grid_wait();
+  ax::grid_go();
+  const T beta = first ? T(0) : (T)__ldcg(&s->beta);
+  const bool uc = __ldcg(&s->use_corr) != 0;
   // explicit roundings: the Jacobi-only step is the same bits whether or not
   // a (zero) correction is present
   auto point = [&](T &pq, T mq, T rq, T cq) {
@@ -1156,9 +1172,9 @@ __global__ void fcg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
       const int64_t n4 = n / 4;
       for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
            v += (int64_t)gridDim.x * blockDim.x) {
-        V pv = first ? V{} : reinterpret_cast<V *>(p)[v];
-        const V rv = reinterpret_cast<const V *>(r)[v], mv = reinterpret_cast<const V *>(minv)[v];
-        const V cv = uc ? reinterpret_cast<const V *>(corr)[v] : V{};
+        auto at = [v](const T *f) { return __ldcg(reinterpret_cast<const V *>(f) + v); };
+        V pv = first ? V{} : at(p);
+        const V rv = at(r), mv = at(minv), cv = uc ? at(corr) : V{};
         point(pv.x, mv.x, rv.x, cv.x);
         point(pv.y, mv.y, rv.y, cv.y);
         point(pv.z, mv.z, rv.z, cv.z);
@@ -1170,8 +1186,8 @@ __global__ void fcg_p_kernel(T *__restrict__ p, const T *__restrict__ r,
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
-    T pq = first ? T(0) : p[q];
-    point(pq, minv[q], r[q], uc ? corr[q] : T(0));
+    T pq = first ? T(0) : __ldcg(p + q);
+    point(pq, __ldcg(minv + q), __ldcg(r + q), uc ? __ldcg(corr + q) : T(0));
     p[q] = pq;
   }
 }
@@ -1234,11 +1250,12 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
       if (rc) return rc;
       if ((rc = gs_sum_t<T>(P->gs, corr, st))) return rc;
     }
-    fcg_dots_kernel<T><<<nb, kRedThreads, 0, st>>>(r, r_old, corr, cm, c, have, first, P->scal,
-                                                   P->partials, n);
-    if (first || !fused_p)
-      fcg_p_kernel<T><<<nb, kRedThreads, 0, st>>>(p, r, minv, corr, P->scal, first, n);
-    return ax::launch_status();
+    int rc = ax::launch_chained(true, fcg_dots_kernel<T>, nb, kRedThreads, 0, st, r, r_old, corr, cm,
+                                c, have, first, P->scal, P->partials, n);
+    if (rc == AX_OK && (first || !fused_p))
+      rc = ax::launch_chained(true, fcg_p_kernel<T>, nb, kRedThreads, 0, st, p, r, minv, corr,
+                              P->scal, first, n);
+    return rc;
   };
   auto read_scalars = [&]() -> int {
     if (cudaMemcpyAsync(P->scal_host, P->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost, st) !=
@@ -1274,12 +1291,16 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
                                        : fcg_update_kernel<T, true, true, true>)
                             : (fused_p ? fcg_update_kernel<T, true, false, !std::is_same_v<T, double>>
                                        : fcg_update_kernel<T, true, false, true>);
-      update<<<nb, kRedThreads, 0, st>>>(x, r, r_old, p, w, c, cm, P->scal, P->partials, n);
+      if (ax::launch_chained(true, update, nb, kRedThreads, 0, st, x, r, r_old, p, w, c, cm, P->scal,
+                             P->partials, n))
+        return AX_ELAUNCH;
     } else {
       if ((rc = apply(w, p, st))) return rc;
-      mask_dot_kernel<T><<<nb, kRedThreads, 0, st>>>(w, p, mask, c, P->partials, n, P->scal);
-      fcg_update_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, r_old, p, w, c, cm, P->scal,
-                                                       P->partials, n);
+      rc = ax::launch_chained(true, mask_dot_kernel<T>, nb, kRedThreads, 0, st, w, p, mask, c,
+                              P->partials, n, P->scal) |
+           ax::launch_chained(true, fcg_update_kernel<T>, nb, kRedThreads, 0, st, x, r, r_old, p, w,
+                              c, cm, P->scal, P->partials, n);
+      if (rc) return AX_ELAUNCH;
     }
     ++it;
     if (it % P->check_every == 0 || it == maxit) {
@@ -1476,15 +1497,17 @@ __global__ void energy_features_kernel(float *__restrict__ X, double *__restrict
   constexpr int KEEP = 4;
   __shared__ double inv_b;
   const size_t base = (size_t)blockIdx.x * N;
+  ax::grid_wait();
+  ax::grid_go();
   double ss = 0.0, z[KEEP];
 #pragma unroll
   for (int q = 0; q < KEEP; ++q) {
     const int k = threadIdx.x + q * kRedThreads;
-    z[q] = k < N ? isc[base + k] * r[base + k] : 0.0;
+    z[q] = k < N ? __ldcg(isc + base + k) * __ldcg(r + base + k) : 0.0;
     ss += z[q] * z[q];
   }
   for (int k = threadIdx.x + KEEP * kRedThreads; k < N; k += kRedThreads) {
-    const double y = isc[base + k] * r[base + k];
+    const double y = __ldcg(isc + base + k) * __ldcg(r + base + k);
     ss += y * y;
   }
   double v[1] = {ss};
@@ -1502,16 +1525,18 @@ __global__ void energy_features_kernel(float *__restrict__ X, double *__restrict
     if (k < N) X[base + k] = (float)(z[q] * inv);
   }
   for (int k = threadIdx.x + KEEP * kRedThreads; k < N; k += kRedThreads)
-    X[base + k] = (float)(isc[base + k] * r[base + k] * inv);
+    X[base + k] = (float)(__ldcg(isc + base + k) * __ldcg(r + base + k) * inv);
 }
 
 // d = e - minv r - corr (corr assembled by gs before)
 __global__ void energy_diff_kernel(double *__restrict__ d, const double *__restrict__ e,
                                    const double *__restrict__ r, const double *__restrict__ minv,
                                    const double *__restrict__ corr, int64_t n) {
+  ax::grid_wait();
+  ax::grid_go();
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x)
-    d[q] = e[q] - minv[q] * r[q] - corr[q];
+    d[q] = __ldcg(e + q) - __ldcg(minv + q) * __ldcg(r + q) - __ldcg(corr + q);
 }
 
 // q = mask .* w (not stored); the partials of <d, q> and the output gradient
@@ -1524,18 +1549,23 @@ __global__ void energy_dot_dy_kernel(float *__restrict__ dY, const double *__res
                                      const double *__restrict__ s, const double *__restrict__ eA,
                                      int N, int nelv, double *__restrict__ partials) {
   __shared__ double scale_b;
-  if (threadIdx.x == 0) scale_b = eA[0] > 0.0 ? -2.0 / eA[0] : 0.0;
+  ax::grid_wait();
+  ax::grid_go();
+  if (threadIdx.x == 0) {
+    const double a0 = __ldcg(eA);
+    scale_b = a0 > 0.0 ? -2.0 / a0 : 0.0;
+  }
   __syncthreads();
   const double scale = scale_b;
   double a = 0.0;
   for (int e = blockIdx.x; e < nelv; e += gridDim.x) {
-    const double se = scale * s[e];
+    const double se = scale * __ldcg(s + e);
     const size_t base = (size_t)e * N;
     for (int k = threadIdx.x; k < N; k += kRedThreads) {
       const size_t p = base + k;
-      const double q = w[p] * mask[p];
-      a += c[p] * d[p] * q;
-      dY[p] = (float)(osc[p] * se * q);
+      const double q = __ldcg(w + p) * __ldcg(mask + p);
+      a += __ldcg(c + p) * __ldcg(d + p) * q;
+      dY[p] = (float)(__ldcg(osc + p) * se * q);
     }
   }
   double v[1] = {a};
@@ -1573,20 +1603,26 @@ extern "C" int ax_mlp_train_energy(ax_poisson *P, ax_mlp *M, const double *r_set
     const double *e = e_set + (size_t)k * n;
     rc = apply_f64(P, q, e, st);
     if (rc) break;
-    mask_dot_kernel<double><<<nb, kRedThreads, 0, st>>>(q, e, P->mask, P->c,
-                                                        part + (size_t)k * nb, n);
+    rc = ax::launch_chained(true, mask_dot_kernel<double>, nb, kRedThreads, 0, st, q, e, P->mask,
+                            P->c, part + (size_t)k * nb, n, (CgScalars *)nullptr);
   }
   pair_sums_kernel<<<K, 32, 0, st>>>(part, eA);
   for (int ep = 0; ep < epochs && rc == AX_OK; ++ep) {
     for (int k = 0; k < K && rc == AX_OK; ++k) {
       const double *r = r_set + (size_t)k * n, *e = e_set + (size_t)k * n;
-      energy_features_kernel<<<P->nelv, kRedThreads, 0, st>>>(M->X, s, r, isc, N);
+      if ((rc = ax::launch_chained(true, energy_features_kernel, P->nelv, kRedThreads, 0, st, M->X, s,
+                                   r, isc, N)))
+        break;
       if ((rc = ax::mlp_train_forward_corr(M, P->nelv, corr, osc, s, st))) break;
       if ((rc = ax_gs_sum(P->gs, corr, st))) break;
-      energy_diff_kernel<<<nb, kRedThreads, 0, st>>>(d, e, r, P->minv, corr, n);
+      if ((rc = ax::launch_chained(true, energy_diff_kernel, nb, kRedThreads, 0, st, d, e, r, P->minv,
+                                   corr, n)))
+        break;
       if ((rc = apply_f64(P, q, d, st))) break;
-      energy_dot_dy_kernel<<<nb, kRedThreads, 0, st>>>(M->dY, q, d, P->mask, P->c, osc, s,
-                                                       eA + k, N, P->nelv, part + (size_t)k * nb);
+      if ((rc = ax::launch_chained(true, energy_dot_dy_kernel, nb, kRedThreads, 0, st, M->dY, q, d,
+                                   P->mask, P->c, osc, s, eA + k, N, P->nelv,
+                                   part + (size_t)k * nb)))
+        break;
       if ((rc = ax::mlp_train_backward(M, P->nelv, st))) break;
       if ((rc = ax::mlp_adam_step(M, lr, st))) break;
     }

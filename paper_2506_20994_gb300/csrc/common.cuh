@@ -35,13 +35,14 @@ inline bool all_nonnull(P... p) {
   return ok;
 }
 
-// Storage -> compute conversion of one element-field value.
+// Storage -> compute conversion of one element-field value (read past L1: the
+// kernels are launched chained, see grid_wait).
 template <typename T>
-AX_D T ld_cvt(const double *p) { return (T)__ldg(p); }
+AX_D T ld_cvt(const double *p) { return (T)__ldcg(p); }
 template <typename T>
-AX_D T ld_cvt(const float *p) { return (T)__ldg(p); }
+AX_D T ld_cvt(const float *p) { return (T)__ldcg(p); }
 template <typename T>
-AX_D T ld_cvt(const __nv_bfloat16 *p) { return (T)__bfloat162float(__ldg(p)); }
+AX_D T ld_cvt(const __nv_bfloat16 *p) { return (T)__bfloat162float(__ldcg(p)); }
 
 // Raises a kernel's dynamic shared-memory limit to `bytes` on the current
 // device when that is above the 48 KB default and above what this kernel was
@@ -94,13 +95,13 @@ inline bool grant_smem(K kernel, size_t bytes, std::atomic<size_t> (&granted)[kM
 AX_D void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 AX_D void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
-inline int launch_chained(bool chained, void (*kern)(P...), unsigned grid, unsigned block, size_t smem,
+inline int launch_chained(bool chained, void (*kern)(P...), dim3 grid, unsigned block, size_t smem,
                           cudaStream_t st, A &&...args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;

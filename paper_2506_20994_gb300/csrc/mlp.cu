@@ -298,6 +298,8 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
   const long long e0 = (long long)blockIdx.x * 16;
   const int nel = (int)min(16ll, (long long)nelv - e0);
 
+  ax::grid_wait();
+  ax::grid_go();
   // the scaled rows, warp w rows w, w + 4, ... (N even: pairs stay in a row)
   for (int row = wp; row < 16; row += kSymWarps) {
     const size_t base = (size_t)(e0 + (row < nel ? row : 0)) * N;
@@ -305,8 +307,8 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
     for (int k = 2 * lane; k < NP; k += 64) {
       uint32_t x = 0u;
       if (row < nel && k < N) {
-        const V rv = *reinterpret_cast<const V *>(r + base + k);
-        const float2 sv = *reinterpret_cast<const float2 *>(sc + base + k);
+        const V rv = __ldcg(reinterpret_cast<const V *>(r + base + k));
+        const float2 sv = __ldcg(reinterpret_cast<const float2 *>(sc + base + k));
         x = pack_bf16(sv.x * to_f32(rv.x), sv.y * to_f32(rv.y));
       }
       *reinterpret_cast<uint32_t *>(xs + row * XS + k) = x;
@@ -366,8 +368,8 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
     const int col = nt * 8 + 2 * t4;
     const bool in = col < N;
     const float2 zero = make_float2(0.f, 0.f);
-    const float2 s0 = in && ok0 ? *reinterpret_cast<const float2 *>(sc + row0 + col) : zero;
-    const float2 s1 = in && ok1 ? *reinterpret_cast<const float2 *>(sc + row1 + col) : zero;
+    const float2 s0 = in && ok0 ? __ldcg(reinterpret_cast<const float2 *>(sc + row0 + col)) : zero;
+    const float2 s1 = in && ok1 ? __ldcg(reinterpret_cast<const float2 *>(sc + row1 + col)) : zero;
     float acc2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int q = 0; q < NT1 / 2; ++q) {
@@ -397,9 +399,10 @@ int sym_apply(T *corr, const T *r, const float *sc, const __nv_bfloat16 *w1,
   const size_t smem = sym_smem<NT1>(NP);
   static std::atomic<size_t> granted[ax::kMaxDevices];
   if (!ax::grant_smem(kern, smem, granted)) return AX_EINVAL;
-  kern<<<(unsigned)((nelv + 15) / 16), kSymWarps * 32, smem, st>>>(corr, r, sc, w1, w2, N, NP,
-                                                                  nelv);
-  return ax::launch_status();
+  // not chained: the few blocks of a small mesh would crowd onto the SMs that
+  // the kernel in front leaves first
+  return ax::launch_chained(false, kern, (unsigned)((nelv + 15) / 16), kSymWarps * 32, smem, st, corr,
+                            r, sc, w1, w2, N, NP, nelv);
 }
 
 // ---------------------------------------------------------------- training
@@ -479,7 +482,7 @@ skinny_kernel(const float *__restrict__ A, const float *__restrict__ B,
       const int r = AT ? v % kRows : v / kChunk, k = AT ? v / kRows : v % kChunk;
       const int m = m0 + r;
       ra[q] = k >= kn ? 0.f
-              : m < Mr ? __ldg(AT ? a + (size_t)(k0 + k) * lda + m : a + (size_t)m * lda + k0 + k)
+              : m < Mr ? __ldcg(AT ? a + (size_t)(k0 + k) * lda + m : a + (size_t)m * lda + k0 + k)
               : ONES && m == Mr ? 1.f : 0.f;
     }
     const int nv = kn * Hd;
@@ -488,7 +491,7 @@ skinny_kernel(const float *__restrict__ A, const float *__restrict__ B,
       for (int q = 0; q < 4 * NB; ++q) {  // value (row v / kChunk of B, k = v % kChunk)
         const int v = tid + q * kThreads, hh = v / kChunk, k = v % kChunk;
         reinterpret_cast<float *>(rb)[q] =
-            hh < Hd && k < kn ? __ldg(b + (size_t)hh * ldb + k0 + k) : 0.f;
+            hh < Hd && k < kn ? __ldcg(b + (size_t)hh * ldb + k0 + k) : 0.f;
       }
     } else {
       const float *src = b + (size_t)k0 * Hd;
@@ -497,16 +500,18 @@ skinny_kernel(const float *__restrict__ A, const float *__restrict__ B,
         const int v = 4 * (tid + q * kThreads);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (v + 3 < nv) {
-          x = __ldg(reinterpret_cast<const float4 *>(src + v));
+          x = __ldcg(reinterpret_cast<const float4 *>(src + v));
         } else {
-          if (v < nv) x.x = __ldg(src + v);
-          if (v + 1 < nv) x.y = __ldg(src + v + 1);
-          if (v + 2 < nv) x.z = __ldg(src + v + 2);
+          if (v < nv) x.x = __ldcg(src + v);
+          if (v + 1 < nv) x.y = __ldcg(src + v + 1);
+          if (v + 2 < nv) x.z = __ldcg(src + v + 2);
         }
         rb[q] = x;
       }
     }
   };
+  ax::grid_wait();
+  ax::grid_go();
   load(0);
   for (int step = 0; step < steps; ++step) {
     if (step) __syncthreads();
@@ -569,7 +574,7 @@ struct EpiHidden {
   const float *b1;
   int Hd, sym;
   AX_D void operator()(int b, int h, float a) const {
-    const float v = a + b1[h];
+    const float v = a + __ldcg(b1 + h);
     H[(size_t)b * Hd + h] = sym ? v : tanhf(v);
   }
 };
@@ -580,7 +585,7 @@ struct EpiBack {
   int Hd, sym;
   AX_D void operator()(int b, int h, float a) const {
     const size_t q = (size_t)b * Hd + h;
-    const float hv = H[q];
+    const float hv = __ldcg(H + q);
     dP[q] = sym ? a : a * (1.f - hv * hv);
   }
 };
@@ -607,26 +612,28 @@ template <class Fin>
 AX_D void out_rows(const float *__restrict__ H, const float *__restrict__ theta, int B, int N,
                    int Hd, Fin fin) {
   __shared__ float4 Hs[64];
+  ax::grid_wait();
+  ax::grid_go();
   const int b0 = blockIdx.x * kRows, o = blockIdx.y * kThreads + threadIdx.x;
   const float *W2 = theta + (size_t)N * Hd + Hd, *b2 = W2 + (size_t)Hd * N;
   if (threadIdx.x < Hd * kRows) {
     const int r = threadIdx.x / Hd, h = threadIdx.x % Hd;
     reinterpret_cast<float *>(Hs)[h * kRows + r] =
-        b0 + r < B ? H[(size_t)(b0 + r) * Hd + h] : 0.f;
+        b0 + r < B ? __ldcg(H + (size_t)(b0 + r) * Hd + h) : 0.f;
   }
   __syncthreads();
   if (o >= N) return;
   float acc[kRows] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 8
   for (int h = 0; h < Hd; ++h) {
-    const float w = __ldg(W2 + (size_t)h * N + o);
+    const float w = __ldcg(W2 + (size_t)h * N + o);
     const float4 v = Hs[h];
     acc[0] = fmaf(v.x, w, acc[0]);
     acc[1] = fmaf(v.y, w, acc[1]);
     acc[2] = fmaf(v.z, w, acc[2]);
     acc[3] = fmaf(v.w, w, acc[3]);
   }
-  const float bo = b2[o];
+  const float bo = __ldcg(b2 + o);
 #pragma unroll
   for (int r = 0; r < kRows; ++r)
     if (b0 + r < B) fin(b0 + r, o, acc[r] + bo);
@@ -641,7 +648,7 @@ fwd_out_loss_kernel(float *__restrict__ Y, float *__restrict__ dY, const float *
   out_rows(H, theta, B, N, Hd, [&](int b, int o, float y) {
     const size_t q = (size_t)b * N + o;
     Y[q] = y;
-    const float res = y - Tt[q];
+    const float res = y - __ldcg(Tt + q);
     dY[q] = 2.f * res / ((float)B * (float)N);
     l += (double)res * (double)res;
   });
@@ -658,7 +665,7 @@ fwd_out_corr_kernel(double *__restrict__ corr, const float *__restrict__ H,
                     const double *__restrict__ s, int B, int N, int Hd) {
   out_rows(H, theta, B, N, Hd, [&](int b, int o, float y) {
     const size_t q = (size_t)b * N + o;
-    corr[q] = osc[q] * s[b] * (double)y;
+    corr[q] = __ldcg(osc + q) * __ldcg(s + b) * (double)y;
   });
 }
 
@@ -681,13 +688,15 @@ __global__ void adam_sym_kernel(float *__restrict__ theta, float *__restrict__ m
                                 float *__restrict__ v, const float *__restrict__ g, int N, int Hd,
                                 float lr, float b1, float b2, float eps, float c1, float c2) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  ax::grid_wait();  // every thread, also one without a parameter
+  ax::grid_go();
   if (q >= (int64_t)N * Hd) return;
-  const float gq = g[q];
-  const float mq = b1 * m[q] + (1.f - b1) * gq;
-  const float vq = b2 * v[q] + (1.f - b2) * gq * gq;
+  const float gq = __ldcg(g + q);
+  const float mq = b1 * __ldcg(m + q) + (1.f - b1) * gq;
+  const float vq = b2 * __ldcg(v + q) + (1.f - b2) * gq * gq;
   m[q] = mq;
   v[q] = vq;
-  const float t = theta[q] - lr * (mq / c1) / (sqrtf(vq / c2) + eps);
+  const float t = __ldcg(theta + q) - lr * (mq / c1) / (sqrtf(vq / c2) + eps);
   theta[q] = t;
   theta[(size_t)N * Hd + Hd + (size_t)(q % Hd) * N + q / Hd] = t;
 }
@@ -746,7 +755,6 @@ inline unsigned blocks_of(int64_t n) { return (unsigned)((n + kThreads - 1) / kT
 inline dim3 out_grid(int B, int N) {
   return dim3((unsigned)((B + kRows - 1) / kRows), (unsigned)((N + kThreads - 1) / kThreads));
 }
-inline unsigned row_blocks(int M) { return (unsigned)((M + kRows - 1) / kRows); }
 
 int ensure_capacity(ax_mlp *M, int B) {
   if (B <= M->cap) return AX_OK;
@@ -801,50 +809,62 @@ __global__ void sum_partials_kernel2(const double *__restrict__ p, int n, double
   ax::warp_sum_partials<1>(p, n, out);
 }
 
+template <bool AT, bool BT, bool ONES, bool CSUM, class Epi, class Csum>
+int launch_skinny(cudaStream_t st, const float *A, const float *B, const float *A2,
+                  const float *B2, int M, int K, int Hd, int lda, int ldb, Epi epi, Csum csum) {
+  return ax::launch_chained(true, skinny_kernel<AT, BT, ONES, CSUM, Epi, Csum>,
+                            (unsigned)((M + kRows - 1) / kRows), kThreads, 0, st, A, B, A2, B2, M,
+                            K, Hd, lda, ldb, epi, csum);
+}
+
 // H = act(X W1 + b1)
-void launch_hidden(ax_mlp *M, int B, cudaStream_t st) {
+int launch_hidden(ax_mlp *M, int B, cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
-  skinny_kernel<false, false, false, false><<<row_blocks(B), kThreads, 0, st>>>(
-      M->X, M->theta, nullptr, nullptr, B, N, Hd, N, Hd,
-      EpiHidden{M->H, M->theta + (size_t)N * Hd, Hd, M->arch == AX_MLP_SYM}, NoCsum{});
+  const EpiHidden epi{M->H, M->theta + (size_t)N * Hd, Hd, M->arch == AX_MLP_SYM};
+  return launch_skinny<false, false, false, false>(st, M->X, M->theta, nullptr, nullptr, B, N, Hd,
+                                                   N, Hd, epi, NoCsum{});
 }
 
 // Gradient from M->X, M->H, M->dY.  Tanh form: all four blocks.  Symmetric
 // form: the gradient of the free parameters W1 (W2's folded in: both are
 // [N][Hd] sums over the rows, X^T dP + dY^T H); the rest of M->grad is zero
 // from the start and stays so.
-void launch_backward(ax_mlp *M, int B, cudaStream_t st) {
+int launch_backward(ax_mlp *M, int B, cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
-  const float *W2 = M->theta + (size_t)N * Hd + Hd;
+  const float *none = nullptr;
   if (M->arch == AX_MLP_SYM) {
     // W2 = W1^T, so the back product reads W1's coalesced rows
-    skinny_kernel<false, false, false, false><<<row_blocks(B), kThreads, 0, st>>>(
-        M->dY, M->theta, nullptr, nullptr, B, N, Hd, N, Hd, EpiBack{M->dP, M->H, Hd, 1},
-        NoCsum{});
-    skinny_kernel<true, false, false, false><<<row_blocks(N), kThreads, 0, st>>>(
-        M->X, M->dP, M->dY, M->H, N, B, Hd, N, Hd, EpiRows{M->grad, Hd}, NoCsum{});
-    return;
+    if (int rc = launch_skinny<false, false, false, false>(st, M->dY, M->theta, none, none, B, N, Hd,
+                                                           N, Hd, EpiBack{M->dP, M->H, Hd, 1},
+                                                           NoCsum{}))
+      return rc;
+    return launch_skinny<true, false, false, false>(st, M->X, M->dP, M->dY, M->H, N, B, Hd, N, Hd,
+                                                    EpiRows{M->grad, Hd}, NoCsum{});
   }
+  const float *W2 = M->theta + (size_t)N * Hd + Hd;
   float *gW2 = M->grad + (size_t)N * Hd + Hd;
-  skinny_kernel<true, false, false, true><<<row_blocks(N), kThreads, 0, st>>>(
-      M->dY, M->H, nullptr, nullptr, N, B, Hd, N, Hd, EpiCols{gW2, N},
-      CsumBias{gW2 + (size_t)Hd * N});
-  skinny_kernel<false, true, false, false><<<row_blocks(B), kThreads, 0, st>>>(
-      M->dY, W2, nullptr, nullptr, B, N, Hd, N, N, EpiBack{M->dP, M->H, Hd, 0}, NoCsum{});
-  skinny_kernel<true, false, true, false><<<row_blocks(N + 1), kThreads, 0, st>>>(
-      M->X, M->dP, nullptr, nullptr, N + 1, B, Hd, N, Hd, EpiRows{M->grad, Hd}, NoCsum{});
+  int rc = launch_skinny<true, false, false, true>(st, M->dY, M->H, none, none, N, B, Hd, N, Hd,
+                                                   EpiCols{gW2, N},
+                                                   CsumBias{gW2 + (size_t)Hd * N});
+  if (rc == AX_OK)
+    rc = launch_skinny<false, true, false, false>(st, M->dY, W2, none, none, B, N, Hd, N, N,
+                                                  EpiBack{M->dP, M->H, Hd, 0}, NoCsum{});
+  if (rc == AX_OK)
+    rc = launch_skinny<true, false, true, false>(st, M->X, M->dP, none, none, N + 1, B, Hd, N, Hd,
+                                                 EpiRows{M->grad, Hd}, NoCsum{});
+  return rc;
 }
 
 // forward + loss + gradient on M->X / M->T (B samples)
 int loss_grad_dev(ax_mlp *M, int B, cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
-  launch_hidden(M, B, st);
+  if (int rc = launch_hidden(M, B, st)) return rc;
   const dim3 og = out_grid(B, N);
-  fwd_out_loss_kernel<<<og, kThreads, 0, st>>>(M->Y, M->dY, M->H, M->T, M->theta, B, N, Hd,
-                                               M->partials);
+  if (ax::launch_chained(true, fwd_out_loss_kernel, og, kThreads, 0, st, M->Y, M->dY, M->H, M->T,
+                         M->theta, B, N, Hd, M->partials))
+    return AX_ELAUNCH;
   sum_partials_kernel2<<<1, 32, 0, st>>>(M->partials, (int)(og.x * og.y), M->loss_dev);
-  launch_backward(M, B, st);
-  return ax::launch_status();
+  return launch_backward(M, B, st);
 }
 
 // Adam on M->grad (symmetric form: the tied parameters together)
@@ -853,8 +873,9 @@ int adam_dev(ax_mlp *M, float lr, float b1, float b2, float eps, cudaStream_t st
   const float c1 = 1.f - powf(b1, (float)M->adam_step);
   const float c2 = 1.f - powf(b2, (float)M->adam_step);
   if (M->arch == AX_MLP_SYM)
-    adam_sym_kernel<<<blocks_of((int64_t)M->n_in * M->n_hid), kThreads, 0, st>>>(
-        M->theta, M->m, M->v, M->grad, M->n_in, M->n_hid, lr, b1, b2, eps, c1, c2);
+    return ax::launch_chained(true, adam_sym_kernel, blocks_of((int64_t)M->n_in * M->n_hid), kThreads,
+                              0, st, M->theta, M->m, M->v, M->grad, M->n_in, M->n_hid, lr, b1, b2,
+                              eps, c1, c2);
   else
     adam_kernel<<<blocks_of(M->nparam), kThreads, 0, st>>>(M->theta, M->m, M->v, M->grad,
                                                            M->nparam, lr, b1, b2, eps, c1, c2);
@@ -883,16 +904,14 @@ int mlp_reserve(ax_mlp *M, int B, int pairs) {
 int mlp_train_forward_corr(ax_mlp *M, int B, double *corr, const double *osc, const double *s,
                            cudaStream_t st) {
   const int N = M->n_in, Hd = M->n_hid;
-  launch_hidden(M, B, st);
-  fwd_out_corr_kernel<<<out_grid(B, N), kThreads, 0, st>>>(corr, M->H, M->theta, osc, s, B, N,
-                                                           Hd);
-  return launch_status();
+  if (int rc = launch_hidden(M, B, st)) return rc;
+  return launch_chained(true, fwd_out_corr_kernel, out_grid(B, N), kThreads, 0, st, corr, M->H,
+                        M->theta, osc, s, B, N, Hd);
 }
 
 // gradient from M->X, M->H and the output gradient M->dY (B rows)
 int mlp_train_backward(ax_mlp *M, int B, cudaStream_t st) {
-  launch_backward(M, B, st);
-  return launch_status();
+  return launch_backward(M, B, st);
 }
 
 int mlp_adam_step(ax_mlp *M, float lr, cudaStream_t st) {

@@ -115,3 +115,70 @@ def test_solvers_repeat_bitwise():
     for _ in range(4):
         x, n = P.cg(b, tol=1e-9)[:2]
         assert n == n0 and torch.equal(x, x0)
+
+
+@pytest.mark.parametrize("dims,lx", [((1, 1, 1), 8), ((8, 8, 8), 8), ((6, 5, 4), 5),
+                                     ((9, 8, 7), 6), ((5, 4, 3), 7), ((16, 16, 4), 3)])
+def test_reduced_precision_chains(dims, lx):
+    """fp32, bf16 and trilinear applies and the fp32 gather-scatter, at orders
+    of the persistent kernels and of the k-loop ones."""
+    c = operator_case(dims, lx, seed=620 + lx)
+    f, h = torch.float32, torch.bfloat16
+    d, e = _scale(c, f), _scale(c, h)
+    dx, dxt = _t(c["dx"], f), _t(c["dxt"], f)
+    G, Gh = [d[k] for k in GKEYS], [e[k] for k in GKEYS]
+    gs = ax.GatherScatter(ax.box_numbering(*dims, lx))
+    bufs = [d["u"].clone(), torch.zeros_like(d["u"]), torch.zeros_like(d["u"])]
+
+    def step32(w, u, k):
+        ax.ax_helm_f32(w, u, dx, dxt, d["h1"], *G, lx)
+        if k % 3 == 2:
+            gs.sum(w)
+    _same(step32, bufs)
+
+    def step16(w, u, k):
+        ax.ax_helm_bf16(w, u.to(h), dx, dxt, e["h1"], *Gh, lx)
+    _same(step16, bufs)
+    cor = _t(ax.box_corners(c["vertices"])).reshape(-1)
+    xi, wq = (_t(a) for a in ax.gll(lx))
+    _same(lambda w, u, k: ax.ax_helm_trilinear_f32(w, u, dx, dxt, d["h1"], cor, xi, wq, lx), bufs)
+
+
+@pytest.mark.parametrize("lx", [2, 3, 4, 5, 7, 9, 13])
+def test_k_loop_and_six_matrix_chains(lx):
+    c = operator_case((5, 4, 3), lx, seed=640 + lx)
+    d = _scale(c)
+    G = [d[k] for k in GKEYS]
+    bufs = [d["u"].clone(), torch.zeros_like(d["u"]), torch.zeros_like(d["u"])]
+    dx, dxt, dy, dyt = d["dx"], d["dxt"], d["dx"].clone(), d["dxt"].clone()
+
+    def step(w, u, k):
+        if k % 2:
+            ax.ax_helm(w, u, dx, dxt, d["h1"], *G, lx)
+        else:
+            ax.ax_helm_xyz(w, u, dx, dy, dx, dxt, dyt, dxt, d["h1"], *G, lx)
+    _same(step, bufs)
+
+
+def test_mixed_solves_and_training_repeat_bitwise():
+    P = ax.Poisson(synth.box_vertices(7, 6, 5, seed=4), 8, h1=ax.fourier_coefficient(3))
+    P.set_check_every(4)
+    b = P.rhs(synth.poisson_source)
+    M = ax.Mlp(512, 32, arch=ax.AX_MLP_SYM,
+               params=ax.mlp_init_params(512, 32, seed=1, arch=ax.AX_MLP_SYM, scale=1.0))
+    runs = [lambda: P.mpcg(b, mode=ax.AX_PREC_F32, tol=1e-9)[0],
+            lambda: P.mpcg(b, mode=ax.AX_PREC_BF16, tol=1e-9, inner_tol=1e-2)[0],
+            lambda: P.fcg(b, M, tol=1e-9)[0], lambda: P.mpfcg(b, M, tol=1e-9)[0]]
+    for run in runs:
+        x0 = run()
+        assert bool(torch.isfinite(x0).all())
+        for _ in range(3):
+            assert torch.equal(run(), x0)
+    R, E = ax.iterate_pairs(P, b, iterates=(2, 8, 32))
+    got = []
+    for _ in range(3):
+        N = ax.Mlp(512, 32, arch=ax.AX_MLP_SYM,
+                   params=ax.mlp_init_params(512, 32, seed=1, arch=ax.AX_MLP_SYM))
+        ax.train_energy(P, N, R, E, epochs=4)
+        got.append(N.get_params())
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
