@@ -120,7 +120,7 @@ __global__ void cg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restri
                                const T *__restrict__ b, const T *__restrict__ mask,
                                const T *__restrict__ minv, const T *__restrict__ c,
                                CgScalars *__restrict__ s, double *__restrict__ partials,
-                               int64_t n) {
+                               int64_t n, const ax::CgMailTo to) {
   T a_rz = 0, a_rr = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -135,12 +135,13 @@ __global__ void cg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restri
   }
   double v[2] = {(double)a_rz, (double)a_rr};
   ax::block_sum<2>(v);
-  ax::finish_sums<2>(v, partials, &s->ticket, [s](const double *t) {
+  ax::finish_sums<2>(v, partials, &s->ticket, [s, to](const double *t) {
     s->rz = t[0];
     s->rr = t[1];
     s->rr0 = t[1];
     s->beta = 0.0;
     s->status = 0;
+    ax::cg_post(to, s, t[1], 0);
   });
 }
 
@@ -177,7 +178,8 @@ __global__ void __launch_bounds__(kRedThreads, kRedPerSm)
 cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
                                  const T *__restrict__ w, const T *__restrict__ cm,
                                  const T *__restrict__ c, CgScalars *__restrict__ s,
-                                 double *__restrict__ partials, int64_t n) {
+                                 double *__restrict__ partials, int64_t n,
+                                 const ax::CgMailTo to) {
   ax::grid_wait();
   ax::grid_go();
   const T alpha = (T)__ldcg(&s->alpha);
@@ -236,12 +238,14 @@ cg_update_kernel(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
   v[0] = (double)a_rz;
   if constexpr (RR) v[1] = (double)a_rr;
   ax::block_sum<NS>(v);
-  ax::finish_sums<NS>(v, partials, &s->ticket, [s](const double *t) {
+  ax::finish_sums<NS>(v, partials, &s->ticket, [s, to](const double *t) {
     const double rz = __ldcg(&s->rz);
     s->beta = (rz != 0.0) ? t[0] / rz : 0.0;
     s->rz = t[0];
     if constexpr (RR) s->rr = t[1];
-    if (!isfinite(t[0]) || (RR && !isfinite(t[NS - 1]))) s->status = 1;
+    const bool bad = !isfinite(t[0]) || (RR && !isfinite(t[NS - 1]));
+    if (bad) s->status = 1;
+    if constexpr (RR) ax::cg_post(to, s, t[1], bad ? 1 : __ldcg(&s->status));
   });
 }
 
@@ -374,6 +378,8 @@ struct ax_poisson {
   double *partials = nullptr;
   CgScalars *scal = nullptr;
   CgScalars *scal_host = nullptr;  // pinned
+  ax::CgMail *mail = nullptr;      // pinned: the convergence test's values
+  unsigned mail_seq = 0;           // of the last one asked for
   // owned fp32 data of the refinement solve (lazily allocated)
   int lowp_mode = 0;  // 0 none, 1 fp32, 2 bf16 operator data
   float *minv32 = nullptr, *mask32 = nullptr, *x32 = nullptr, *r32 = nullptr, *p32 = nullptr,
@@ -499,6 +505,26 @@ int apply_fused_update(ax_poisson *P, float *w, float *p, const float *r, const 
   return apply_lowp(P, w, p, st, P->dotp, &up, &job);
 }
 
+// Asks the next reduction that forms rr for its values (address and number)
+ax::CgMailTo next_mail(ax_poisson *P) { return ax::CgMailTo{P->mail, ++P->mail_seq}; }
+// Waits for the values last asked for; AX_ELAUNCH if the stream failed or ran
+// dry without them.
+int wait_mail(const ax_poisson *P, cudaStream_t st) {
+  auto here = [P] { return __atomic_load_n(&P->mail->seq, __ATOMIC_ACQUIRE) == P->mail_seq; };
+  for (unsigned spin = 1; !here(); ++spin) {
+    if (spin % 16384) continue;
+    const cudaError_t e = cudaStreamQuery(st);
+    if (e == cudaErrorNotReady) {
+      (void)cudaGetLastError();  // not an error, but it would be taken for one later
+      continue;
+    }
+    if (e == cudaSuccess && here()) break;
+    (void)cudaGetLastError();
+    return AX_ELAUNCH;
+  }
+  return AX_OK;
+}
+
 // Generic PCG loop on vectors of type T (fp64 with the fp64 operator, or
 // fp32 with the low-precision operator).  x0 = 0.  Returns AX_OK when
 // sqrt(rr/rr0) <= tol, AX_ENOTCONV at maxit, AX_EBREAKDOWN on breakdown.
@@ -508,77 +534,73 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
              double *relres, cudaStream_t st) {
   const int64_t n = P->n;
   const unsigned nb = kRedBlocks;
+  if (iters) *iters = 0;
+  if (relres) *relres = 0.0;
   cg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, p, b, mask, minv, c, P->scal, P->partials,
-                                               n);
+                                                n, next_mail(P));
   if (ax::launch_status()) return AX_ELAUNCH;
-  if (cudaMemcpyAsync(P->scal_host, P->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost, st) !=
-          cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return AX_ELAUNCH;
-  const double rr0 = P->scal_host->rr0;
-  int it = 0;
-  double rel = rr0 > 0 ? 1.0 : 0.0;
-  if (rr0 == 0.0 || tol >= 1.0) {
-    if (iters) *iters = 0;
-    if (relres) *relres = 0.0;
-    return AX_OK;
-  }
-  int status = AX_ENOTCONV;
   // fp64 with prepared geometry: p . Ap comes out of the apply itself (for
   // a continuous, masked p the assembled dot equals the element-local sum
   // of p . A_e p), and the mask moves into the update
-  const int nparts = fused_parts(P, (const T *)nullptr);
-  const bool fused = nparts > 0;
+  const bool fused = fused_parts(P, (const T *)nullptr) > 0;
   // after the first iteration the next direction is formed inside the apply,
   // in fp64 together with the x update of the step before
   const bool fused_p = fused && fuses_update(P, (const T *)nullptr);
   const bool fused_x = fused_p && std::is_same_v<T, double>;
-  while (it < maxit) {
-    int rc;
-    if (fused) {
-      rc = (fused_p && it > 0) ? apply_fused_update(P, w, p, r, minv, x, st)
-                               : apply_fused(P, w, p, st);
-      if (rc) return rc;
-      // rr only where the host will test it (after this iteration)
-      const bool checked = (it + 1) % P->check_every == 0 || it + 1 == maxit;
-      auto update = fused_x ? (checked ? cg_update_kernel<T, true, true, !std::is_same_v<T, double>>
-                                       : cg_update_kernel<T, true, false, !std::is_same_v<T, double>>)
+  // The first half of iteration `it`: direction, apply, alpha.  It touches no
+  // result (x only to complete the step before), so it is launched before the
+  // host has tested that step: the GPU goes on while the test's values travel.
+  auto front = [&](int it) -> int {
+    if (fused_p && it > 0) return apply_fused_update(P, w, p, r, minv, x, st);
+    int rc = AX_OK;
+    if (it > 0)
+      rc = ax::launch_chained(true, cg_p_kernel<T>, nb, kRedThreads, 0, st, p, r, minv, P->scal, n);
+    if (rc) return rc;
+    if (fused) return apply_fused(P, w, p, st);
+    if ((rc = apply(w, p, st))) return rc;
+    return ax::launch_chained(true, mask_dot_kernel<T>, nb, kRedThreads, 0, st, w, p, mask, c,
+                              P->partials, n, P->scal);
+  };
+  // The second half: x (unless the next apply does it), r, beta; rr only where
+  // the host will test it.
+  auto back = [&](bool checked) -> int {
+    constexpr bool X64 = std::is_same_v<T, double>;
+    auto update = !fused    ? cg_update_kernel<T>
+                  : fused_x ? (checked ? cg_update_kernel<T, true, true, !X64>
+                                       : cg_update_kernel<T, true, false, !X64>)
                             : (checked ? cg_update_kernel<T, true, true, true>
                                        : cg_update_kernel<T, true, false, true>);
-      if (ax::launch_chained(true, update, nb, kRedThreads, 0, st, x, r, p, w, cm, c, P->scal,
-                             P->partials, n))
-        return AX_ELAUNCH;
-    } else {
-      rc = apply(w, p, st);
-      if (rc) return rc;
-      rc = ax::launch_chained(true, mask_dot_kernel<T>, nb, kRedThreads, 0, st, w, p, mask, c,
-                              P->partials, n, P->scal) |
-           ax::launch_chained(true, cg_update_kernel<T>, nb, kRedThreads, 0, st, x, r, p, w, cm, c,
-                              P->scal, P->partials, n);
-      if (rc) return AX_ELAUNCH;
-    }
-    ++it;
-    if (it % P->check_every == 0 || it == maxit) {
-      if (cudaMemcpyAsync(P->scal_host, P->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost,
-                          st) != cudaSuccess ||
-          cudaStreamSynchronize(st) != cudaSuccess)
-        return AX_ELAUNCH;
-      if (P->scal_host->status) {
-        status = AX_EBREAKDOWN;
-        break;
-      }
-      rel = std::sqrt(std::max(P->scal_host->rr, 0.0) / rr0);
-      if (rel <= tol) {
-        status = AX_OK;
-        break;
-      }
-    }
-    if (!fused_p && ax::launch_chained(true, cg_p_kernel<T>, nb, kRedThreads, 0, st, p, r, minv,
-                                       P->scal, n))
-      return AX_ELAUNCH;
+    return ax::launch_chained(true, update, nb, kRedThreads, 0, st, x, r, p, w, cm, c, P->scal,
+                              P->partials, n, checked ? next_mail(P) : ax::CgMailTo{});
+  };
+  int rc = maxit > 0 ? front(0) : AX_OK;
+  if (rc == AX_OK) rc = wait_mail(P, st);
+  if (rc) return rc;
+  const double rr0 = P->mail->rr;
+  int it = 0, status = AX_ENOTCONV;
+  double rel = rr0 > 0 ? 1.0 : 0.0;
+  if (rr0 == 0.0 || tol >= 1.0) {
+    status = AX_OK;
+    rel = 0.0;
   }
-  if constexpr (std::is_same_v<T, double>)
-    if (fused_x && it > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
+  while (status == AX_ENOTCONV && it < maxit) {
+    const bool checked = (it + 1) % P->check_every == 0 || it + 1 == maxit;
+    if ((rc = back(checked))) return rc;
+    ++it;
+    if (it < maxit) {
+      if ((rc = front(it))) return rc;
+    } else if constexpr (std::is_same_v<T, double>) {
+      if (fused_x) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
+    }
+    if (!checked) continue;
+    if ((rc = wait_mail(P, st))) return rc;
+    if (P->mail->status) {
+      status = AX_EBREAKDOWN;
+      break;
+    }
+    rel = std::sqrt(std::max(P->mail->rr, 0.0) / rr0);
+    if (rel <= tol) status = AX_OK;
+  }
   if (ax::launch_status()) return AX_ELAUNCH;
   if (iters) *iters = it;
   if (relres) *relres = rel;
@@ -660,6 +682,7 @@ int ax_poisson_destroy(ax_poisson *P) {
   cudaFree(P->hb32);
   cudaFree(P->scal);
   if (P->scal_host) cudaFreeHost(P->scal_host);
+  if (P->mail) cudaFreeHost(P->mail);
   delete P;
   return AX_OK;
 }
@@ -706,8 +729,10 @@ int ax_poisson_create(ax_poisson **out, int lx, int nelv, const double *dx, cons
   int rc = alloc(&P->minv, n) | alloc(&P->cm, n) | alloc(&P->w, n) | alloc(&P->r, n) |
            alloc(&P->p, n) | alloc(&P->partials, 4 * (size_t)kRedBlocks) |
            alloc(&P->scal, 1);
-  if (rc == AX_OK && cudaMallocHost((void **)&P->scal_host, sizeof(CgScalars)) != cudaSuccess)
+  if (rc == AX_OK && (cudaMallocHost((void **)&P->scal_host, sizeof(CgScalars)) != cudaSuccess ||
+                      cudaMallocHost((void **)&P->mail, sizeof(ax::CgMail)) != cudaSuccess))
     rc = AX_ENOMEM;
+  if (rc == AX_OK) *P->mail = ax::CgMail{};
   if (rc) {
     ax_poisson_destroy(P);
     return AX_ENOMEM;
@@ -803,8 +828,14 @@ int ax_cg_solve(ax_poisson *P, double *x, const double *b, double tol, int maxit
   if (!P || !x || !b || maxit < 0 || !(tol >= 0)) return AX_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   auto A = [P](double *w, const double *u, cudaStream_t s) { return apply_f64(P, w, u, s); };
-  return pcg_loop<double>(P, x, b, P->r, P->p, P->w, P->mask, P->minv, P->c, P->cm, A, tol,
-                          maxit, iters, relres, st);
+  const int rc = pcg_loop<double>(P, x, b, P->r, P->p, P->w, P->mask, P->minv, P->c, P->cm, A, tol,
+                                  maxit, iters, relres, st);
+  // x is complete (its last update may still be on its way)
+  if (cudaStreamSynchronize(st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return AX_ELAUNCH;
+  }
+  return rc;
 }
 
 int ax_mpcg_solve(ax_poisson *P, int mode, double *x, const double *b, double tol,
@@ -1024,7 +1055,8 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
                                   const T *__restrict__ p, const T *__restrict__ w,
                                   const T *__restrict__ c, const T *__restrict__ cm,
                                   CgScalars *__restrict__ s,
-                                  double *__restrict__ partials, int64_t n) {
+                                  double *__restrict__ partials, int64_t n,
+                                  const ax::CgMailTo to) {
   ax::grid_wait();
   ax::grid_go();
   const T alpha = (T)__ldcg(&s->alpha);
@@ -1080,7 +1112,10 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
   if constexpr (RR) {
     double v[1] = {(double)a_rr};
     ax::block_sum<1>(v);
-    ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) { s->rr = t[0]; });
+    ax::finish_sums<1>(v, partials, &s->ticket, [s, to](const double *t) {
+      s->rr = t[0];
+      ax::cg_post(to, s, t[0], __ldcg(&s->status));
+    });
   }
 }
 
@@ -1197,7 +1232,8 @@ template <typename T>
 __global__ void fcg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
                                 const T *__restrict__ b, const T *__restrict__ mask,
                                 const T *__restrict__ c, CgScalars *__restrict__ s,
-                                double *__restrict__ partials, int64_t n) {
+                                double *__restrict__ partials, int64_t n,
+                                const ax::CgMailTo to) {
   T a = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -1209,12 +1245,13 @@ __global__ void fcg_init_kernel(T *__restrict__ x, T *__restrict__ r, T *__restr
   }
   double v[1] = {(double)a};
   ax::block_sum<1>(v);
-  ax::finish_sums<1>(v, partials, &s->ticket, [s](const double *t) {
+  ax::finish_sums<1>(v, partials, &s->ticket, [s, to](const double *t) {
     s->rr = t[0];
     s->rr0 = t[0];
     s->status = 0;
     s->fallbacks = 0;
     s->use_corr = 0;
+    ax::cg_post(to, s, t[0], 0);
   });
 }
 
@@ -1264,11 +1301,12 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
       return AX_ELAUNCH;
     return AX_OK;
   };
-  fcg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, r_old, b, mask, c, P->scal, P->partials, n);
+  fcg_init_kernel<T><<<nb, kRedThreads, 0, st>>>(x, r, r_old, b, mask, c, P->scal, P->partials, n,
+                                                 next_mail(P));
   int rc = precondition(1);
   if (rc) return rc;
-  if ((rc = read_scalars())) return rc;
-  const double rr0 = P->scal_host->rr0;
+  if ((rc = wait_mail(P, st))) return rc;
+  const double rr0 = P->mail->rr;
   double rel = rr0 > 0 ? 1.0 : 0.0;
   int it = 0, status = AX_ENOTCONV;
   if (rr0 == 0.0 || tol >= 1.0) status = AX_OK;
@@ -1292,37 +1330,41 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
                             : (fused_p ? fcg_update_kernel<T, true, false, !std::is_same_v<T, double>>
                                        : fcg_update_kernel<T, true, false, true>);
       if (ax::launch_chained(true, update, nb, kRedThreads, 0, st, x, r, r_old, p, w, c, cm, P->scal,
-                             P->partials, n))
+                             P->partials, n, checked ? next_mail(P) : ax::CgMailTo{}))
         return AX_ELAUNCH;
     } else {
       if ((rc = apply(w, p, st))) return rc;
       rc = ax::launch_chained(true, mask_dot_kernel<T>, nb, kRedThreads, 0, st, w, p, mask, c,
                               P->partials, n, P->scal) |
            ax::launch_chained(true, fcg_update_kernel<T>, nb, kRedThreads, 0, st, x, r, r_old, p, w,
-                              c, cm, P->scal, P->partials, n);
+                              c, cm, P->scal, P->partials, n,
+                              checked ? next_mail(P) : ax::CgMailTo{});
       if (rc) return AX_ELAUNCH;
     }
     ++it;
-    if (it % P->check_every == 0 || it == maxit) {
-      if ((rc = read_scalars())) return rc;
-      if (P->scal_host->status) {
+    // the next step's preconditioner touches no result: it runs while the
+    // host waits for this step's test
+    if (it < maxit && (rc = precondition(0))) return rc;
+    if (checked) {
+      if ((rc = wait_mail(P, st))) return rc;
+      if (P->mail->status) {
         status = AX_EBREAKDOWN;
         break;
       }
-      rel = std::sqrt(std::max(P->scal_host->rr, 0.0) / rr0);
+      rel = std::sqrt(std::max(P->mail->rr, 0.0) / rr0);
       if (rel <= tol) {
         status = AX_OK;
         break;
       }
     }
-    if ((rc = precondition(0))) return rc;
   }
   if constexpr (std::is_same_v<T, double>)
     if (fused_p && applied > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
   if ((rc = read_scalars())) return rc;
   if (iters) *iters = it;
   if (relres) *relres = rel;
-  if (fallbacks) *fallbacks = P->scal_host->fallbacks;
+  // of the steps taken: the preconditioner may have run once more
+  if (fallbacks) *fallbacks = it > 0 ? P->mail->fallbacks : P->scal_host->fallbacks;
   return status;
 }
 

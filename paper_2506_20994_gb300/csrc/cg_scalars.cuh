@@ -14,6 +14,29 @@ struct CgScalars {
   unsigned ticket;  // blocks done of the reduction in flight (finish_sums)
 };
 
+// What the host tests for convergence, in pinned host memory: the reduction
+// that forms rr writes it there itself, seq last, and the host polls seq.  (A
+// copy of the scalars and a stream synchronisation cost some 15 us per test,
+// through which the GPU stood idle.)
+struct CgMail {
+  double rr;
+  int status, fallbacks;
+  unsigned seq;
+};
+struct CgMailTo {
+  CgMail *mail = nullptr;  // null: none
+  unsigned seq = 0;
+};
+AX_D void cg_post(const CgMailTo &to, const CgScalars *s, double rr, int status) {
+  if (!to.mail) return;
+  volatile CgMail *m = to.mail;
+  m->rr = rr;
+  m->status = status;
+  m->fallbacks = __ldcg(&s->fallbacks);
+  __threadfence_system();
+  m->seq = to.seq;
+}
+
 // alpha = rz / <p, Ap>
 AX_D void cg_set_alpha(CgScalars *s, double pap) {
   const double rz = __ldcg(&s->rz);
