@@ -84,9 +84,8 @@ struct Cfg {
   static_assert(UBYTES % 16 == 0 && GFBYTES % 16 == 0, "bulk copies need 16-byte runs");
 };
 
-// At lx = 8 each thread keeps its coefficient rows of both matrices in
-// registers (48 words) instead of reading them from shared memory in every
-// contraction.
+// The single-mesh kernels keep each thread's coefficient rows of both matrices
+// in registers (48 words at lx = 8) where they fit.
 constexpr bool kE32CoefRegs = true;
 
 // Resident CTAs per SM the launch bounds ask for.
@@ -146,8 +145,10 @@ struct SeqOne {
 // sync() / sync_and(p) its barriers.  DOT: adds this thread's share of
 // u . w to dsum (fp32 per element, fp64 across elements).  err: set to 1 if
 // a staged copy never arrived (the body then stops).
-// CREG (lx = 8 only): coefficient rows in registers (same arithmetic, so
-// the same bits, as reading them from shared memory).
+// CREG (lx 6, 8, 10): coefficient rows in registers (same arithmetic, so the
+// same bits, as reading them from shared memory, a third of the line reads'
+// traffic: fp32 at lx 6 60.8 -> 55.1 us, lx 10 65.1 -> 60.7 us at 5.8 M
+// points; lx 12 spills and slows, 64.5 -> 73.7).
 template <int LX, class SU, class SG, bool DOT, bool PUPD, bool CREG, class Seq, class Sync,
           class SyncAnd>
 AX_D void e32_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd sync_and,
@@ -155,7 +156,7 @@ AX_D void e32_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   static_assert(!PUPD || std::is_same_v<SU, float>, "the fused update keeps fp32 vectors");
   using C = Cfg<LX, SU, SG, PUPD>;
   constexpr int H = C::H, N = C::N, H2 = C::H2, NT = C::NT, N3 = C::N3;
-  constexpr bool kCoefRegs = CREG && LX == 8;
+  constexpr bool kCoefRegs = CREG && LX <= 10;
   u64 *cf = reinterpret_cast<u64 *>(sm);
   u64 *Lb = reinterpret_cast<u64 *>(sm + C::OFF_LINES);
   unsigned char *stg = sm + C::OFF_STAGE;
@@ -208,14 +209,24 @@ AX_D void e32_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   // the same with the coefficient row held in registers
   auto chain2r = [&](const u64 *ln, int L0, int L1, const u64 (&cr)[H], u64 &a0, u64 &a1)
                      __attribute__((always_inline)) {
+    if constexpr (C::VEC) {
 #pragma unroll
-    for (int q = 0; q < H / 2; ++q) {
-      const ulonglong2 l0 = *reinterpret_cast<const ulonglong2 *>(ln + lpos<LX>(L0, 2 * q));
-      const ulonglong2 l1 = *reinterpret_cast<const ulonglong2 *>(ln + lpos<LX>(L1, 2 * q));
-      a0 = q == 0 ? mul2(cr[2 * q], l0.x) : fma2(cr[2 * q], l0.x, a0);
-      a1 = q == 0 ? mul2(cr[2 * q], l1.x) : fma2(cr[2 * q], l1.x, a1);
-      a0 = fma2(cr[2 * q + 1], l0.y, a0);
-      a1 = fma2(cr[2 * q + 1], l1.y, a1);
+      for (int q = 0; q < H / 2; ++q) {
+        const ulonglong2 l0 = *reinterpret_cast<const ulonglong2 *>(ln + lpos<LX>(L0, 2 * q));
+        const ulonglong2 l1 = *reinterpret_cast<const ulonglong2 *>(ln + lpos<LX>(L1, 2 * q));
+        a0 = q == 0 ? mul2(cr[2 * q], l0.x) : fma2(cr[2 * q], l0.x, a0);
+        a1 = q == 0 ? mul2(cr[2 * q], l1.x) : fma2(cr[2 * q], l1.x, a1);
+        a0 = fma2(cr[2 * q + 1], l0.y, a0);
+        a1 = fma2(cr[2 * q + 1], l1.y, a1);
+      }
+    } else {
+      a0 = mul2(cr[0], ln[lpos<LX>(L0, 0)]);
+      a1 = mul2(cr[0], ln[lpos<LX>(L1, 0)]);
+#pragma unroll
+      for (int l = 1; l < H; ++l) {
+        a0 = fma2(cr[l], ln[lpos<LX>(L0, l)], a0);
+        a1 = fma2(cr[l], ln[lpos<LX>(L1, l)], a1);
+      }
     }
   };
   // y at rows (row, N - row) of lines L0 and L1; cof: one matrix's
@@ -600,6 +611,10 @@ int launch(float *w, const SU *u, const float *dx, const float *dxt, const SG *c
   m.dx = dx;
   m.dxt = dxt;
   const E32Upd none{};
+  // Without partials the launch takes this variant's own grid (the common one
+  // is that of the fused update's larger stage): a chained launch has to fill
+  // every SM, see dispatch of the warp-per-element kernel.
+  const int full = (int)std::min<long long>(grid<LX, SU, SG, false, false>(), nelv);
   if (up) {
     if constexpr (std::is_same_v<SU, float>) {
       if (!dotp || !up->pw || !up->r || !up->minv || !up->beta) return AX_EINVAL;
@@ -615,7 +630,7 @@ int launch(float *w, const SU *u, const float *dx, const float *dxt, const SG *c
                           dotp, none);
   }
   using C = Cfg<LX, SU, SG>;
-  return launch_chained(true, ax_eo32_kernel<LX, SU, SG, false>, nb, C::NTB, C::SMEM, st, m, nelv, err,
+  return launch_chained(true, ax_eo32_kernel<LX, SU, SG, false>, full, C::NTB, C::SMEM, st, m, nelv, err,
                         dotp, none);
 }
 

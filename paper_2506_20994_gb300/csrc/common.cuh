@@ -123,6 +123,30 @@ AX_D void prefetch_l2(const void *p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// The whole 16-byte granules inside f[first, first + count) towards L2 (at odd
+// lx an element's run is not made of them, a block's almost is).
+template <typename S>
+AX_D void prefetch_span(const S *f, long long first, long long count) {
+  const uintptr_t a = (reinterpret_cast<uintptr_t>(f + first) + 15u) & ~(uintptr_t)15u;
+  const uintptr_t b = reinterpret_cast<uintptr_t>(f + first + count) & ~(uintptr_t)15u;
+  if (b > a) prefetch_l2(reinterpret_cast<const void *>(a), (unsigned)(b - a));
+}
+// Thread t < 8 of a block: field t (u, then the geometry) of the elements
+// [e0, e0 + nel).
+template <typename SU, typename S>
+AX_D void prefetch_elements(const SU *u, const S *h1, const S *g11, const S *g22, const S *g33,
+                            const S *g12, const S *g13, const S *g23, long long e0, long long nel,
+                            int n3) {
+  const int t = threadIdx.x;
+  if (t >= 8 || nel <= 0) return;
+  if (t == 0) {
+    prefetch_span(u, e0 * n3, nel * n3);
+    return;
+  }
+  const S *f = t == 1 ? g11 : t == 2 ? g22 : t == 3 ? g33 : t == 4 ? g12 : t == 5 ? g13
+             : t == 6 ? g23 : h1;
+  prefetch_span(f, e0 * n3, nel * n3);
+}
 // Explicitly rounded arithmetic (never contracted by the compiler).
 AX_D double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 AX_D float mul_rn(float a, float b) { return __fmul_rn(a, b); }
