@@ -196,8 +196,12 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
   }
 }
 
+// Blocks per SM the launch bounds ask for: the low orders gain from more warps
+// (64 or 80 registers; lx 4 132 -> 127 us, lx 5 159 -> 147, lx 7 181 -> 170 at
+// 5.8 M points), lx 3 and lx >= 8 do not.
+constexpr int df64_minb(int lx) { return lx == 3 || lx == 4 ? 4 : lx >= 5 && lx <= 7 ? 3 : 0; }
 template <int LX>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, df64_minb(LX))
 ax_df64_kernel(double *__restrict__ w, const double *__restrict__ u,
                const double *__restrict__ dx, const double *__restrict__ dxt,
                const double *__restrict__ h1, const double *__restrict__ g11,

@@ -43,7 +43,7 @@ constexpr size_t tri_smem(int epb) {
 }
 
 template <int LX, bool H1>
-__global__ void __launch_bounds__(256, LX <= 8 ? 4 : LX <= 12 ? 3 : 2)
+__global__ void __launch_bounds__(256, LX <= 4 ? 5 : LX <= 8 ? 4 : LX <= 12 ? 3 : 2)
 ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
                   const float *__restrict__ dx, const float *__restrict__ dxt,
                   const float *__restrict__ h1, const double *__restrict__ corners,
@@ -114,8 +114,12 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
     cf[t] = 0.5f * (float)(__ldcg(x + c1 * 3 + d) - __ldcg(x + c0 * 3 + d));
   }
 
-  float uk[LX];
+  float uk[LX], hk[H1 ? LX : 1];  // the columns of u and h1
   if (own) {
+    if constexpr (H1) {
+#pragma unroll
+      for (int k = 0; k < LX; ++k) hk[k] = active ? __ldcg(h1 + base + (size_t)k * N2) : 0.f;
+    }
 #pragma unroll
     for (int k = 0; k < LX; ++k) {
       uk[k] = active ? __ldcg(u + base + (size_t)k * N2) : 0.f;
@@ -195,16 +199,15 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
         const float A22 = __fmaf_rn(a, f, -b * d);
         const float det = __fmaf_rn(a, A00, __fmaf_rn(b, A10, c * A20));
         float s = __fdividef(wij * swq[k], det);  // fp32 operator: ~2 ulp is ample
-        if (H1) s *= __ldcg(h1 + base + (size_t)k * N2);
-        const float g11 = s * __fmaf_rn(A00, A00, __fmaf_rn(A01, A01, A02 * A02));
-        const float g22 = s * __fmaf_rn(A10, A10, __fmaf_rn(A11, A11, A12 * A12));
-        const float g33 = s * __fmaf_rn(A20, A20, __fmaf_rn(A21, A21, A22 * A22));
-        const float g12 = s * __fmaf_rn(A00, A10, __fmaf_rn(A01, A11, A02 * A12));
-        const float g13 = s * __fmaf_rn(A00, A20, __fmaf_rn(A01, A21, A02 * A22));
-        const float g23 = s * __fmaf_rn(A10, A20, __fmaf_rn(A11, A21, A12 * A22));
-        wr = __fmaf_rn(g11, ur, __fmaf_rn(g12, us, g13 * ut));
-        ws = __fmaf_rn(g12, ur, __fmaf_rn(g22, us, g23 * ut));
-        wt = __fmaf_rn(g13, ur, __fmaf_rn(g23, us, g33 * ut));
+        if constexpr (H1) s *= hk[k];
+        // w = s A (A^T grad), A^T grad = sum of the rows times ur, us, ut: 21
+        // operations where the six factors of G and their product take 33
+        const float tx = __fmaf_rn(A00, ur, __fmaf_rn(A10, us, A20 * ut));
+        const float ty = __fmaf_rn(A01, ur, __fmaf_rn(A11, us, A21 * ut));
+        const float tz = __fmaf_rn(A02, ur, __fmaf_rn(A12, us, A22 * ut));
+        wr = s * __fmaf_rn(A00, tx, __fmaf_rn(A01, ty, A02 * tz));
+        ws = s * __fmaf_rn(A10, tx, __fmaf_rn(A11, ty, A12 * tz));
+        wt = s * __fmaf_rn(A20, tx, __fmaf_rn(A21, ty, A22 * tz));
       }
       swr[k * N2 + p] = wr;
       sws[k * N2 + p] = ws;
