@@ -465,16 +465,18 @@ int mass_fused(ax_poisson *P, double *w, const double *u, cudaStream_t st) {
   return P->hb ? ax::mass_add<double>(w, P->hb, u, P->n, P->dotp + P->ndot, st) : AX_OK;
 }
 template <typename T>
-ax::AlphaJob alpha_job(const ax_poisson *P) {
-  return ax::AlphaJob{P->dotp, fused_parts(P, (const T *)nullptr), P->scal};
+ax::AlphaJob alpha_job(const ax_poisson *P, bool chained) {
+  return ax::AlphaJob{P->dotp, fused_parts(P, (const T *)nullptr), P->scal, chained};
 }
-int apply_fused(ax_poisson *P, double *w, const double *u, cudaStream_t st) {
+int apply_fused(ax_poisson *P, double *w, const double *u, cudaStream_t st,
+                bool chained = true) {
   int rc = ax::op_apply_dot(P->op, w, u, P->dotp, st);
   if (rc == AX_OK) rc = mass_fused(P, w, u, st);
-  return rc ? rc : ax::gs_sum_alpha(P->gs, w, alpha_job<double>(P), st);
+  return rc ? rc : ax::gs_sum_alpha(P->gs, w, alpha_job<double>(P, chained), st);
 }
-int apply_fused(ax_poisson *P, float *w, const float *u, cudaStream_t st) {
-  const ax::AlphaJob job = alpha_job<float>(P);
+int apply_fused(ax_poisson *P, float *w, const float *u, cudaStream_t st,
+                bool chained = true) {
+  const ax::AlphaJob job = alpha_job<float>(P, chained);
   return apply_lowp(P, w, u, st, P->dotp, nullptr, &job);
 }
 // The direction update p = minv r + beta p folded into the apply that reads
@@ -484,24 +486,25 @@ bool fuses_update(const ax_poisson *P, const float *) { return P->dotp && P->low
 // fp64: the previous step's x += alpha p as well, from the old p it reads
 int apply_fused_update(ax_poisson *P, double *w, double *p, const double *r,
                        const double *minv, double *x, cudaStream_t st,
-                       const double *corr = nullptr) {
+                       const double *corr = nullptr, bool chained = true) {
   const ax::OpUpdate up{p, r, minv, corr, x, &P->scal->alpha, &P->scal->beta,
                         corr ? &P->scal->use_corr : nullptr};
   int rc = ax::op_update_apply_dot(P->op, w, up, P->dotp, st);
   if (rc == AX_OK) rc = mass_fused(P, w, p, st);
-  return rc ? rc : ax::gs_sum_alpha(P->gs, w, alpha_job<double>(P), st);
+  return rc ? rc : ax::gs_sum_alpha(P->gs, w, alpha_job<double>(P, chained), st);
 }
 // fp32 vectors (the refinement's inner CG, even-odd fp32 kernel): the same
 // fusion without x, p = minv .* r + beta p in fp32 inside the apply
 int apply_fused_update(ax_poisson *P, float *w, float *p, const float *r, const float *minv,
-                       float *, cudaStream_t st, const float *corr = nullptr) {
+                       float *, cudaStream_t st, const float *corr = nullptr,
+                       bool chained = true) {
   if (corr) return AX_EINVAL;  // the flexible loop keeps its own direction kernel
   ax::E32Upd up;
   up.pw = p;
   up.r = r;
   up.minv = minv;
   up.beta = &P->scal->beta;
-  const ax::AlphaJob job = alpha_job<float>(P);
+  const ax::AlphaJob job = alpha_job<float>(P, chained);
   return apply_lowp(P, w, p, st, P->dotp, &up, &job);
 }
 
@@ -547,16 +550,24 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
   // in fp64 together with the x update of the step before
   const bool fused_p = fused && fuses_update(P, (const T *)nullptr);
   const bool fused_x = fused_p && std::is_same_v<T, double>;
+  // The gather-scatter begins while the apply ends only on smaller meshes: its
+  // blocks, and those of the update chained behind it, then stand ready, but
+  // once the grids are many times what the chip holds they only take the
+  // running kernel's places.  us an iteration at lx = 8, chained against not:
+  // fp32 6^3 elements 18.1 / 20.5, 10^3 26.8 / 25.2 (bf16 data 22.3 / 24.3),
+  // 16^3 47.7 / 46.0, 20^3 82.9 / 76.4, 32^3 301 / 271; fp64 16^3 94.7 / 99.0,
+  // 24^3 279.2 / 282.1, 28^3 436 / 439, 32^3 646.8 / 642.6.
+  const bool gs_chained = n < (std::is_same_v<T, double> ? int64_t(1) << 24 : int64_t(1) << 19);
   // The first half of iteration `it`: direction, apply, alpha.  It touches no
   // result (x only to complete the step before), so it is launched before the
   // host has tested that step: the GPU goes on while the test's values travel.
   auto front = [&](int it) -> int {
-    if (fused_p && it > 0) return apply_fused_update(P, w, p, r, minv, x, st);
+    if (fused_p && it > 0) return apply_fused_update(P, w, p, r, minv, x, st, nullptr, gs_chained);
     int rc = AX_OK;
     if (it > 0)
       rc = ax::launch_chained(true, cg_p_kernel<T>, nb, kRedThreads, 0, st, p, r, minv, P->scal, n);
     if (rc) return rc;
-    if (fused) return apply_fused(P, w, p, st);
+    if (fused) return apply_fused(P, w, p, st, gs_chained);
     if ((rc = apply(w, p, st))) return rc;
     return ax::launch_chained(true, mask_dot_kernel<T>, nb, kRedThreads, 0, st, w, p, mask, c,
                               P->partials, n, P->scal);
@@ -1123,7 +1134,9 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
 // with cm = c * minv the Jacobi pair costs 3 multiply-adds and the correction
 // pair 3 more (in fp64 the narrow pipe, not memory, bounds this kernel).  From
 // them rz (first: of <z0, r0>, else with Notay's beta) and the choice between
-// the learned and the Jacobi step.  fp32: 16-byte accesses.
+// the learned and the Jacobi step.  16-byte accesses, two in flight: with one
+// 8-byte load at a time the fp64 iteration without a network took 822 us
+// against 728 us at 32768 elements, lx = 8.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads, kRedPerSm)
 fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
@@ -1145,23 +1158,28 @@ fcg_dots_kernel(const T *__restrict__ r, const T *__restrict__ r_old,
     }
   };
   int64_t q0 = 0;
-  if constexpr (sizeof(T) == 4) {
-    if (aligned16(r, r_old, corr, cm, c)) {
-      using V = float4;
-      const int64_t n4 = n / 4;
-#pragma unroll 2
-      for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4;
-           v += (int64_t)gridDim.x * blockDim.x) {
-        auto at = [v](const T *p) { return __ldcg(reinterpret_cast<const V *>(p) + v); };
-        const V rv = at(r), ro = at(r_old), mv = at(cm);
-        const V cv = have_corr ? at(c) : V{}, ev = have_corr ? at(corr) : V{};
-        point(rv.x, ro.x, mv.x, cv.x, ev.x);
-        point(rv.y, ro.y, mv.y, cv.y, ev.y);
-        point(rv.z, ro.z, mv.z, cv.z, ev.z);
-        point(rv.w, ro.w, mv.w, cv.w, ev.w);
-      }
-      q0 = n4 * 4;
-    }
+  if (aligned16(r, r_old, corr, cm, c)) {  // 16-byte accesses
+    using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+    constexpr int NV = 16 / sizeof(T);
+    V rv[2], ov[2], mv[2], cv[2], ev[2];
+    auto at = [](const T *f, int64_t v) { return __ldcg(reinterpret_cast<const V *>(f) + v); };
+    walk2(
+        n / NV,
+        [&](int k, int64_t v) {
+          rv[k] = at(r, v);
+          ov[k] = at(r_old, v);
+          mv[k] = at(cm, v);
+          cv[k] = have_corr ? at(c, v) : V{};
+          ev[k] = have_corr ? at(corr, v) : V{};
+        },
+        [&](int k, int64_t) {
+#pragma unroll
+          for (int l = 0; l < NV; ++l)
+            point(reinterpret_cast<const T *>(&rv[k])[l], reinterpret_cast<const T *>(&ov[k])[l],
+                  reinterpret_cast<const T *>(&mv[k])[l], reinterpret_cast<const T *>(&cv[k])[l],
+                  reinterpret_cast<const T *>(&ev[k])[l]);
+        });
+    q0 = n / NV * NV;
   }
   for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x)

@@ -50,11 +50,13 @@ AX_D void cg_set_alpha(CgScalars *s, double pap) {
 }
 
 // The apply's partials of <p, Ap>, summed by one extra block of the
-// gather-scatter that follows the apply, which then sets alpha.
+// gather-scatter that follows the apply, which then sets alpha.  chained: the
+// gather-scatter may begin while the apply ends.
 struct AlphaJob {
   const double *partials = nullptr;
   int n = 0;
   CgScalars *s = nullptr;
+  bool chained = true;
 };
 
 }  // namespace ax

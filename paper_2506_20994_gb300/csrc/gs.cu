@@ -98,7 +98,7 @@ int gs_sum_launch(ax_gs *g, T *v, const ax::AlphaJob *job, cudaStream_t st) {
   if (g->n_shared > 0 && !v) return AX_EINVAL;
   const unsigned grid = (unsigned)((g->n_shared + kGsThreads - 1) / kGsThreads);
   if (job)
-    return ax::launch_chained(true, gs_sum_kernel<T, true>, grid + 1, kGsThreads, 0, st, v, g->d_pairs,
+    return ax::launch_chained(job->chained, gs_sum_kernel<T, true>, grid + 1, kGsThreads, 0, st, v, g->d_pairs,
                               g->n_pairs, g->d_off, g->d_idx, g->n_multi, *job);
   return ax::launch_chained(true, gs_sum_kernel<T, false>, grid, kGsThreads, 0, st, v, g->d_pairs,
                             g->n_pairs, g->d_off, g->d_idx, g->n_multi, ax::AlphaJob{});
