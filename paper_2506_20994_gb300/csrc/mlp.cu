@@ -255,7 +255,7 @@ mlp_apply_kernel(T *__restrict__ corr, const T *__restrict__ r, const T *__restr
 
 // Symmetric form with its scale precomputed (sc = sqrt(minv), fp32) and an
 // even number of points per element: a block takes 16 elements (the rows of
-// the mma tiles) through both layers.  All four warps load and scale the rows
+// the mma tiles) through both layers.  All the warps load and scale the rows
 // together (every load of a row in flight at once) into shared memory as
 // bf16; the warps then share layer 1's hidden n-tiles and, from the hidden
 // layer in shared memory, layer 2's output tiles.  Weights come through L1/L2.
@@ -263,9 +263,12 @@ mlp_apply_kernel(T *__restrict__ corr, const T *__restrict__ r, const T *__restr
 // (8 rows x 4 words) touch every bank once.
 // With one warp streaming 16 elements by itself, 4096 elements were 256 warps
 // on 152 SMs, each a chain of 32 load latencies: 42 us, against 24 us here
-// (fp32, lx = 8, 48 hidden units).  Sums keep their order (k ascending in each
-// tile), so the results are the same bits.
-constexpr int kSymWarps = 4;  // warps per block
+// (fp32, lx = 8, 48 hidden units) with four warps.  Eight shorten the chain of
+// each warp again: a refinement iteration with the network (lx = 8) takes 84.8
+// against 93.9 us at 16^3 elements, 40.8 / 45.3 at 6^3, 268 / 273 at 26^3;
+// sixteen 83.2 at 16^3 but 277 at 26^3.  Sums keep their order (k ascending in
+// each tile), so the results are the same bits.
+constexpr int kSymWarps = 8;  // warps per block
 
 template <typename T>
 struct Pair;  // two consecutive values of T
@@ -316,7 +319,7 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
   }
   __syncthreads();
 
-  // layer 1: hidden n-tiles wp, wp + 4
+  // layer 1: hidden n-tiles wp, wp + kSymWarps
   const __nv_bfloat16 *x0 = xs + g * XS + 2 * t4, *x1 = x0 + 8 * XS;
   constexpr int TW = (NT1 + kSymWarps - 1) / kSymWarps;
   float acc[TW][4];
@@ -351,7 +354,7 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
   }
   __syncthreads();
 
-  // layer 2: output tiles wp, wp + 4, ...; corr = sc * y
+  // layer 2: output tiles wp, wp + kSymWarps, ...; corr = sc * y
   uint32_t a2[NT1 / 2][4];
 #pragma unroll
   for (int q = 0; q < NT1 / 2; ++q) {
