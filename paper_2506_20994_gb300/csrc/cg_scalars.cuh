@@ -7,7 +7,7 @@
 namespace ax {
 
 struct CgScalars {
-  double rz, rz_new, rr, rr0, pap, alpha, beta;
+  double rz, rr, rr0, pap, alpha, beta;
   int status;     // 0 ok, 1 breakdown (p.Ap <= 0 or non-finite)
   int use_corr;   // flexible CG: 1 if the learned correction is in z
   int fallbacks;  // flexible CG: steps that fell back to Jacobi
