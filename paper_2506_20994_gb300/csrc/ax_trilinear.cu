@@ -14,7 +14,8 @@
 // fp32 (differences of nearby fp64 coordinates, so the fp32 values keep full
 // relative precision).  Per thread (i, j) of the k-loop schedule: the t-column
 // of J is constant over k and the r- and s-columns are linear in the
-// k-position, so J costs 12 fp32 operations per point and G about 50 more.
+// k-position, so J costs 12 fp32 operations per point, adj(J) and det J about
+// 20 and the product with the gradient 21 (G itself is not formed).
 // Reads u (and h1 unless it is constant 1) and writes w: 8 or 12 bytes per
 // point against 36 for the stored-geometry fp32 kernel.
 #include "common.cuh"
