@@ -1,0 +1,54 @@
+"""The solvers on both sides of the mesh size from which the gather-scatter is
+launched without overlap, and the flexible loop's wide loads with and without
+a scalar remainder: the residual is formed anew with the library's operator."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2506_20994_gb300 as ax  # noqa: E402
+from paper_2506_20994_gb300 import synth  # noqa: E402
+
+TOL = 1e-7
+
+
+def _solve_and_check(dims, lx, solve):
+    P = ax.Poisson(synth.box_vertices(*dims), lx)
+    b = P.rhs(synth.poisson_source)
+    x, relres = solve(P, b)
+    Ax = torch.empty_like(b)
+    P.apply(Ax, x)
+    m = P.d["mask"].reshape(b.shape)
+    r, s = (m * (b - Ax)).norm(), (m * b).norm()
+    # the returned figure weighs shared points by 1/copies (1 to 8 of them), so
+    # the plain norms' ratio is within a factor sqrt(8) of it
+    assert relres <= TOL
+    assert float(r / s) <= 8 ** 0.5 * TOL * 1.01
+
+
+# 512000 and 563200 points: below and above the line for fp32 vectors
+@pytest.mark.parametrize("mode", [ax.AX_PREC_F32, ax.AX_PREC_BF16])
+@pytest.mark.parametrize("dims", [(10, 10, 10), (11, 10, 10)])
+def test_refinement_around_the_size_line(dims, mode):
+    def solve(P, b):
+        q = P.mpcg(b, mode=mode, tol=TOL)
+        return q[0], q[-2]
+    _solve_and_check(dims, 8, solve)
+
+
+# 2^24 points and one element layer less: the fp64 line
+@pytest.mark.parametrize("dims", [(32, 32, 31), (32, 32, 32)])
+def test_cg_around_the_size_line(dims):
+    def solve(P, b):
+        q = P.cg(b, tol=TOL)
+        return q[0], q[-2]
+    _solve_and_check(dims, 8, solve)
+
+
+# an even and an odd number of points (lx odd: the last one by itself)
+@pytest.mark.parametrize("dims,lx", [((3, 3, 3), 5), ((3, 3, 3), 6), ((1, 1, 1), 7)])
+def test_flexible_loop_points_odd_and_even(dims, lx):
+    def solve(P, b):
+        q = P.fcg(b, None, tol=TOL)
+        return q[0], q[2]
+    _solve_and_check(dims, lx, solve)
