@@ -70,6 +70,12 @@ DF_HD float sub(float a, float b) { return __fsub_rn(a, b); }
 DF_HD float mul(float a, float b) { return __fmul_rn(a, b); }
 DF_HD float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 DF_HD int f2i_rn(float a) { return __float2int_rn(a); }
+// a - b with subnormal operands and results taken as zero
+DF_HD float sub_ftz(float a, float b) {
+  float r;
+  asm("sub.rn.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 #else
 // Host twins (used by the host-side self-test entry point only); volatile
 // keeps the host compiler from contracting the error-free transformations.
@@ -78,6 +84,12 @@ DF_HD float sub(float a, float b) { volatile float r = a - b; return r; }
 DF_HD float mul(float a, float b) { volatile float r = a * b; return r; }
 DF_HD float fma(float a, float b, float c) { return __builtin_fmaf(a, b, c); }
 DF_HD int f2i_rn(float a) { return (int)__builtin_nearbyintf(a); }
+DF_HD float sub_ftz(float a, float b) {
+  auto flush = [](float v) {
+    return __builtin_fabsf(v) < 0x1p-126f ? __builtin_copysignf(0.f, v) : v;
+  };
+  return flush(sub(flush(a), flush(b)));
+}
 #endif
 
 // max(a + b, c), one instruction on the device
@@ -90,14 +102,18 @@ DF_HD int addmax(int a, int b, int c) {
 }
 
 // --- fp64 -> double-float split, integer ops only ---------------------------
-// hi = x truncated to 24 significant bits; lo = the next 23 bits of x, so
-// |x - (hi + lo)| < 2^-46 |x| for 2^-103 <= |x| < 2^128.  Smaller magnitudes
-// keep an absolute error below 2^-125 (hi flushes toward zero below 2^-126).
+// hi = x truncated to 24 significant bits; lo = the next 23 bits of x, taken
+// as zero where it would be subnormal.  So |x - (hi + lo)| is below
+//   max(2^-46 |x|, 2^-126)  for 2^-103 <= |x| < 2^128,
+//   2^-23 |x|               for 2^-126 <= |x| < 2^-103 (lo = 0),
+//   max(|x|, 2^-146)        below (lo = 0, hi at most 7 2^-149).
 // Nine integer instructions and one subtraction: lo is the difference of two
 // fp32 numbers of its sign and of exponent(hi) - 23, one with the 23 bits as
-// its mantissa and one with none (exact); the exponent is clamped at zero,
-// where both are subnormal.  (Scaling the 23 bits by a power of two chosen by
-// a compare took sixteen.)
+// its mantissa and one with none (exact).  Where exponent(hi) - 23 would be
+// no normal exponent it is clamped at zero: both numbers are subnormal then,
+// their difference has no relation to x's scale, and the flushing subtraction
+// makes it zero.  (Scaling the 23 bits by a power of two chosen by a compare
+// took sixteen.)
 DF_HD df2 split(double x) {
   const uint64_t b = d2u(x);
   const uint32_t hw = (uint32_t)(b >> 32), lw = (uint32_t)b;
@@ -108,7 +124,7 @@ DF_HD df2 split(double x) {
   const uint32_t base = (uint32_t)addmax((int)(fm & 0x7F800000u), -(23 << 23), 0) | sgn;
   df2 o;
   o.hi = u2f(fm | sgn);
-  o.lo = sub(u2f(base | ((lw >> 6) & 0x7FFFFFu)), u2f(base));
+  o.lo = sub_ftz(u2f(base | ((lw >> 6) & 0x7FFFFFu)), u2f(base));
   return o;
 }
 

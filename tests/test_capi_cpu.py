@@ -122,6 +122,26 @@ def test_df64_small_and_special_values():
     assert back[0] == 0.0 and back[1] == 0.0
 
 
+def test_df64_split_near_the_bottom_of_the_range():
+    """The split's error at every magnitude below 2^-70, with random mantissas:
+    2^-46 |x| but for a tail that would be subnormal (below 2^-126, taken as
+    zero); 24 bits where there is no tail; and no stray value for fp64
+    subnormals, whose low mantissa bits are all set."""
+    g = synth.rng(8)
+    m = g.uniform(1.0, 2.0, size=40000) * np.where(g.uniform(size=40000) < 0.5, -1.0, 1.0)
+    x = np.ldexp(m, g.integers(-1074, -70, size=m.size))
+    low = np.ldexp(m[:4000], g.integers(-150, -70, size=4000))  # where the bounds change
+    edges = np.ldexp(np.outer([1.0, 2.0 - 2.0 ** -52], np.ones(80)), -np.arange(70, 150)).ravel()
+    x = np.concatenate([x, low, edges, -edges, [1e-310, -1e-300, 5e-324, 2.0 ** -1022]])
+    hi, lo, _ = ax.df64_roundtrip(x)
+    a = np.abs(x)
+    err = np.abs(x - (hi.astype(np.float64) + lo.astype(np.float64)))
+    bound = np.where(a >= 2.0 ** -103, np.maximum(2.0 ** -46 * a, 2.0 ** -126),
+                     np.where(a >= 2.0 ** -126, 2.0 ** -23 * a, np.maximum(a, 2.0 ** -146)))
+    assert np.all(err <= bound)
+    assert np.all(lo[a < 2.0 ** -103] == 0.0)
+
+
 def test_df64_join_rounds_pairs():
     """join(hi, lo) of a normalised pair is within one fp64 ulp of hi + lo,
     including pairs that cross a power of two downwards."""
