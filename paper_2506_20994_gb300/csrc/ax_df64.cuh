@@ -100,16 +100,16 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
   if constexpr (LX % 2 == 0) prefetch_elements(u, h1, g11, g22, g33, g12, g13, g23, e0, nel, N3);
 
   df2 uk[LX];
-  unsigned ukey = 0u, gkey = 0u, hkey = 0u;  // exponent keys of u, G, h1
+  guard::Key ukey, gkey, hkey;  // exponent keys of u, G, h1
   if (own) {
 #pragma unroll
     for (int k = 0; k < LX; ++k) {
       const double x = active ? __ldcg(u + base + (size_t)k * N2) : 0.0;
-      ukey = max(ukey, guard::key(x));
+      ukey.note(x);
       uk[k] = split(x);
       su[k * N2 + p] = uk[k];
     }
-    if (active) atomicMax(&rec.ex[le][0], ukey);
+    if (active) atomicMax(&rec.ex[le][0], ukey.get());
   }
   __syncthreads();
 
@@ -133,10 +133,13 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
         const double v11 = __ldcg(g11 + q), v22 = __ldcg(g22 + q), v33 = __ldcg(g33 + q);
         const double v12 = __ldcg(g12 + q), v13 = __ldcg(g13 + q), v23 = __ldcg(g23 + q);
         const double vh = __ldcg(h1 + q);
-        gkey = max(gkey, max(max(guard::key(v11), guard::key(v22)),
-                             max(max(guard::key(v33), guard::key(v12)),
-                                 max(guard::key(v13), guard::key(v23)))));
-        hkey = max(hkey, guard::key(vh));
+        gkey.note(v11);
+        gkey.note(v22);
+        gkey.note(v33);
+        gkey.note(v12);
+        gkey.note(v13);
+        gkey.note(v23);
+        hkey.note(vh);
         const df2 a11 = split(v11), a22 = split(v22);
         const df2 a33 = split(v33), a12 = split(v12);
         const df2 a13 = split(v13), a23 = split(v23);
@@ -165,8 +168,8 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
       }
     }
     if (active) {
-      atomicMax(&rec.ex[le][1], gkey);
-      atomicMax(&rec.ex[le][2], hkey);
+      atomicMax(&rec.ex[le][1], gkey.get());
+      atomicMax(&rec.ex[le][2], hkey.get());
     }
   }
   __syncthreads();

@@ -164,7 +164,7 @@ __global__ void geo_urange_kernel(unsigned *__restrict__ keys, int nelv, int fd)
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nelv) return;
   unsigned packed, zero_ok;
-  guard::u_range(guard::field(keys[2 * e]), guard::field(keys[2 * e + 1]), fd, packed, zero_ok);
+  guard::u_range(keys[2 * e], keys[2 * e + 1], fd, packed, zero_ok);
   keys[2 * e] = packed;
   keys[2 * e + 1] = zero_ok;
 }
@@ -246,6 +246,7 @@ bool eop_coefficients(int lx, const double *dx_h, const double *dxt_h, void *out
   int ex = 0;
   std::frexp(dmax, &ex);
   *dfield = dmax > 0.0 ? ex - 1 + 1023 : 0;
+  if (dmax > 0.0 && *dfield < 1) *dfield = 2047;  // subnormal: fp64 units
   auto bits = [](float f) { return (unsigned long long)df::f2u(f); };
   const int CS = H + 1;
   df::dd2 *cf = static_cast<df::dd2 *>(out);

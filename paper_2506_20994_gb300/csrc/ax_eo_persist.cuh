@@ -357,7 +357,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       const double dmax = __longlong_as_double((long long)drec[0]);
       const double ddev = __longlong_as_double((long long)drec[1]);
       raw_ok = isfinite(dmax) && ddev <= dmax * 0x1p-46;
-      raw_fd = (int)((drec[0] >> 52) & 0x7FFull);
+      raw_fd = guard::d_field(drec[0]);
     } else {
       for (int q = tid; q < (int)(C::COEF_BYTES / 16); q += C::NTB)
         reinterpret_cast<ulonglong2 *>(sm)[q] =
@@ -444,7 +444,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     // ---- phase 1: this element's u (or the direction formed here), split,
     // lines of the three directions; the next element's inputs start loading
     double ucur[2][2];
-    unsigned uk = 0u;
+    guard::Key ukk;
     double xv[2][2];
     if constexpr (PUPD) {
       if (real && up.x) {
@@ -466,7 +466,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
           if (real) up.pw[eb + pidx(b, a)] = x;
         }
         ucur[b][a] = x;
-        uk = max(uk, guard::key(x));
+        ukk.note(x);
       }
     df2 v[2][2];
 #pragma unroll
@@ -483,7 +483,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       }
     }
     if (real && more) load_in(nxp);
-    uk = __reduce_max_sync(0xffffffffu, real ? uk : 0u);
+    const unsigned uk = __reduce_max_sync(0xffffffffu, real ? ukk.get() : 0u);
     if ((tid & 31) == 0) kslot[tid >> 5] = uk;
     publish(Lb, v, v, v);
     sync();
@@ -494,7 +494,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 
     // ---- phase 3: pointwise h1 G with this element's staged geometry
     const bool got = mbar_wait(bar, parity, kWaitLimit);
-    unsigned gk = 0u, hk = 0u;  // RAW: exponent keys of this thread's G and h1 values
+    guard::Key gk, hk;  // RAW: exponent keys of this thread's G and h1 values
     {
       const u64 zero = pk(0.f, 0.f);
 #pragma unroll
@@ -506,11 +506,9 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 #pragma unroll
           for (int f = 0; f < 7; ++f) {
             const double v0 = Gr[f * N3 + q0], v1 = Gr[f * N3 + q1];
-            const unsigned k = max(guard::key(v0), guard::key(v1));
-            if (f < 6)
-              gk = max(gk, k);
-            else
-              hk = max(hk, k);
+            guard::Key &k = f < 6 ? gk : hk;
+            k.note(v0);
+            k.note(v1);
             const df2 s0 = split(v0), s1 = split(v1);
             g[f] = dd2{pk(s0.hi, s1.hi), pk(s0.lo, s1.lo)};
           }
@@ -544,11 +542,11 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       }
     }
     if constexpr (RAW) {
-      gk = __reduce_max_sync(0xffffffffu, real ? gk : 0u);
-      hk = __reduce_max_sync(0xffffffffu, real ? hk : 0u);
+      const unsigned gw = __reduce_max_sync(0xffffffffu, real ? gk.get() : 0u);
+      const unsigned hw = __reduce_max_sync(0xffffffffu, real ? hk.get() : 0u);
       if ((tid & 31) == 0) {
-        gslot[2 * (tid >> 5)] = gk;
-        gslot[2 * (tid >> 5) + 1] = hk;
+        gslot[2 * (tid >> 5)] = gw;
+        gslot[2 * (tid >> 5) + 1] = hw;
       }
     }
     // every thread is done with the geometry and the gradient lines
@@ -590,10 +588,9 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
         gke = max(gke, gslot[2 * q]);
         hke = max(hke, gslot[2 * q + 1]);
       }
-      bad = !raw_ok || !guard::window_ok(guard::field(uke), guard::field(gke),
-                                         guard::field(hke), raw_fd);
+      bad = !raw_ok || !guard::window_ok(uke, gke, hke, raw_fd);
     } else {
-      bad = !guard::u_in_range(ur_e, guard::field(uke));
+      bad = !guard::u_in_range(ur_e, uke);
     }
 
     // ---- phase 4: lines of the weighted gradient

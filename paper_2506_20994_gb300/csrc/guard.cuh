@@ -14,10 +14,11 @@
 // fp64 units, so that it gets IEEE fp64 semantics.  The same routine serves
 // the even-odd kernels when the matrices are not centro-antisymmetric.
 //
-// Values below 2^-1022 (fp64 subnormals) count as zero in the exponent
-// record; inside the window the double-float split flushes any value more
-// than ~2^125 below the element's largest one, an absolute change below
-// 2^-47 of that element's scale.
+// Inside the window the double-float split changes a value by at most 2^-126
+// where its own bound is not met (df64.cuh), below 2^-47 of the element's
+// scale.  A factor of zeros alone is inside it (w = 0) as long as nothing
+// infinite can meet the zeros; one whose largest value is an fp64 subnormal is
+// not.
 #pragma once
 
 #include <stdint.h>
@@ -28,20 +29,38 @@ namespace ax {
 namespace guard {
 
 // Ordered key of |x|'s binary exponent: the fp64 high word shifted left by
-// one (sign dropped).  max over values, then `field` recovers the biased
-// exponent (0: zero or subnormal, 2047: Inf or NaN).
-AX_D unsigned key(double x) {
-  return (unsigned)(__double_as_longlong(x) >> 31) & 0xFFFFFFFEu;
-}
+// one (sign dropped), its last bit set where the low word holds anything, so
+// that only a zero has key 0.  max over values, then `field` recovers the
+// biased exponent (0: zero or subnormal, 2047: Inf or NaN).
+AX_D unsigned hkey(double x) { return (unsigned)__double2hiint(x) << 1; }
+AX_D unsigned key(double x) { return hkey(x) + min((unsigned)__double2loint(x), 1u); }
+// The key of several values' maximum, low words or-ed together: half an
+// instruction a value for the last bit where `key` takes one (ax_helm on raw
+// arrays at lx = 8, 32768 elements: 378 us without the bit, 384 so, 391 with
+// `key`).
+struct Key {
+  unsigned h = 0u, l = 0u;
+  AX_D void note(double x) {
+    h = max(h, hkey(x));
+    l |= (unsigned)__double2loint(x);
+  }
+  AX_D unsigned get() const { return h + min(l, 1u); }
+};
 AX_HD int field(unsigned k) { return (int)(k >> 21); }
 
-// Window of the double-float arithmetic, from the biased exponent fields of
-// the element maxima of u, G, h1 and of the matrices D (fd).  A zero factor
-// gives w = 0 exactly; a non-finite one must go to fp64 units.
-AX_HD bool window_ok(int fu, int fg, int fh, int fd) {
+// Window of the double-float arithmetic, from the keys of the element maxima
+// of u, G and h1 and the biased exponent field of the matrices D (fd, 2047
+// where they are subnormal).  A non-finite factor must go to fp64 units.  A
+// zero one gives w = 0 exactly where the other factors and the products in
+// front of it stay finite in fp32.
+AX_HD bool window_ok(unsigned ku, unsigned kg, unsigned kh, int fd) {
+  const int fu = field(ku), fg = field(kg), fh = field(kh);
   if (fu == 2047 || fg == 2047 || fh == 2047 || fd == 2047) return false;
-  if (fu == 0 || fg == 0 || fh == 0 || fd == 0) return true;
   const int a = fu - 1023, b = fg - 1023, c = fh - 1023, d = fd - 1023;
+  if (ku == 0u || kg == 0u || kh == 0u || fd == 0) {  // a zero counts as 2^-1023
+    return a <= 90 && b <= 90 && c <= 90 && d <= 24 && a + d <= 100 && a + b + d <= 100 &&
+           a + b + c + d <= 100;
+  }
   auto in = [](int x, int lo, int hi) { return x >= lo && x <= hi; };
   // each factor: head and tail normal fp32 numbers
   if (!in(a, -78, 90) || !in(b, -78, 90) || !in(c, -78, 90) || !in(d, -24, 24)) return false;
@@ -52,29 +71,23 @@ AX_HD bool window_ok(int fu, int fg, int fh, int fd) {
          in(a + b + c + 2 * d, -90, 100);
 }
 
-// For fixed G, h1 and D exponent fields, the u fields window_ok accepts form
-// one interval; u_range packs it as {lo | hi << 16, zero_ok} (zero_ok: an
-// all-zero u is fine, i.e. nothing is non-finite), u_in_range tests it.
-AX_HD void u_range(int fg, int fh, int fd, unsigned &packed, unsigned &zero_ok) {
+// For fixed G and h1 keys and D exponent field, the u fields window_ok accepts
+// form one interval; u_range packs it as {lo | hi << 16, zero_ok} (zero_ok: an
+// all-zero u is fine), u_in_range tests it.
+AX_HD void u_range(unsigned kg, unsigned kh, int fd, unsigned &packed, unsigned &zero_ok) {
   int lo = 1, hi = 0;  // empty
-  zero_ok = (fg != 2047 && fh != 2047 && fd != 2047) ? 1u : 0u;
-  if (zero_ok) {
-    if (fg == 0 || fh == 0 || fd == 0) {
-      lo = 1;
-      hi = 2046;  // a zero factor: any finite u
-    } else {
-      for (int fu = 1; fu <= 2046; ++fu) {  // the window is an interval in fu
-        if (window_ok(fu, fg, fh, fd)) {
-          if (lo > hi) lo = fu;
-          hi = fu;
-        }
-      }
+  zero_ok = window_ok(0u, kg, kh, fd) ? 1u : 0u;
+  for (int fu = 1; fu <= 2046; ++fu) {  // the window is an interval in fu
+    if (window_ok((unsigned)fu << 21, kg, kh, fd)) {
+      if (lo > hi) lo = fu;
+      hi = fu;
     }
   }
   packed = (unsigned)lo | ((unsigned)hi << 16);
 }
-AX_HD bool u_in_range(uint2 r, int fu) {
-  if (fu == 0) return r.y != 0u;
+AX_HD bool u_in_range(uint2 r, unsigned ku) {
+  if (ku == 0u) return r.y != 0u;
+  const int fu = field(ku);
   return fu >= (int)(r.x & 0xFFFFu) && fu <= (int)(r.x >> 16);
 }
 
@@ -108,9 +121,10 @@ AX_D void note_pair(Record &r, double a, double mirrored) {
   atomicMax(&r.dmax, abs_bits(a) > abs_bits(mirrored) ? abs_bits(a) : abs_bits(mirrored));
   atomicMax(&r.ddev, abs_bits(__dadd_rn(a, mirrored)));
 }
-// field of the largest |D|
-AX_D int d_field(const Record &r) {
-  return (int)((r.dmax >> 52) & 0x7FFull);
+// field of the largest |D| from its bits; 2047 where that is a subnormal
+AX_D int d_field(unsigned long long dmax) {
+  const int f = (int)((dmax >> 52) & 0x7FFull);
+  return f == 0 && dmax != 0ull ? 2047 : f;
 }
 // matrices centro-antisymmetric to 2^-46 of their largest entry (the split of
 // the even-odd kernels reads only half the rows; a defect this small changes
@@ -121,7 +135,7 @@ AX_D bool centro_ok(const Record &r) {
   return dev <= dmax * 0x1p-46;
 }
 AX_D bool elem_ok(const Record &r, int le) {
-  return window_ok(field(r.ex[le][0]), field(r.ex[le][1]), field(r.ex[le][2]), d_field(r));
+  return window_ok(r.ex[le][0], r.ex[le][1], r.ex[le][2], d_field(r.dmax));
 }
 
 // w_e = D^T (h1 G (D u_e)) of one element with fp64 units, in the loop order

@@ -183,3 +183,51 @@ def test_batched_launch_scaled_meshes():
     torch.cuda.synchronize()
     for w, ref in zip(outs, refs):
         _check(w.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("lx", [5, 6, 8, 10])
+@pytest.mark.parametrize("how", ENTRIES + ["batch"], ids=ENTRY_IDS + ["batch"])
+def test_subnormal_and_zero_factors(lx, how):
+    """Elements in which one factor holds only fp64 subnormals, next to large
+    other factors (the product is far from zero in fp64), and elements in which
+    one factor is zero while another is beyond the fp32 range (the result is
+    zero, not 0 * Inf).  Subnormals down to 1e-309 carry 2^-48 relative, and
+    sums of lx terms of them lose less than 1e-13."""
+    if how == ax.AX_VARIANT_F64_DF_EO and lx % 2:
+        pytest.skip("the even-odd kernel takes even lx")
+    c = operator_case((4, 2, 1), lx, seed=960 + lx)
+    u, h1 = c["u"].copy(), c["h1"].copy()
+    G = {k: c[k].copy() for k in GKEYS}
+
+    def scale(e, su, sg, sh):
+        u[e] *= su
+        h1[e] *= sh
+        for k in GKEYS:
+            G[k][e] *= sg
+
+    scale(0, 1e-309, 1e27, 1e27)
+    scale(1, 1e27, 1e-309, 1e27)
+    scale(2, 1e27, 1e27, 1e-309)
+    scale(3, 0.0, 1e39, 1.0)
+    scale(4, 1e39, 1.0, 0.0)
+    scale(5, 1e30, 0.0, 1e30)
+    G["g12"][6][...] = 0.0
+    u[7][...] = 0.0
+    u[7][1, 1, 1] = 1e-315  # one subnormal in an element of zeros
+    c.update(G, u=u, h1=h1)
+    ref = _oracle(c)
+    if how == "batch":
+        t = {k: _dev(c[k]) for k in ("u", "dx", "dxt", "h1") + GKEYS}
+        t["w"] = torch.full_like(t["u"], 5.0)
+        ax.Batch([dict(lx=lx, **t)]).launch()
+        torch.cuda.synchronize()
+        got = t["w"].cpu().numpy()
+    else:
+        got = _run(c, how)
+    for e in (0, 1, 2, 6):
+        assert np.abs(ref[e]).max() > 1e-270
+        _check(got[e], ref[e])
+    for e in (3, 4, 5):
+        assert not ref[e].any() and not got[e].any()
+    # products of a 28-bit subnormal: within the spacing of fp64 there, a few times
+    assert np.all(np.abs(got[7] - ref[7]) <= 4e3 * 5e-324 * np.abs(c["dx"]).max() ** 2)
