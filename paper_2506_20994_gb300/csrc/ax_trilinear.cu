@@ -143,7 +143,31 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
     const float b1 = __fmaf_rn(cf[24 + d * 4 + 3], pi1, cf[24 + d * 4 + 2] * pi0);
     Jt[d] = __fmaf_rn(b1, pj1, b0 * pj0);
   }
-  const float wij = swq[i] * swq[j];
+  // The column's edge vectors scaled by a power of two into |.| < 1/4, and
+  // that power put back with the weights: adj(J) and det J are then of order
+  // one whatever the size of the element (unscaled, h^2 and h^3 met u), and
+  // the products with u stay within fp32 wherever u, G grad u and w do.  Exact
+  // but for subnormals, and not measurable (25^3 elements at lx 6: 28.1 us both
+  // ways).
+  float big = fmaxf(fmaxf(fabsf(Jt[0]), fabsf(Jt[1])), fabsf(Jt[2]));
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) big = fmaxf(fmaxf(big, fabsf(P[d][c])), fabsf(Q[d][c]));
+  // exponent field of the scale: that of 2^-3 over big's own, normal both ways
+  const int se = max(251 - (int)(__float_as_uint(big) >> 23), 1);
+  const float down = __uint_as_float((unsigned)se << 23);
+  const float up = __uint_as_float((unsigned)(254 - se) << 23);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      P[d][c] *= down;
+      Q[d][c] *= down;
+    }
+    Jt[d] *= down;
+  }
+  const float wij = swq[i] * swq[j] * up;
 
   float wacc[LX];
   if (own) {
@@ -201,14 +225,16 @@ ax_tri_f32_kernel(float *__restrict__ w, const float *__restrict__ u,
         const float det = __fmaf_rn(a, A00, __fmaf_rn(b, A10, c * A20));
         float s = __fdividef(wij * swq[k], det);  // fp32 operator: ~2 ulp is ample
         if constexpr (H1) s *= hk[k];
-        // w = s A (A^T grad), A^T grad = sum of the rows times ur, us, ut: 21
-        // operations where the six factors of G and their product take 33
-        const float tx = __fmaf_rn(A00, ur, __fmaf_rn(A10, us, A20 * ut));
-        const float ty = __fmaf_rn(A01, ur, __fmaf_rn(A11, us, A21 * ut));
-        const float tz = __fmaf_rn(A02, ur, __fmaf_rn(A12, us, A22 * ut));
-        wr = s * __fmaf_rn(A00, tx, __fmaf_rn(A01, ty, A02 * tz));
-        ws = s * __fmaf_rn(A10, tx, __fmaf_rn(A11, ty, A12 * tz));
-        wt = s * __fmaf_rn(A20, tx, __fmaf_rn(A21, ty, A22 * tz));
+        // w = A (s A^T grad), A^T grad = sum of the rows times ur, us, ut: 21
+        // operations where the six factors of G and their product take 33 (s
+        // in the middle: for a thin element A A^T grad alone is its thickness
+        // squared times u)
+        const float tx = s * __fmaf_rn(A00, ur, __fmaf_rn(A10, us, A20 * ut));
+        const float ty = s * __fmaf_rn(A01, ur, __fmaf_rn(A11, us, A21 * ut));
+        const float tz = s * __fmaf_rn(A02, ur, __fmaf_rn(A12, us, A22 * ut));
+        wr = __fmaf_rn(A00, tx, __fmaf_rn(A01, ty, A02 * tz));
+        ws = __fmaf_rn(A10, tx, __fmaf_rn(A11, ty, A12 * tz));
+        wt = __fmaf_rn(A20, tx, __fmaf_rn(A21, ty, A22 * tz));
       }
       swr[k * N2 + p] = wr;
       sws[k * N2 + p] = ws;

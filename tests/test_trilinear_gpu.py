@@ -106,3 +106,20 @@ def test_trilinear_full_size_sampled():
                          *[geo[k] for k in GKEYS], lx)
     assert rel_l2(w[idx], ref) <= TOL
     assert np.isfinite(w).all()
+
+
+@pytest.mark.parametrize("lx", [3, 6, 8, 13])
+@pytest.mark.parametrize("h,mag", [(1e-8, 1e-20), (1e8, 1e20), (1e-9, 1e25), (1e9, 1e-25),
+                                   (1e-12, 1.0), (1e12, 1.0)])
+def test_trilinear_scales(lx, h, mag):
+    """Meshes and fields far from order one whose u, G and w are ordinary fp32
+    numbers: h^4 u and h^-3 of the adjugate form would not be."""
+    v = synth.box_vertices(3, 2, 1, seed=21) * h
+    geo = oracle.box_geometry(v, lx)
+    u = synth.uniform(geo["jac"].shape, seed=22) * mag
+    h1 = synth.uniform(geo["jac"].shape, seed=23, lo=0.5, hi=2.0)
+    dx, dxt = oracle.d_buffers(lx)
+    ref = oracle.ax_helm(u, dx, dxt, h1, *[geo[k] for k in GKEYS], lx)
+    scale = np.abs(ref).max()
+    assert 1e-30 < scale < 1e35
+    assert rel_l2(_run(u, h1, v, lx) / scale, ref / scale) <= TOL
