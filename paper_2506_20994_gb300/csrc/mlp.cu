@@ -936,8 +936,12 @@ int mlp_correction(const ax_mlp *M, T *corr, const T *r, const T *minv, const T 
   if (nelv <= 0) return AX_OK;
   const Layout L = layout(M);
   const char *base = reinterpret_cast<const char *>(M->theta_bf);
-  if (M->arch == AX_MLP_SYM && sc && M->n_in % 2 == 0 && (L.HP == 16 || L.HP == 32 ||
-                                                          L.HP == 48 || L.HP == 64)) {
+  // the kernel for pairs of values reads and writes r, sc and corr as pairs: a
+  // caller's r may start between two (ax_precondition passes it on)
+  auto pairs = [](const void *p, size_t size) { return (uintptr_t)p % (2 * size) == 0; };
+  if (M->arch == AX_MLP_SYM && sc && M->n_in % 2 == 0 &&
+      (L.HP == 16 || L.HP == 32 || L.HP == 48 || L.HP == 64) && pairs(r, sizeof(T)) &&
+      pairs(corr, sizeof(T)) && pairs(sc, sizeof(float))) {
     auto w1 = reinterpret_cast<const __nv_bfloat16 *>(base + L.w1t);
     auto w2 = reinterpret_cast<const __nv_bfloat16 *>(base + L.w2t);
     switch (L.HP) {

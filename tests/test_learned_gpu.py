@@ -286,3 +286,25 @@ def test_sym_trained_preconditioner_cuts_iterations():
     r2, bf = P.residual(b2, x2).reshape(-1), b2.reshape(-1)
     c = P.gs.inverse_multiplicity()
     assert float(torch.sum(c * r2 * r2)) <= (1.5e-8) ** 2 * float(torch.sum(c * bf * bf))
+
+
+@pytest.mark.parametrize("arch", [ax.AX_MLP_SYM, ax.AX_MLP_TANH], ids=["sym", "tanh"])
+@pytest.mark.parametrize("lx,n_hid", [(4, 16), (6, 33), (7, 48)])
+def test_precondition_of_a_residual_between_two_pairs(lx, n_hid, arch):
+    """r as a view that starts one value into a buffer (8-byte aligned): the
+    same result as from an aligned copy.  The two forms of the symmetric apply
+    take the same bf16 operands into fp32 sums, so at most the bf16 rounding of
+    a hidden value (2^-8 of it) differs."""
+    P = ax.Poisson(synth.box_vertices(3, 2, 2, seed=lx), lx)
+    n = P.nelv * lx ** 3
+    theta = (_sym_params(lx ** 3, n_hid, seed=lx) if arch == ax.AX_MLP_SYM
+             else _random_params(lx ** 3, n_hid, seed=lx))
+    M = ax.Mlp(lx ** 3, n_hid, params=theta, arch=arch)
+    r = torch.as_tensor(synth.uniform((n,), seed=5), device="cuda")
+    buf = torch.empty(n + 1, dtype=torch.float64, device="cuda")
+    buf[1:] = r
+    assert buf[1:].data_ptr() % 16 == 8 and r.data_ptr() % 16 == 0
+    jac = P.precondition(r, None)
+    corr, corr_v = P.precondition(r, M) - jac, P.precondition(buf[1:], M) - jac
+    assert float(corr.norm()) > 0
+    assert float((corr_v - corr).norm()) <= 2.0 ** -8 * float(corr.norm())
