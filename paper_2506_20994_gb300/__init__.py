@@ -760,7 +760,13 @@ def _poisson_mpfcg(self, b, mlp=None, mode=_lib.AX_PREC_F32, tol=1e-8, inner_tol
 
 
 def _poisson_precondition(self, r, mlp=None):
+    """z = minv .* r (+ the learned correction) for a contiguous fp64 CUDA
+    tensor r of the handle's size (ax_precondition)."""
     import torch
+    if r.dtype != torch.float64 or not r.is_cuda:
+        raise TypeError("precondition needs an fp64 CUDA tensor")
+    if not r.is_contiguous() or r.numel() != int(np.prod(self.shape)):
+        raise ValueError("precondition needs a contiguous tensor of the handle's size")
     z = torch.empty_like(r)
     check("ax_precondition", lib().ax_precondition(self._h, mlp.handle if mlp is not None
                                                    else None, z.data_ptr(), r.data_ptr(),

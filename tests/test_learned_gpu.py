@@ -308,3 +308,17 @@ def test_precondition_of_a_residual_between_two_pairs(lx, n_hid, arch):
     corr, corr_v = P.precondition(r, M) - jac, P.precondition(buf[1:], M) - jac
     assert float(corr.norm()) > 0
     assert float((corr_v - corr).norm()) <= 2.0 ** -8 * float(corr.norm())
+
+
+def test_precondition_refuses_what_it_cannot_read():
+    P = ax.Poisson(synth.box_vertices(2, 2, 2, seed=1), 4)
+    r = torch.zeros(P.nelv * 64, dtype=torch.float64, device="cuda")
+    assert not P.precondition(r.reshape(P.shape)).any()
+    with pytest.raises(TypeError):
+        P.precondition(r.float())
+    with pytest.raises(TypeError):
+        P.precondition(r.cpu())
+    with pytest.raises(ValueError):
+        P.precondition(r[:-1])
+    with pytest.raises(ValueError):
+        P.precondition(r.reshape(2, -1).t())
