@@ -21,6 +21,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "alloc.h"
 #include "common.cuh"
 #include "dispatch.h"
 #include "gs.h"
@@ -620,24 +621,20 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
 
 int ensure_lowp(ax_poisson *P, int mode, cudaStream_t st) {
   if (P->lowp_mode == mode) return AX_OK;
-  if (P->lowp_mode != 0) {  // switch modes: drop the old operator copies
-    cudaFree(P->h1lp);
-    for (auto &q : P->glp) cudaFree(q), q = nullptr;
-    P->h1lp = nullptr;
-  }
-  const int64_t n = P->n;
-  const size_t lx2 = (size_t)P->lx * P->lx;
-  int rc = AX_OK;
-  if (!P->x32) {
-    rc |= alloc(&P->minv32, n) | alloc(&P->mask32, n) | alloc(&P->x32, n) | alloc(&P->r32, n) |
-          alloc(&P->p32, n) | alloc(&P->w32, n) | alloc(&P->q32, n) | alloc(&P->c32, n) |
-          alloc(&P->cm32, n) | alloc(&P->dx32, lx2) | alloc(&P->dxt32, lx2) | alloc(&P->r64, n);
-    if (rc) return AX_ENOMEM;
-  }
-  const size_t es = mode == 2 ? sizeof(__nv_bfloat16) : sizeof(float);
-  if (cudaMalloc(&P->h1lp, n * es) != cudaSuccess) return AX_ENOMEM;
-  for (auto &q : P->glp)
-    if (cudaMalloc(&q, n * es) != cudaSuccess) return AX_ENOMEM;
+  const size_t n = (size_t)P->n, lx2 = (size_t)P->lx * P->lx;
+  if (!P->x32)
+    if (int rc = ax::alloc_all({{&P->minv32, n}, {&P->mask32, n}, {&P->x32, n}, {&P->r32, n},
+                                {&P->p32, n}, {&P->w32, n}, {&P->q32, n}, {&P->c32, n},
+                                {&P->cm32, n}, {&P->dx32, lx2}, {&P->dxt32, lx2}, {&P->r64, n}}))
+      return rc;
+  if (P->hb && !P->hb32 && alloc(&P->hb32, n)) return AX_ENOMEM;
+  // the operator copies, in place of those of another mode
+  P->lowp_mode = 0;
+  const size_t nb_op = n * (mode == 2 ? sizeof(__nv_bfloat16) : sizeof(float));
+  if (int rc = ax::alloc_all({{&P->h1lp, nb_op}, {&P->glp[0], nb_op}, {&P->glp[1], nb_op},
+                              {&P->glp[2], nb_op}, {&P->glp[3], nb_op}, {&P->glp[4], nb_op},
+                              {&P->glp[5], nb_op}}))
+    return rc;
   const unsigned nb = kRedBlocks;
   auto conv = [&](void *out, const double *in, int64_t m) {
     if (mode == 2)
@@ -653,10 +650,8 @@ int ensure_lowp(ax_poisson *P, int mode, cudaStream_t st) {
   to_f32_kernel<<<nb, kRedThreads, 0, st>>>(P->cm32, P->cm, n);
   to_f32_kernel<<<1, 256, 0, st>>>(P->dx32, P->dx, (int64_t)lx2);
   to_f32_kernel<<<1, 256, 0, st>>>(P->dxt32, P->dxt, (int64_t)lx2);
-  if (P->hb) {  // the Helmholtz mass term of the inner operator
-    if (!P->hb32 && alloc(&P->hb32, n)) return AX_ENOMEM;
+  if (P->hb)  // the Helmholtz mass term of the inner operator
     to_f32_kernel<<<nb, kRedThreads, 0, st>>>(P->hb32, P->hb, n);
-  }
   if (ax::launch_status()) return AX_ELAUNCH;
   P->lowp_mode = mode;
   // the even-odd fp32 kernel where it applies (library buffers are aligned),
@@ -1395,8 +1390,8 @@ int ensure_sqm(ax_poisson *P, cudaStream_t st) {
 
 int ensure_fcg64(ax_poisson *P, cudaStream_t st) {
   if (int rc = ensure_sqm(P, st)) return rc;
-  if (P->r_old) return AX_OK;
-  return alloc(&P->r_old, P->n) | alloc(&P->corr, P->n) ? AX_ENOMEM : AX_OK;
+  const size_t n = (size_t)P->n;
+  return P->corr ? AX_OK : ax::alloc_all({{&P->r_old, n}, {&P->corr, n}});
 }
 
 }  // namespace
@@ -1451,9 +1446,10 @@ extern "C" int ax_mpfcg_solve(ax_poisson *P, const ax_mlp *M, int mode, double *
   cudaStream_t st = (cudaStream_t)stream;
   int rc = ensure_lowp(P, mode == AX_PREC_BF16 ? 2 : 1, st);
   if (rc) return rc;
-  if (!P->r_old32 && (alloc(&P->r_old32, P->n) | alloc(&P->corr32, P->n))) return AX_ENOMEM;
-  if ((rc = ensure_sqm(P, st))) return rc;
   const int64_t n = P->n;
+  if (!P->corr32 && (rc = ax::alloc_all({{&P->r_old32, (size_t)n}, {&P->corr32, (size_t)n}})))
+    return rc;
+  if ((rc = ensure_sqm(P, st))) return rc;
   const unsigned nb = kRedBlocks;
   double *sc = reinterpret_cast<double *>(P->scal);
   auto norm_r = [&](double *out_host) -> int {

@@ -21,6 +21,7 @@
 #include <new>
 #include <vector>
 
+#include "alloc.h"
 #include "common.cuh"
 #include "df64.cuh"
 #include "mlp.cuh"
@@ -761,26 +762,13 @@ inline dim3 out_grid(int B, int N) {
 
 int ensure_capacity(ax_mlp *M, int B) {
   if (B <= M->cap) return AX_OK;
-  cudaFree(M->X);
-  cudaFree(M->T);
-  cudaFree(M->H);
-  cudaFree(M->Y);
-  cudaFree(M->dY);
-  cudaFree(M->dP);
-  cudaFree(M->partials);
-  cudaFree(M->es);
   M->cap = 0;
   const size_t bn = (size_t)B * M->n_in, bh = (size_t)B * M->n_hid;
   const dim3 og = out_grid(B, M->n_in);
   const size_t nblk = (size_t)og.x * og.y;
-  if (cudaMalloc(&M->X, bn * 4) != cudaSuccess || cudaMalloc(&M->T, bn * 4) != cudaSuccess ||
-      cudaMalloc(&M->Y, bn * 4) != cudaSuccess || cudaMalloc(&M->dY, bn * 4) != cudaSuccess ||
-      cudaMalloc(&M->H, bh * 4) != cudaSuccess || cudaMalloc(&M->dP, bh * 4) != cudaSuccess ||
-      cudaMalloc(&M->es, (size_t)B * 8) != cudaSuccess ||
-      cudaMalloc(&M->partials, nblk * 8) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return AX_ENOMEM;
-  }
+  if (int rc = ax::alloc_all({{&M->X, bn}, {&M->T, bn}, {&M->Y, bn}, {&M->dY, bn}, {&M->H, bh},
+                              {&M->dP, bh}, {&M->es, (size_t)B}, {&M->partials, nblk}}))
+    return rc;
   M->cap = B;
   return AX_OK;
 }
@@ -892,13 +880,8 @@ namespace ax {
 int mlp_reserve(ax_mlp *M, int B, int pairs) {
   if (int rc = ensure_capacity(M, B)) return rc;
   if (pairs <= M->kcap) return AX_OK;
-  cudaFree(M->ek);
-  M->ek = nullptr;
   M->kcap = 0;
-  if (cudaMalloc(&M->ek, (2 + ax::kRedBlocks) * (size_t)pairs * sizeof(double)) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return AX_ENOMEM;
-  }
+  if (int rc = alloc_all({{&M->ek, (2 + ax::kRedBlocks) * (size_t)pairs}})) return rc;
   M->kcap = pairs;
   return AX_OK;
 }
