@@ -592,7 +592,10 @@ int ax_fcg_solve(ax_poisson *P, const ax_mlp *M, double *x, const double *b, dou
  * Adam (fixed lr) on L_k = ||e_k - z(r_k)||_A^2 / ||e_k||_A^2 with z the
  * preconditioner of ax_precondition, every element one training row, the
  * K pairs visited in order for `epochs` passes.  Writes the mean L_k of the
- * last pass.  Allocates scratch (freed on return); synchronises stream. */
+ * last pass.  Works in P's solver vectors and in a workspace that M grows to
+ * the largest nelv and K it has seen (16 bytes a point and some, 16 bytes a
+ * pair and at most 0.3 MB) and keeps until it is destroyed; synchronises
+ * stream. */
 int ax_mlp_train_energy(ax_poisson *P, ax_mlp *M, const double *r_set, const double *e_set,
                         int K, int epochs, float lr, double *final_loss, void *stream);
 

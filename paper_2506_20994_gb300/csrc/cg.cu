@@ -1648,21 +1648,28 @@ extern "C" int ax_mlp_train_energy(ax_poisson *P, ax_mlp *M, const double *r_set
   const unsigned nb = kRedBlocks;
   const int sym = M->arch == AX_MLP_SYM;
   int rc = ax::mlp_reserve(M, P->nelv, K);
-  if (rc == AX_OK) rc = ensure_fcg64(P, st);
   if (rc) return rc;
-  // scratch: the solvers' own vectors, idle here
-  double *d = P->r, *q = P->w, *isc = P->p, *osc = P->r_old, *corr = P->corr;
-  double *s = M->es, *eA = M->ek, *Lk = M->ek + K, *part = M->ek + 2 * K;
+  // scratch: the solvers' own three vectors, idle here (the correction is read
+  // before q is written), and the network's T and Y, which this loss has not
+  double *d = P->r, *q = P->w, *corr = P->w, *isc = P->p;
+  double *osc = reinterpret_cast<double *>(M->T);
   energy_scales_kernel<<<nb, kRedThreads, 0, st>>>(isc, osc, P->minv, P->mask, P->c, sym, n);
+  double *s = M->es, *eA = M->ek, *Lk = M->ek + K, *part = M->ek + 2 * K;
+  constexpr int kBlk = ax::kEnergyPairs;  // pairs whose partials have a place in `part`
+  // the sums of the pairs whose partials wait, up to pair k
+  auto sums = [&](double *out, int k) {
+    if ((k + 1) % kBlk == 0 || k + 1 == K)
+      pair_sums_kernel<<<k % kBlk + 1, 32, 0, st>>>(part, out + k / kBlk * kBlk);
+  };
   // ||e_k||_A^2 once per pair
   for (int k = 0; k < K && rc == AX_OK; ++k) {
     const double *e = e_set + (size_t)k * n;
     rc = apply_f64(P, q, e, st);
     if (rc) break;
     rc = ax::launch_chained(true, mask_dot_kernel<double>, nb, kRedThreads, 0, st, q, e, P->mask,
-                            P->c, part + (size_t)k * nb, n, (CgScalars *)nullptr);
+                            P->c, part + (size_t)(k % kBlk) * nb, n, (CgScalars *)nullptr);
+    sums(eA, k);
   }
-  pair_sums_kernel<<<K, 32, 0, st>>>(part, eA);
   for (int ep = 0; ep < epochs && rc == AX_OK; ++ep) {
     for (int k = 0; k < K && rc == AX_OK; ++k) {
       const double *r = r_set + (size_t)k * n, *e = e_set + (size_t)k * n;
@@ -1677,13 +1684,13 @@ extern "C" int ax_mlp_train_energy(ax_poisson *P, ax_mlp *M, const double *r_set
       if ((rc = apply_f64(P, q, d, st))) break;
       if ((rc = ax::launch_chained(true, energy_dot_dy_kernel, nb, kRedThreads, 0, st, M->dY, q, d,
                                    P->mask, P->c, osc, s, eA + k, N, P->nelv,
-                                   part + (size_t)k * nb)))
+                                   part + (size_t)(k % kBlk) * nb)))
         break;
+      if (ep + 1 == epochs) sums(Lk, k);  // the last epoch's losses
       if ((rc = ax::mlp_train_backward(M, P->nelv, st))) break;
       if ((rc = ax::mlp_adam_step(M, lr, st))) break;
     }
   }
-  pair_sums_kernel<<<K, 32, 0, st>>>(part, Lk);  // the last epoch's losses
   if (rc == AX_OK) rc = ax::mlp_refresh(M, st);
   std::vector<double> hl(K), he(K);
   if (rc == AX_OK &&

@@ -766,9 +766,11 @@ int ensure_capacity(ax_mlp *M, int B) {
   const size_t bn = (size_t)B * M->n_in, bh = (size_t)B * M->n_hid;
   const dim3 og = out_grid(B, M->n_in);
   const size_t nblk = (size_t)og.x * og.y;
-  if (int rc = ax::alloc_all({{&M->X, bn}, {&M->T, bn}, {&M->Y, bn}, {&M->dY, bn}, {&M->H, bh},
+  M->Y = nullptr;
+  if (int rc = ax::alloc_all({{&M->X, bn}, {&M->T, 2 * bn}, {&M->dY, bn}, {&M->H, bh},
                               {&M->dP, bh}, {&M->es, (size_t)B}, {&M->partials, nblk}}))
     return rc;
+  M->Y = M->T + bn;
   M->cap = B;
   return AX_OK;
 }
@@ -881,7 +883,9 @@ int mlp_reserve(ax_mlp *M, int B, int pairs) {
   if (int rc = ensure_capacity(M, B)) return rc;
   if (pairs <= M->kcap) return AX_OK;
   M->kcap = 0;
-  if (int rc = alloc_all({{&M->ek, (2 + ax::kRedBlocks) * (size_t)pairs}})) return rc;
+  if (int rc = alloc_all({{&M->ek, 2 * (size_t)pairs +
+                                       (size_t)std::min(pairs, kEnergyPairs) * kRedBlocks}}))
+    return rc;
   M->kcap = pairs;
   return AX_OK;
 }
@@ -964,7 +968,7 @@ extern "C" {
 
 int ax_mlp_destroy(ax_mlp *M) {
   if (!M) return AX_OK;
-  float *f[] = {M->theta, M->grad, M->m, M->v, M->X, M->T, M->H, M->Y, M->dY, M->dP};
+  float *f[] = {M->theta, M->grad, M->m, M->v, M->X, M->T, M->H, M->dY, M->dP};
   for (float *p : f) cudaFree(p);
   cudaFree(M->theta_bf);
   cudaFree(M->partials);

@@ -17,10 +17,12 @@ struct ax_mlp {
   int adam_step = 0;
   // training workspace for batches up to cap samples
   int cap = 0;
-  float *X = nullptr, *T = nullptr, *H = nullptr, *Y = nullptr, *dY = nullptr, *dP = nullptr;
+  float *X = nullptr, *T = nullptr, *H = nullptr, *dY = nullptr, *dP = nullptr;
+  float *Y = nullptr;  // behind T, in its allocation
   double *partials = nullptr;
   double *es = nullptr;  // energy training: each row's scale s_e (cap of them)
-  double *ek = nullptr;  // energy training, kcap pairs: ||e||_A^2, losses, their partials
+  double *ek = nullptr;  // energy training, kcap pairs: ||e||_A^2, losses, and the
+                         // partials of up to kEnergyPairs of them
   int kcap = 0;
   double *loss_dev = nullptr;
 };
@@ -31,6 +33,10 @@ namespace ax {
 inline int64_t mlp_off_b1(const ax_mlp *M) { return (int64_t)M->n_in * M->n_hid; }
 inline int64_t mlp_off_w2(const ax_mlp *M) { return mlp_off_b1(M) + M->n_hid; }
 inline int64_t mlp_off_b2(const ax_mlp *M) { return mlp_off_w2(M) + (int64_t)M->n_hid * M->n_in; }
+
+// Pairs of the energy training whose partial sums wait to be added (4.9 KB
+// each; more pairs than this are added in runs of it).
+constexpr int kEnergyPairs = 64;
 
 // Training internals (fp32, on the workspace of ax_mlp):
 int mlp_reserve(ax_mlp *M, int B, int pairs);               // workspace for B rows

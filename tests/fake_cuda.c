@@ -9,11 +9,17 @@
 typedef struct { unsigned x, y, z; } dim3_t;
 enum { MAXP = 4096 };
 static void *live[MAXP];
+static size_t size[MAXP];
 static int fail_in, bad_frees, launches, query_result;
 
 int fake_live(void) {
   int n = 0;
   for (int k = 0; k < MAXP; ++k) n += live[k] != NULL;
+  return n;
+}
+long long fake_bytes(void) {
+  long long n = 0;
+  for (int k = 0; k < MAXP; ++k) n += live[k] ? (long long)size[k] : 0;
   return n;
 }
 void fake_fail_in(int n) { fail_in = n; } /* the n-th allocation from now on; 0: none */
@@ -26,6 +32,7 @@ int cudaMalloc(void **p, size_t n) {
   if (fail_in > 0 && --fail_in == 0) return 2;
   for (int k = 0; k < MAXP; ++k)
     if (!live[k]) {
+      size[k] = n;
       *p = live[k] = calloc(n + 256, 1);
       return 0;
     }

@@ -30,6 +30,12 @@ def test_failed_allocation_is_made_up_for(fake, what):
     assert r.returncode == 0, r.stdout + r.stderr
 
 
+def test_training_holds_no_more_than_its_workspace(fake):
+    """Energy training leaves nothing in the problem's handle, and past the 64
+    places of 608 partial sums its workspace grows by 16 bytes a pair."""
+    test_failed_allocation_is_made_up_for(fake, "held")
+
+
 # ------------------------------------------------ in the process with the fake
 def _program(fake, what):
     import paper_2506_20994_gb300 as ax
@@ -51,14 +57,32 @@ def _program(fake, what):
     def ok(rc):
         assert rc == 0, rc
 
-    def session(call, fail):
-        """All handles made, `call` with its `fail`-th allocation failing (0:
-        none), called again; returns the allocations held then."""
+    def handles():
         gs, P, M = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
         ok(L.ax_gs_setup(ref(gs), glob, n, None))
         ok(L.ax_poisson_create(ref(P), lx, nel, a(dx), a(dxt), one, *geom, one, gs, None))
         ok(L.ax_mlp_create_ex(ref(M), lx ** 3, 16, ax.AX_MLP_SYM))
         ok(L.ax_mlp_set_params(M, params, par.size, None))
+        return gs, P, M
+
+    if what == "held":
+        F.fake_bytes.restype = ctypes.c_longlong
+        gs, P, M = handles()
+        own = F.fake_bytes()
+        held = {}
+        for K in (1, 64, 1000):
+            ok(L.ax_mlp_train_energy(P, M, out, out, K, 1, 1e-3, ref(num), None))
+            held[K] = F.fake_bytes() - own
+        assert held[1000] - held[64] == 16 * (1000 - 64), held
+        ok(L.ax_mlp_destroy(M))
+        ok(L.ax_mlp_create_ex(ref(M), lx ** 3, 16, ax.AX_MLP_SYM))
+        assert F.fake_bytes() == own, (F.fake_bytes(), own)
+        return
+
+    def session(call, fail):
+        """All handles made, `call` with its `fail`-th allocation failing (0:
+        none), called again; returns the allocations held then."""
+        gs, P, M = handles()
         F.fake_fail_in(fail)
         rc = call(P, M)
         hit = fail > 0 and F.fake_pending() == 0
