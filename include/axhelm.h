@@ -334,7 +334,13 @@ int ax_jacobi_noalloc(double *minv, const double *dx, const double *h1, const do
 /* Jacobi-preconditioned CG in fp64 from x0 = 0 until ||r|| <= tol ||b||
  * (b is masked first).  Writes the iteration count and the final relative
  * residual.  Synchronises stream.  Returns AX_OK, AX_ENOTCONV (maxit
- * reached), AX_EBREAKDOWN (p.Ap <= 0 or non-finite) or AX_EINVAL. */
+ * reached), AX_EBREAKDOWN (p.Ap <= 0 or non-finite), AX_EINVAL, or AX_ELAUNCH
+ * (a launch failed, the stream reports an error or cannot run, as under
+ * capture).  The host waits for each convergence test as the device's flags
+ * say (cudaSetDeviceFlags): by default it polls, one core busy; with
+ * cudaDeviceScheduleYield it gives up its time slice while it polls; with
+ * cudaDeviceScheduleBlockingSync it sleeps.  The same holds for the other
+ * solvers. */
 int ax_cg_solve(ax_poisson *P, double *x, const double *b, double tol, int maxit, int *iters,
                 double *relres, void *stream);
 

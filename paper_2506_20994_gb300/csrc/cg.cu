@@ -13,6 +13,8 @@
 // nodes).  Inner products run over unique global nodes, i.e. the local sum
 // weighted by 1/multiplicity.  The scalars of the iteration live on the
 // device; the host reads the residual norm every `check_every` iterations.
+#include <sched.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
@@ -512,10 +514,22 @@ int apply_fused_update(ax_poisson *P, float *w, float *p, const float *r, const 
 // Asks the next reduction that forms rr for its values (address and number)
 ax::CgMailTo next_mail(ax_poisson *P) { return ax::CgMailTo{P->mail, ++P->mail_seq}; }
 // Waits for the values last asked for; AX_ELAUNCH if the stream failed or ran
-// dry without them.
+// dry without them.  The host waits as the process asked the runtime to
+// (cudaSetDeviceFlags): by polling, by polling and giving up its time slice, or
+// asleep until the stream is done, which then includes the half iteration
+// launched meanwhile.
 int wait_mail(const ax_poisson *P, cudaStream_t st) {
   auto here = [P] { return __atomic_load_n(&P->mail->seq, __ATOMIC_ACQUIRE) == P->mail_seq; };
+  unsigned flags = 0u;
+  if (cudaGetDeviceFlags(&flags) != cudaSuccess) (void)cudaGetLastError();
+  flags &= cudaDeviceScheduleMask;
+  if (flags == cudaDeviceScheduleBlockingSync) {
+    if (cudaStreamSynchronize(st) == cudaSuccess && here()) return AX_OK;
+    (void)cudaGetLastError();
+    return AX_ELAUNCH;
+  }
   for (unsigned spin = 1; !here(); ++spin) {
+    if (flags == cudaDeviceScheduleYield && spin % 64 == 0) sched_yield();
     if (spin % 16384) continue;
     const cudaError_t e = cudaStreamQuery(st);
     if (e == cudaErrorNotReady) {

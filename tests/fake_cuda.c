@@ -10,7 +10,8 @@ typedef struct { unsigned x, y, z; } dim3_t;
 enum { MAXP = 4096 };
 static void *live[MAXP];
 static size_t size[MAXP];
-static int fail_in, bad_frees, launches, query_result;
+static int fail_in, bad_frees, launches, query_result, queries, syncs;
+static unsigned flags;
 
 int fake_live(void) {
   int n = 0;
@@ -26,7 +27,10 @@ void fake_fail_in(int n) { fail_in = n; } /* the n-th allocation from now on; 0:
 int fake_pending(void) { return fail_in; }
 int fake_bad_frees(void) { return bad_frees; }
 int fake_launches(void) { return launches; }
-void fake_query(int rc) { query_result = rc; }
+/* what a stream query returns from now on, and the device's flags */
+void fake_stream(int rc, unsigned f) { query_result = rc; flags = f; queries = syncs = 0; }
+int fake_queries(void) { return queries; }
+int fake_syncs(void) { return syncs; }
 
 int cudaMalloc(void **p, size_t n) {
   if (fail_in > 0 && --fail_in == 0) return 2;
@@ -57,12 +61,12 @@ int cudaMemcpyAsync(void *d, const void *s, size_t n, int k, void *st) {
 }
 int cudaMemset(void *d, int v, size_t n) { memset(d, v, n); return 0; }
 int cudaMemsetAsync(void *d, int v, size_t n, void *st) { (void)st; memset(d, v, n); return 0; }
-int cudaStreamSynchronize(void *st) { (void)st; return 0; }
-int cudaStreamQuery(void *st) { (void)st; return query_result; }
+int cudaStreamSynchronize(void *st) { (void)st; ++syncs; return 0; }
+int cudaStreamQuery(void *st) { (void)st; ++queries; return query_result; }
 int cudaGetLastError(void) { return 0; }
 int cudaPeekAtLastError(void) { return 0; }
 int cudaGetDevice(int *d) { *d = 0; return 0; }
-int cudaGetDeviceFlags(unsigned *f) { *f = 0; return 0; }
+int cudaGetDeviceFlags(unsigned *f) { *f = flags; return 0; }
 int cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
 int cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int b, size_t s,

@@ -1,7 +1,9 @@
-"""Allocations that fail half-way through a group, on the library's host side
-(a fake runtime over host memory, no GPU): the call returns AX_ENOMEM, the next
-one allocates whatever is missing instead of using it, nothing is freed twice
-and nothing is left when the handles are gone."""
+"""The library's host side under a fake runtime over host memory, no GPU.
+
+Allocations that fail half-way through a group: the call returns AX_ENOMEM, the
+next one allocates whatever is missing instead of using it, nothing is freed
+twice and nothing is left when the handles are gone.  Solves whose kernels
+never report: they return AX_ELAUNCH, waiting the way the process asked for."""
 import ctypes
 import os
 import subprocess
@@ -34,6 +36,13 @@ def test_training_holds_no_more_than_its_workspace(fake):
     """Energy training leaves nothing in the problem's handle, and past the 64
     places of 608 partial sums its workspace grows by 16 bytes a pair."""
     test_failed_allocation_is_made_up_for(fake, "held")
+
+
+def test_wait_for_a_stream_that_fails_or_runs_dry(fake):
+    """The convergence test's values never come: AX_ELAUNCH from every solver
+    once the stream is idle or reports an error; and a process that asked for
+    blocking synchronisation gets it instead of polling."""
+    test_failed_allocation_is_made_up_for(fake, "wait")
 
 
 # ------------------------------------------------ in the process with the fake
@@ -77,6 +86,21 @@ def _program(fake, what):
         ok(L.ax_mlp_destroy(M))
         ok(L.ax_mlp_create_ex(ref(M), lx ** 3, 16, ax.AX_MLP_SYM))
         assert F.fake_bytes() == own, (F.fake_bytes(), own)
+        return
+
+    if what == "wait":
+        gs, P, M = handles()
+        solves = [lambda: L.ax_cg_solve(P, out, b, 1e-8, 9, None, None, None),
+                  lambda: L.ax_fcg_solve(P, M, out, b, 1e-8, 9, None, None, None, None)]
+        for solve in solves:
+            for result in (0, 700):  # idle; an earlier kernel's fault, as reported
+                for flags in (0, 1, 2):  # automatic, spin, yield
+                    F.fake_stream(result, flags)
+                    assert solve() == _lib.AX_ELAUNCH
+                    assert F.fake_queries() == 1
+            F.fake_stream(0, 4)  # blocking: asked only once it has waited
+            assert solve() == _lib.AX_ELAUNCH
+            assert F.fake_queries() == 0 and F.fake_syncs() >= 1
         return
 
     def session(call, fail):
