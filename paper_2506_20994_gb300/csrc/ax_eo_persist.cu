@@ -79,12 +79,12 @@ int eop_launch_t(const EopArgs &a, cudaStream_t st) {
       const int gh = eop_grid<LX, false, false, true>();
       if (gh <= 0) return AX_ELAUNCH;
       const unsigned nb = (unsigned)std::min<long long>(gh, std::max(a.nelv, 1));
-      return launch_chained(a.chained, eop::ax_eop_kernel<LX, false, false, false, true>, nb,
+      return launch_chained(true, eop::ax_eop_kernel<LX, false, false, false, true>, nb,
                             C::NTB, C::SMEM, st, m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr,
                             a.alpha);
     }
   }
-  return launch_chained(a.chained, eop::ax_eop_kernel<LX, DOT, PUPD>, grid, C::NTB, C::SMEM, st,
+  return launch_chained(true, eop::ax_eop_kernel<LX, DOT, PUPD>, grid, C::NTB, C::SMEM, st,
                         m, (long long)a.nelv, a.err, a.dotp, up, a.beta, a.use_corr, a.alpha);
 }
 
@@ -138,6 +138,9 @@ int eop_blocks_lx(int nelv, bool dot) {
   return std::min(g, std::max(nelv, 1));
 }
 
+// An apply chained behind the last of these kernels reads gp in front of its
+// wait: gp is written by the first one, and each begins when the one before it
+// has finished.  (The ranges, the last one's, are read behind the wait.)
 template <int LX>
 int eop_prepare_lx(df::dd2 *gp, const guard::RawGeo &r, int nelv, int fmask, int dfield,
                    cudaStream_t st) {

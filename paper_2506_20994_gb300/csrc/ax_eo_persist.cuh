@@ -440,7 +440,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     const EopMesh &M = seq.mesh(cmesh);
     const size_t eb = (size_t)seq.elem(pos) * N3;
     // this element's admissible exponent fields of u (guard.cuh, u_range)
-    const uint2 ur_e = RAW ? make_uint2(0u, 0u) : __ldg(M.urange + seq.elem(pos));
+    const uint2 ur_e = RAW ? make_uint2(0u, 0u) : __ldcg(M.urange + seq.elem(pos));
     // ---- phase 1: this element's u (or the direction formed here), split,
     // lines of the three directions; the next element's inputs start loading
     double ucur[2][2];

@@ -123,10 +123,6 @@ struct EopArgs {
   const double *r = nullptr, *minv = nullptr, *beta = nullptr, *corr = nullptr;
   const double *alpha = nullptr;
   const int *use_corr = nullptr;
-  // The launch may begin before the kernel in front of it is done; the handle's
-  // prepared geometry and coefficients are read at once, so the launch that
-  // follows their (re)writing must not be chained.
-  bool chained = false;
   const double *hb = nullptr;  // plain apply: w += hb .* u (the Helmholtz mass term)
   long long drop = -1;  // testing aid: element whose geometry copy is not issued
 };

@@ -21,10 +21,6 @@ struct ax_op {
   int *err = nullptr;           // device word: a staged copy never arrived (owned)
   int dfield = 0;               // exponent field of the matrices' largest entry
   double *hb = nullptr;         // h2 .* B of the Helmholtz form (owned), or null
-  // the prepared geometry was rewritten on this stream and no apply has
-  // followed there yet
-  bool rewritten = false;
-  cudaStream_t rewritten_on = nullptr;
   long long drop = -1;          // testing aid (ax_op_inject_copy_loss)
 };
 
@@ -43,10 +39,8 @@ namespace {
 // the fastest fp64 form for these orders
 bool op_prepares(int lx) { return ax::eop_supported(lx); }
 
-ax::EopArgs eop_args(ax_op *op, double *w, const double *u, cudaStream_t st) {
+ax::EopArgs eop_args(const ax_op *op, double *w, const double *u) {
   ax::EopArgs a;
-  a.chained = !op->rewritten;
-  if (st == op->rewritten_on) op->rewritten = false;
   a.w = w;
   a.u = u;
   a.coef = op->coef;
@@ -138,8 +132,6 @@ extern "C" int ax_op_set_h1(ax_op *op, const double *h1, void *stream) {
   if (!op || !h1) return AX_EINVAL;
   op->h1 = h1;
   if (!op->gp) return AX_OK;
-  op->rewritten = true;
-  op->rewritten_on = (cudaStream_t)stream;
   const double *const *g = op->g;
   return ax::eop_prepare(op->lx, op->gp, ax::guard::RawGeo{h1, g[0], g[1], g[2], g[3], g[4], g[5]},
                          op->nelv, 0x40, op->dfield, (cudaStream_t)stream);
@@ -168,13 +160,13 @@ extern "C" int ax_op_apply(ax_op *op, double *w, const double *u, void *stream) 
   if (!op || (op->nelv > 0 && (!w || !u))) return AX_EINVAL;
   if (op->nelv == 0) return AX_OK;
   if (op->gp && op->drop < 0) {  // one kernel, with the mass term where there is one
-    ax::EopArgs a = eop_args(op, w, u, (cudaStream_t)stream);
+    ax::EopArgs a = eop_args(op, w, u);
     a.hb = op->hb;
     return ax::eop_launch(op->lx, a, (cudaStream_t)stream);
   }
   int rc;
   if (op->gp) {
-    rc = ax::eop_launch(op->lx, eop_args(op, w, u, (cudaStream_t)stream), (cudaStream_t)stream);
+    rc = ax::eop_launch(op->lx, eop_args(op, w, u), (cudaStream_t)stream);
   } else {
     const double *const *g = op->g;
     rc = ax_helm(w, u, op->dx, op->dxt, op->h1, g[0], g[1], g[2], g[3], g[4], g[5], op->lx,
@@ -193,7 +185,7 @@ int op_dot_blocks(const ax_op *op) {
 
 int op_apply_dot(ax_op *op, double *w, const double *u, double *partials, cudaStream_t st) {
   if (!op || !op->gp || !partials) return AX_EINVAL;
-  EopArgs a = eop_args(op, w, u, st);
+  EopArgs a = eop_args(op, w, u);
   a.dotp = partials;
   return eop_launch(op->lx, a, st);
 }
@@ -203,7 +195,7 @@ int op_update_apply_dot(ax_op *op, double *w, const OpUpdate &up, double *partia
   if (!op || !op->gp || !partials || !up.p || !up.r || !up.minv || !up.beta ||
       (up.x && !up.alpha))
     return AX_EINVAL;
-  EopArgs a = eop_args(op, w, nullptr, st);
+  EopArgs a = eop_args(op, w, nullptr);
   a.dotp = partials;
   a.pw = up.p;
   a.r = up.r;

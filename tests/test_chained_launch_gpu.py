@@ -182,3 +182,122 @@ def test_mixed_solves_and_training_repeat_bitwise():
         ax.train_energy(P, N, R, E, epochs=4)
         got.append(N.get_params())
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
+
+
+def test_rewrite_then_capture_then_eager_apply():
+    """An apply that is only recorded between the rewrite of the geometry and
+    the apply that follows it on the stream."""
+    lx = 8
+    c = operator_case((9, 8, 7), lx, seed=613)
+    d = _scale(c)
+    op = ax.Operator(lx, d["dx"], d["dxt"], d["h1"], *[d[k] for k in GKEYS])
+    h = [d["h1"], (d["h1"] * 1.25).contiguous()]
+    ref = []
+    for q in (0, 1):
+        op.set_h1(h[q])
+        torch.cuda.synchronize()
+        ref.append(torch.empty_like(d["u"]))
+        op.apply(ref[q], d["u"])
+        torch.cuda.synchronize()
+    w, a = torch.empty_like(d["u"]), torch.empty_like(d["u"])
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        for k in range(20):
+            op.set_h1(h[k % 2])
+            g = torch.cuda.CUDAGraph()
+            g.capture_begin(capture_error_mode="relaxed")  # (the context manager synchronises)
+            op.apply(a, d["u"])
+            g.capture_end()
+            op.apply(w, d["u"])
+            s.synchronize()
+            assert torch.equal(w, ref[k % 2])
+            g.replay()
+            s.synchronize()
+            assert torch.equal(a, ref[k % 2])
+
+
+def test_one_handle_on_two_streams_and_threads():
+    """Applies of one handle from two host threads, each on its own stream,
+    between rewrites of its geometry that both wait for."""
+    import threading
+    lx = 8
+    c = operator_case((6, 5, 4), lx, seed=614)
+    d = _scale(c)
+    op = ax.Operator(lx, d["dx"], d["dxt"], d["h1"], *[d[k] for k in GKEYS])
+    gate, errors = threading.Barrier(2, timeout=60), []
+
+    def work(t):
+        try:
+            s = torch.cuda.Stream()
+            u = (d["u"] * (1.0 + t)).contiguous()
+            a, b = torch.empty_like(u), torch.empty_like(u)
+            torch.cuda.synchronize()
+            with torch.cuda.stream(s):
+                for k in range(10):
+                    gate.wait()
+                    if k % 2 == t:  # this thread rewrites, both wait for it
+                        op.set_h1((d["h1"] * (1.0 + 0.1 * k)).contiguous())
+                        s.synchronize()
+                    gate.wait()
+                    op.apply(a, u)
+                    op.apply(b, a)
+                    got = b.clone()
+                    s.synchronize()
+                    op.apply(a, u)
+                    s.synchronize()
+                    op.apply(b, a)
+                    s.synchronize()
+                    if not torch.equal(got, b):
+                        errors.append((t, k))
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+            gate.abort()
+    th = [threading.Thread(target=work, args=(t,)) for t in (0, 1)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not errors
+
+
+def test_chains_that_fork_and_join_under_capture():
+    """A recorded chain whose links come from another stream's event, a copy
+    and a memset as well as from the kernel in front."""
+    lx = 8
+    c = operator_case((6, 5, 4), lx, seed=615)
+    d = _scale(c)
+    op = ax.Operator(lx, d["dx"], d["dxt"], d["h1"], *[d[k] for k in GKEYS])
+    u = d["u"]
+    a, b, x, y = (torch.zeros_like(u) for _ in range(4))
+
+    def chain(s, t):
+        with torch.cuda.stream(s):
+            op.apply(a, u)
+        t.wait_stream(s)
+        with torch.cuda.stream(t):  # first on t: its link is the event
+            op.apply(b, a)
+            x.copy_(b)
+            op.apply(y, x)
+        with torch.cuda.stream(s):
+            x2 = a * 2.0
+            s.wait_stream(t)  # two links: the kernel on s and the event of t
+            op.apply(a, y)
+            a.add_(x2)
+            b.zero_()
+            op.apply(x, a)
+            return x
+    s, t = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ref = chain(s, t)
+    torch.cuda.synchronize()
+    ref = ref.clone()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        chain(s, t)
+    for _ in range(5):
+        x.zero_()
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(x, ref)
