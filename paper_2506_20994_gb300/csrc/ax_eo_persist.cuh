@@ -641,7 +641,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
 #pragma unroll
             for (int a = 0; a < 2; ++a) {
               const size_t q = eb + pidx(b, a);
-              M.w[q] = __fma_rn(hv[b][a], ucur[b][a], M.w[q]);
+              M.w[q] = __fma_rn(hv[b][a], ucur[b][a], __ldcg(M.w + q));
             }
         }
       }

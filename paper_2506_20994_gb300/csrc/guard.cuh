@@ -141,9 +141,9 @@ AX_D bool elem_ok(const Record &r, int le) {
 // w_e = D^T (h1 G (D u_e)) of one element with fp64 units, in the loop order
 // of Listing 2 (reference gradient, pointwise h1 G, transposed sum).  Run by
 // the `nt` threads of the element (rank `r`); `sync()` synchronises at least
-// those threads.  `scr` holds 3 lx^3 doubles of shared memory.  u is read with
-// coherent loads (a solver kernel may have written it earlier in the same
-// launch).  dot (optional): adds this thread's share of u . w.  Threads with
+// those threads.  `scr` holds 3 lx^3 doubles of shared memory.  u is read past
+// L1 (the kernel in front of a chained launch may have written it, or the
+// caller earlier in the same one).  dot (optional): adds this thread's share of u . w.  Threads with
 // `on` false only take part in the two barriers.
 template <int LX, class Sync>
 __device__ __noinline__ void element_f64(bool on, double *__restrict__ w, const double *u, const double *__restrict__ dx,
@@ -161,9 +161,9 @@ __device__ __noinline__ void element_f64(bool on, double *__restrict__ w, const 
     double ur = 0.0, us = 0.0, ut = 0.0;
 #pragma unroll 4
     for (int l = 0; l < LX; ++l) {
-      ur = __fma_rn(__ldcg(dx + l * LX + i), u[eb + (k * LX + j) * LX + l], ur);
-      us = __fma_rn(__ldcg(dy + l * LX + j), u[eb + (k * LX + l) * LX + i], us);
-      ut = __fma_rn(__ldcg(dz + l * LX + k), u[eb + (l * LX + j) * LX + i], ut);
+      ur = __fma_rn(__ldcg(dx + l * LX + i), __ldcg(u + eb + (k * LX + j) * LX + l), ur);
+      us = __fma_rn(__ldcg(dy + l * LX + j), __ldcg(u + eb + (k * LX + l) * LX + i), us);
+      ut = __fma_rn(__ldcg(dz + l * LX + k), __ldcg(u + eb + (l * LX + j) * LX + i), ut);
     }
     const size_t q = eb + p;
     const double a11 = __ldcg(g11 + q), a22 = __ldcg(g22 + q), a33 = __ldcg(g33 + q);
@@ -184,7 +184,7 @@ __device__ __noinline__ void element_f64(bool on, double *__restrict__ w, const 
       acc = __fma_rn(__ldcg(dzt + l * LX + k), st[(l * LX + j) * LX + i], acc);
     }
     w[eb + p] = acc;
-    if (dot) *dot = __fma_rn(u[eb + p], acc, *dot);
+    if (dot) *dot = __fma_rn(__ldcg(u + eb + p), acc, *dot);
   }
   sync();  // the scratch is reused by the caller
 }

@@ -301,3 +301,28 @@ def test_chains_that_fork_and_join_under_capture():
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(x, ref)
+
+
+@pytest.mark.parametrize("lx", [6, 7, 8])
+def test_chains_of_elements_in_fp64_units(lx):
+    """Every element outside the double-float window (recomputed with fp64
+    units), with the mass term, in vectors that start between two sectors, so
+    that neighbouring elements share one."""
+    c = operator_case((9, 8, 7), lx, seed=650 + lx)
+    d = _scale(c)
+    G = [d[k] for k in GKEYS]
+    op = ax.Operator(lx, d["dx"], d["dxt"], d["h1"], *G)
+    h2 = torch.full_like(d["u"], 0.1)
+    op.set_h2(h2, torch.ones_like(h2))
+    n = d["u"].numel()
+    raw = [torch.zeros(n + 1, dtype=torch.float64, device="cuda") for _ in range(3)]
+    raw[0][1:] = d["u"].reshape(-1) * 1e-60
+
+    def step(w, u, k):
+        op.apply(w[1:], u[1:])
+    _same(step, raw)
+
+    def step_raw(w, u, k):
+        ax.ax_helm(w[1:].view(d["u"].shape), u[1:].view(d["u"].shape), d["dx"], d["dxt"], d["h1"],
+                   *G, lx)
+    _same(step_raw, raw)
