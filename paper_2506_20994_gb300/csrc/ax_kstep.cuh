@@ -101,18 +101,19 @@ __device__ __forceinline__ void kstep_body(W *__restrict__ w, const SU *__restri
 
   for (int t = threadIdx.x; VEC && t < N2; t += blockDim.x) {
     const int a = t / LX, b = t % LX;
-    Fd[b * RS + a] = dx[t];
-    Bd[b * RS + a] = dxt[t];
-    Td[a * RS + b] = dxt[t];
+    const T f = __ldcg(dx + t), g = __ldcg(dxt + t);
+    Fd[b * RS + a] = f;
+    Bd[b * RS + a] = g;
+    Td[a * RS + b] = g;
   }
   for (int t = threadIdx.x; !VEC && t < N2; t += blockDim.x) {
-    sdx[t] = dx[t];
-    sdxt[t] = dxt[t];
+    sdx[t] = __ldcg(dx + t);
+    sdxt[t] = __ldcg(dxt + t);
     if constexpr (XYZ) {
-      sdy[t] = dy[t];
-      sdz[t] = dz[t];
-      sdyt[t] = dyt[t];
-      sdzt[t] = dzt[t];
+      sdy[t] = __ldcg(dy + t);
+      sdz[t] = __ldcg(dz + t);
+      sdyt[t] = __ldcg(dyt + t);
+      sdzt[t] = __ldcg(dzt + t);
     }
   }
   const bool active = own && le < nel;

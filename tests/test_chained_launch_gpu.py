@@ -326,3 +326,40 @@ def test_chains_of_elements_in_fp64_units(lx):
         ax.ax_helm(w[1:].view(d["u"].shape), u[1:].view(d["u"].shape), d["dx"], d["dxt"], d["h1"],
                    *G, lx)
     _same(step_raw, raw)
+
+
+@pytest.mark.parametrize("lx", [3, 4, 5, 7, 8, 13])
+def test_matrices_written_by_the_kernel_in_front(lx):
+    """The 1-D matrices rewritten between two applies by a library kernel
+    chained in front of the second (a gather-scatter that doubles every entry
+    it pairs up)."""
+    c = operator_case((9, 8, 7) if lx < 9 else (3, 3, 2), lx, seed=660 + lx)
+    f = torch.float32
+    d = _scale(c, f)
+    G = [d[k] for k in GKEYS]
+    ids = np.arange(lx * lx) // 2  # pairs of neighbouring entries share an id
+    gs = ax.GatherScatter(ids)
+    dx0, dxt0 = _t(c["dx"], f).reshape(-1), _t(c["dxt"], f).reshape(-1)
+
+    def chain(wait):
+        dx, dxt, out = dx0.clone(), dxt0.clone(), []
+        torch.cuda.synchronize()
+        for _ in range(6):
+            w = torch.empty_like(d["u"])
+            ax.ax_helm_f32(w, d["u"], dx, dxt, d["h1"], *G, lx)
+            if wait:
+                torch.cuda.synchronize()
+            gs.sum(dx)
+            if wait:
+                torch.cuda.synchronize()
+            gs.sum(dxt)
+            if wait:
+                torch.cuda.synchronize()
+            out.append(w)
+        torch.cuda.synchronize()
+        return out
+    ref = chain(True)
+    assert not torch.equal(ref[0], ref[1])
+    for _ in range(5):
+        for a, b in zip(chain(False), ref):
+            assert torch.equal(a, b)
