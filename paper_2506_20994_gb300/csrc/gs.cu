@@ -41,13 +41,16 @@ constexpr int kGsThreads = 256;
 // Block 0 of a launch with an alpha job: the partials in the order of a
 // 1024-thread block (virtual thread t adds t, t + 1024, ...; shuffle tree per
 // 32; the 32 sums in order), four virtual threads to each of this block's.
-__device__ __noinline__ void alpha_block(const ax::AlphaJob &job) {
+// (Not inlined, and its arguments by value: by reference they made a stack
+// frame that every thread of the kernel filled, 67 instead of 58 us at 26^3
+// elements, lx 10.)
+__device__ __noinline__ void alpha_block(const double *partials, int n, ax::CgScalars *s) {
   __shared__ double sh[32];
 #pragma unroll
   for (int v = 0; v < 1024 / kGsThreads; ++v) {
     const int vt = (int)threadIdx.x + v * kGsThreads;
     double a = 0.0;
-    for (int b = vt; b < job.n; b += 1024) a += __ldcg(job.partials + b);
+    for (int b = vt; b < n; b += 1024) a += __ldcg(partials + b);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
     if ((vt & 31) == 0) sh[vt >> 5] = a;
@@ -56,7 +59,7 @@ __device__ __noinline__ void alpha_block(const ax::AlphaJob &job) {
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int k = 0; k < 32; ++k) t += sh[k];
-    ax::cg_set_alpha(job.s, t);
+    ax::cg_set_alpha(s, t);
   }
 }
 
@@ -72,7 +75,7 @@ __global__ void gs_sum_kernel(T *__restrict__ v, const int2 *__restrict__ pairs,
   ax::grid_wait();
   ax::grid_go();
   if (ALPHA && blockIdx.x == 0) {
-    alpha_block(job);
+    alpha_block(job.partials, job.n, job.s);
     return;
   }
   const int64_t s = (int64_t)(blockIdx.x - (ALPHA ? 1 : 0)) * blockDim.x + threadIdx.x;
@@ -96,12 +99,10 @@ int gs_sum_launch(ax_gs *g, T *v, const ax::AlphaJob *job, cudaStream_t st) {
   if (!g) return AX_EINVAL;
   if (g->n_shared == 0 && !job) return AX_OK;
   if (g->n_shared > 0 && !v) return AX_EINVAL;
-  const unsigned grid = (unsigned)((g->n_shared + kGsThreads - 1) / kGsThreads);
-  if (job)
-    return ax::launch_chained(job->chained, gs_sum_kernel<T, true>, grid + 1, kGsThreads, 0, st, v, g->d_pairs,
-                              g->n_pairs, g->d_off, g->d_idx, g->n_multi, *job);
-  return ax::launch_chained(true, gs_sum_kernel<T, false>, grid, kGsThreads, 0, st, v, g->d_pairs,
-                            g->n_pairs, g->d_off, g->d_idx, g->n_multi, ax::AlphaJob{});
+  const unsigned grid = (unsigned)((g->n_shared + kGsThreads - 1) / kGsThreads) + (job ? 1 : 0);
+  auto kern = job ? gs_sum_kernel<T, true> : gs_sum_kernel<T, false>;
+  return ax::launch_chained(!job || job->chained, kern, grid, kGsThreads, 0, st, v, g->d_pairs, g->n_pairs,
+                            g->d_off, g->d_idx, g->n_multi, job ? *job : ax::AlphaJob{});
 }
 
 }  // namespace
