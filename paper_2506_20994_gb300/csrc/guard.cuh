@@ -75,13 +75,21 @@ AX_HD bool window_ok(unsigned ku, unsigned kg, unsigned kh, int fd) {
 // form one interval; u_range packs it as {lo | hi << 16, zero_ok} (zero_ok: an
 // all-zero u is fine), u_in_range tests it.
 AX_HD void u_range(unsigned kg, unsigned kh, int fd, unsigned &packed, unsigned &zero_ok) {
-  int lo = 1, hi = 0;  // empty
   zero_ok = window_ok(0u, kg, kh, fd) ? 1u : 0u;
-  for (int fu = 1; fu <= 2046; ++fu) {  // the window is an interval in fu
-    if (window_ok((unsigned)fu << 21, kg, kh, fd)) {
-      if (lo > hi) lo = fu;
-      hi = fu;
-    }
+  // every bound of window_ok is linear in u's exponent
+  const int b = field(kg) - 1023, c = field(kh) - 1023, d = fd - 1023;
+  const bool zero = kg == 0u || kh == 0u || fd == 0;
+  int hi = min(min(90, 100 - d), min(100 - b - d, 100 - b - c - d)), lo = -1022;
+  if (!zero) {
+    hi = min(hi, 100 - b - c - 2 * d);
+    lo = max(max(max(-78, -90 - d), max(-90 - b - d, -90 - b - c - d)), -90 - b - c - 2 * d);
+  }
+  lo += 1023;
+  hi += 1023;
+  // the bounds on the other factors, the same for every u
+  if (lo > hi || !window_ok((unsigned)lo << 21, kg, kh, fd)) {
+    lo = 1;  // empty
+    hi = 0;
   }
   packed = (unsigned)lo | ((unsigned)hi << 16);
 }
