@@ -227,11 +227,12 @@ int launch_df64(double *w, const double *u, const double *dx, const double *dxt,
                 cudaStream_t stream) {
   if (epb <= 0) epb = 256 / (LX * LX) < 1 ? 1 : 256 / (LX * LX);
   if (epb * LX * LX > 256) return AX_EINVAL;
-  const size_t smem = df64_smem<LX>(epb);
   auto kern = ax_df64_kernel<LX>;
-  static std::atomic<size_t> granted[kMaxDevices];
-  if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
+  static std::atomic<unsigned> occ[kMaxDevices];
+  static std::atomic<size_t> granted[kMaxDevices];
+  const size_t smem = spread_smem(kern, grid, epb * LX * LX, df64_smem<LX>(epb), occ);
+  if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   return launch_chained(true, kern, grid, epb * LX * LX, smem, stream, w, u, dx, dxt, h1, g11, g22,
                         g33, g12, g13, g23, nelv, epb);
 }

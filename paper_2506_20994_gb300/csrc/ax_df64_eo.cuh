@@ -383,11 +383,12 @@ int launch_df64eo(double *w, const double *u, const double *dx, const double *dx
   constexpr int H3 = (LX / 2) * (LX / 2) * (LX / 2);
   if (epb <= 0) epb = 256 / H3 < 1 ? 1 : 256 / H3;
   if (epb * H3 > 256) return AX_EINVAL;
-  const size_t smem = df64eo_smem<LX>(epb);
   auto kern = ax_df64eo_kernel<LX>;
-  static std::atomic<size_t> granted[kMaxDevices];
-  if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
+  static std::atomic<unsigned> occ[kMaxDevices];
+  static std::atomic<size_t> granted[kMaxDevices];
+  const size_t smem = spread_smem(kern, grid, epb * H3, df64eo_smem<LX>(epb), occ);
+  if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   return launch_chained(true, kern, grid, epb * H3, smem, stream, w, u, dx, dxt, h1, g11, g22, g33, g12, g13, g23, nelv, epb);
 }
 

@@ -311,11 +311,14 @@ int launch_kstep(W *w, const SU *u, const T *dx, const T *dxt, const S *h1, cons
                  int nelv, int epb, cudaStream_t stream, double *dotp = nullptr) {
   if (epb <= 0) epb = kstep_default_epb(LX);
   if (epb * LX * LX > 1024) return AX_EINVAL;
-  const size_t smem = kstep_smem<LX, T, false, kstep_vec<LX, T>()>(epb);
   auto kern = dotp ? ax_kstep_kernel<LX, SU, S, T, W, true> : ax_kstep_kernel<LX, SU, S, T, W>;
-  static std::atomic<size_t> granted[2][kMaxDevices];  // per kernel
-  if (!grant_smem(kern, smem, granted[dotp != nullptr])) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
+  static std::atomic<unsigned> occ[2][kMaxDevices];    // per kernel
+  static std::atomic<size_t> granted[2][kMaxDevices];
+  const size_t smem = spread_smem(kern, grid, epb * LX * LX,
+                                  kstep_smem<LX, T, false, kstep_vec<LX, T>()>(epb),
+                                  occ[dotp != nullptr]);
+  if (!grant_smem(kern, smem, granted[dotp != nullptr])) return AX_EINVAL;
   return launch_chained(true, kern, grid, epb * LX * LX, smem, stream, w, u, dx, dxt, h1, g11, g22,
                         g33, g12, g13, g23, nelv, epb, dotp);
 }

@@ -291,11 +291,12 @@ int launch_tri(float *w, const float *u, const float *dx, const float *dxt, cons
                const double *corners, const double *xi, const double *wq, int nelv,
                cudaStream_t st) {
   const int epb = 256 / (LX * LX) < 1 ? 1 : 256 / (LX * LX);
-  const size_t smem = tri_smem<LX>(epb);
   auto kern = h1 ? ax_tri_f32_kernel<LX, true> : ax_tri_f32_kernel<LX, false>;
-  static std::atomic<size_t> granted[2][kMaxDevices];
-  if (!grant_smem(kern, smem, granted[h1 != nullptr])) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
+  static std::atomic<unsigned> occ[2][kMaxDevices];
+  static std::atomic<size_t> granted[2][kMaxDevices];
+  const size_t smem = spread_smem(kern, grid, epb * LX * LX, tri_smem<LX>(epb), occ[h1 != nullptr]);
+  if (!grant_smem(kern, smem, granted[h1 != nullptr])) return AX_EINVAL;
   return launch_chained(true, kern, grid, epb * LX * LX, smem, st, w, u, dx, dxt, h1, corners, xi,
                         wq, nelv, epb);
 }

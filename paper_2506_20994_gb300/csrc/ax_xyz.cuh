@@ -61,9 +61,11 @@ int launch_xyz(AX_XYZ_PARAMS, cudaStream_t st) {
     smem = kstep_smem<LX, double, true>(epb);
     kern = ax_kstep_xyz_kernel<LX>;
   }
-  static std::atomic<size_t> granted[kMaxDevices];
-  if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   const unsigned grid = (unsigned)((nelv + epb - 1) / epb);
+  static std::atomic<unsigned> occ[kMaxDevices];
+  static std::atomic<size_t> granted[kMaxDevices];
+  smem = spread_smem(kern, grid, epb * LX * LX, smem, occ);
+  if (!grant_smem(kern, smem, granted)) return AX_EINVAL;
   return launch_chained(true, kern, grid, epb * LX * LX, smem, st, AX_XYZ_ARGS);
 }
 

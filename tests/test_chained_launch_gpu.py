@@ -363,3 +363,30 @@ def test_matrices_written_by_the_kernel_in_front(lx):
     for _ in range(5):
         for a, b in zip(chain(False), ref):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dims,lx", [((11, 11, 11), 7), ((12, 20, 10), 5), ((20, 20, 1), 13),
+                                     ((20, 20, 1), 9), ((10, 10, 3), 11)])
+def test_chains_of_grids_that_fill_part_of_a_wave(dims, lx):
+    """Grids of two and more blocks per SM that are less than one full wave:
+    their blocks are held to an even share of each SM."""
+    c = operator_case(dims, lx, seed=670 + lx)
+    d = _scale(c)
+    G = [d[k] for k in GKEYS]
+    bufs = [d["u"].clone(), torch.zeros_like(d["u"]), torch.zeros_like(d["u"])]
+    _same(lambda w, u, k: ax.ax_helm(w, u, d["dx"], d["dxt"], d["h1"], *G, lx), bufs, n=9)
+    _same(lambda w, u, k: ax.ax_helm_xyz(w, u, d["dx"], d["dx"], d["dx"], d["dxt"], d["dxt"],
+                                         d["dxt"], d["h1"], *G, lx), bufs, n=6)
+    f = torch.float32
+    e = _scale(c, f)
+    Gf = [e[k] for k in GKEYS]
+    buf32 = [e["u"].clone(), torch.zeros_like(e["u"]), torch.zeros_like(e["u"])]
+    _same(lambda w, u, k: ax.ax_helm_f32(w, u, e["dx"], e["dxt"], e["h1"], *Gf, lx), buf32, n=9)
+    cor = _t(ax.box_corners(c["vertices"])).reshape(-1)
+    xi, wq = (_t(a) for a in ax.gll(lx))
+    _same(lambda w, u, k: ax.ax_helm_trilinear_f32(w, u, e["dx"], e["dxt"], e["h1"], cor, xi, wq, lx),
+          buf32, n=9)
+    w = torch.empty_like(d["u"])
+    ax.ax_helm(w, d["u"], d["dx"], d["dxt"], d["h1"], *G, lx)
+    ref = c["w"] * float(d["h1"].max() / _t(c["h1"]).max())  # linear in h1
+    assert float((w - _t(ref)).norm()) <= 1e-12 * float(_t(ref).norm())
