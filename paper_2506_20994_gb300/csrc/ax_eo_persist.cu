@@ -192,7 +192,8 @@ int eopr_launch(int lx, double *w, const double *u, const double *dx, const doub
 
 int eop_launch(int lx, const EopArgs &a, cudaStream_t st) {
   if (a.pw && !(a.dotp && a.r && a.minv && a.beta)) return AX_EINVAL;
-  if ((a.corr && !a.use_corr) || (a.x && !a.alpha) || (a.hb && a.dotp)) return AX_EINVAL;
+  if ((a.corr && !a.use_corr) || (a.x && (!a.alpha || !eop_x_update(lx))) || (a.hb && a.dotp))
+    return AX_EINVAL;
   switch (lx) {
     case 6: return eop_launch_lx<6>(a, st);
     case 8: return eop_launch_lx<8>(a, st);

@@ -32,6 +32,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "dispatch.h"
 #include "df64.cuh"
 #include "guard.cuh"
 
@@ -63,6 +64,8 @@ struct Cfg {
   static constexpr size_t SMEM = OFF_MISC + 16 + NW * 8 + NW * 8 + 16;
   // resident CTAs per SM the launch bounds ask for
   static constexpr int MINB = LX == 6 ? 8 : LX == 8 ? 4 : LX == 10 ? 2 : 1;
+  // the fused direction update may carry the solver's x update (EopUpd::x)
+  static constexpr bool XUP = eop_x_update(LX);
   static_assert(LINE_BYTES >= 3 * (size_t)N3 * 8, "fallback scratch must fit the lines");
 };
 
@@ -184,7 +187,14 @@ struct EopMesh {
 // (+ corr when use_corr) + beta pw, formed in place in front of the apply;
 // x (may be null) += alpha pw with the old pw: the previous step's solution
 // update, whose read of pw is this one's (at 56 % of HBM the apply has the
-// bandwidth to spare that the solver's vector kernels lack).
+// bandwidth to spare that the solver's vector kernels lack); only at the orders
+// of eop_x_update.  The vectors are read through L1: at lx 6 and 10 an
+// element's rows are no whole 32-byte sectors, and past L1 each sector came
+// twice (an apply at 26^3 elements, lx 10: 595 -> 554 us; an iteration at 32^3,
+// lx 8: 632 -> 619 us).  In a chained launch this is safe because only the
+// solver loops launch this form, behind a kernel that reads these vectors past
+// L1 (the update or the dots), and that kernel's own launch has emptied L1 of
+// what the apply before it had read.
 struct EopUpd {
   double *pw;
   const double *r, *minv, *corr;
@@ -205,6 +215,7 @@ struct EopPos {
 // pointer every per-element access would be a load.
 struct SeqOne {
   static constexpr bool kRotate10 = true;  // line layout, see lpos
+  static constexpr bool kOneMesh = true;   // coefficients staged once
   EopMesh m;
   long long nelv;
   AX_D bool first(EopPos &p) const {
@@ -395,14 +406,14 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   if constexpr (RAW) ready();
   sync();  // the barrier is initialised before anyone waits on it
   if (tid == 0 && have) issue_geo(pos);
-  bool staged = false;  // the first run's coefficients are
-  if constexpr (!RAW) {
-    if (have) {
-      load_coef(seq.mesh(seq.mesh_of(pos)));
-      staged = true;
-    }
-    ready();
+  // one mesh: the coefficients at once, in front of ready() where they may be
+  // (not with the direction update: the loop is slower so, an iteration at 26^3
+  // elements, lx 10, 791 against 763 us; at lx 6, 8 and 12 within 0.5 %)
+  constexpr bool kEarly = Seq::kOneMesh && !PUPD;
+  if constexpr (kEarly) {
+    if (have) load_coef(seq.mesh(0));
   }
+  if constexpr (!RAW) ready();
 
   double uv[2][2] = {{0.0, 0.0}, {0.0, 0.0}};      // u (or r) of the element in turn
   double mv[2][2], pv[2][2], qv[2][2];             // PUPD: minv, old direction, corr
@@ -415,10 +426,10 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
       for (int a = 0; a < 2; ++a) {
         const size_t q = eb + pidx(b, a);
         if constexpr (PUPD) {
-          uv[b][a] = __ldcg(up.r + q);
-          mv[b][a] = __ldcg(up.minv + q);
-          pv[b][a] = __ldcg(up.pw + q);
-          qv[b][a] = up.corr ? __ldcg(up.corr + q) : 0.0;
+          uv[b][a] = up.r[q];
+          mv[b][a] = up.minv[q];
+          pv[b][a] = up.pw[q];
+          qv[b][a] = up.corr ? up.corr[q] : 0.0;
         } else {
           uv[b][a] = __ldcg(M.u + q);
         }
@@ -432,8 +443,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
   // behind a test that is false after the first element, cost 6 %)
   while (have) {
     cmesh = seq.mesh_of(pos);
-    if (!staged) load_coef(seq.mesh(cmesh));  // the previous element's last barrier freed them
-    staged = false;
+    if constexpr (!kEarly) load_coef(seq.mesh(cmesh));  // freed by the last barrier
   for (; have && seq.mesh_of(pos) == cmesh; parity ^= 1u) {
     EopPos nxp;
     const bool more = seq.advance(pos, nxp);
@@ -446,12 +456,12 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     double ucur[2][2];
     guard::Key ukk;
     double xv[2][2];
-    if constexpr (PUPD) {
+    if constexpr (PUPD && C::XUP) {
       if (real && up.x) {
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
-          for (int a = 0; a < 2; ++a) xv[b][a] = __ldcg(up.x + eb + pidx(b, a));
+          for (int a = 0; a < 2; ++a) xv[b][a] = up.x[eb + pidx(b, a)];
       }
     }
 #pragma unroll
@@ -473,7 +483,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     for (int b = 0; b < 2; ++b)
 #pragma unroll
       for (int a = 0; a < 2; ++a) v[b][a] = split(ucur[b][a]);
-    if constexpr (PUPD) {
+    if constexpr (PUPD && C::XUP) {
       if (real && up.x) {
 #pragma unroll
         for (int b = 0; b < 2; ++b)
@@ -572,7 +582,7 @@ AX_D void eop_run(unsigned char *sm, int tid, const Seq &seq, Sync sync, SyncAnd
     if (tid == 0 && more) {
       fence_async_smem();
       issue_geo(nxp);
-      if constexpr (PUPD) {
+      if constexpr (PUPD && C::XUP) {
         if (up.x) prefetch_l2(up.x + (size_t)seq.elem(nxp) * N3, N3 * 8);
       }
       if constexpr (HB) prefetch_l2(M.hb + (size_t)seq.elem(nxp) * N3, N3 * 8);
@@ -674,7 +684,9 @@ ax_eop_kernel(const EopMesh mesh, long long nelv, int *__restrict__ err,
     grid_go();
     if constexpr (PUPD) {  // solver scalars live on the device
       up.beta = __ldcg(beta_p);
-      if (up.x) up.alpha = __ldcg(alpha_p);
+      if constexpr (C::XUP) {
+        if (up.x) up.alpha = __ldcg(alpha_p);
+      }
       up.use_corr = up.corr != nullptr && __ldcg(use_corr_p) != 0;
     }
   };

@@ -65,6 +65,7 @@ __host__ __device__ constexpr int batch_kloop_epb(int lx) {
 template <class M>
 struct SeqItemsT {
   static constexpr bool kRotate10 = false;  // line layout of the fp64 body, see eop::lpos
+  static constexpr bool kOneMesh = false;   // coefficients staged before each run of a mesh
   const BatchItem *items;
   int ib, ie, slot, S;
   const M *meshes;

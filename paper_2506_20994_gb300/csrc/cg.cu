@@ -49,10 +49,18 @@ using ax::CgScalars;
 // ---------------------------------------------------------------- kernels
 // Walks the block-strided vectors v = first, + stride, ... < n two at a time:
 // load(slot, v) for both, then work(slot, v) for both, so that two vectors'
-// loads are in flight before the first one's stores.
-template <class Load, class Work>
+// loads are in flight before the first one's stores.  TWO false: one at a time
+// (where two vectors' values exceed the registers that four blocks per SM leave).
+template <bool TWO = true, class Load, class Work>
 __device__ __forceinline__ void walk2(int64_t n, Load load, Work work) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  if constexpr (!TWO) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+      load(0, v);
+      work(0, v);
+    }
+    return;
+  }
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += 2 * stride) {
     const bool two = v + stride < n;
     load(0, v);
@@ -486,7 +494,10 @@ int apply_fused(ax_poisson *P, float *w, const float *u, cudaStream_t st,
 // p next (fp64 with prepared geometry); false where no such kernel exists.
 bool fuses_update(const ax_poisson *P, const double *) { return P->dotp && P->ndot > 0; }
 bool fuses_update(const ax_poisson *P, const float *) { return P->dotp && P->lowp_eo32; }
-// fp64: the previous step's x += alpha p as well, from the old p it reads
+bool x_in_apply(const ax_poisson *P, const double *) { return ax::eop_x_update(P->lx); }
+bool x_in_apply(const ax_poisson *, const float *) { return false; }
+// fp64: the previous step's x += alpha p as well (x given), from the old p it
+// reads
 int apply_fused_update(ax_poisson *P, double *w, double *p, const double *r,
                        const double *minv, double *x, cudaStream_t st,
                        const double *corr = nullptr, bool chained = true) {
@@ -510,6 +521,10 @@ int apply_fused_update(ax_poisson *P, float *w, float *p, const float *r, const 
   const ax::AlphaJob job = alpha_job<float>(P, chained);
   return apply_lowp(P, w, p, st, P->dotp, &up, &job);
 }
+
+// Whether a loop's gather-scatter is chained behind the apply.
+bool chains_gs(const ax_poisson *P, const double *) { return P->n < (int64_t(1) << 24); }
+bool chains_gs(const ax_poisson *P, const float *) { return P->n < (int64_t(1) << 19); }
 
 // Asks the next reduction that forms rr for its values (address and number)
 ax::CgMailTo next_mail(ax_poisson *P) { return ax::CgMailTo{P->mail, ++P->mail_seq}; }
@@ -562,22 +577,16 @@ int pcg_loop(ax_poisson *P, T *x, const T *b, T *r, T *p, T *w, const T *mask, c
   // of p . A_e p), and the mask moves into the update
   const bool fused = fused_parts(P, (const T *)nullptr) > 0;
   // after the first iteration the next direction is formed inside the apply,
-  // in fp64 together with the x update of the step before
+  // in fp64 at some orders together with the x update of the step before
   const bool fused_p = fused && fuses_update(P, (const T *)nullptr);
-  const bool fused_x = fused_p && std::is_same_v<T, double>;
-  // The gather-scatter begins while the apply ends only on smaller meshes: its
-  // blocks, and those of the update chained behind it, then stand ready, but
-  // once the grids are many times what the chip holds they only take the
-  // running kernel's places.  us an iteration at lx = 8, chained against not:
-  // fp32 6^3 elements 18.1 / 20.5, 10^3 26.8 / 25.2 (bf16 data 22.3 / 24.3),
-  // 16^3 47.7 / 46.0, 20^3 82.9 / 76.4, 32^3 301 / 271; fp64 16^3 94.7 / 99.0,
-  // 24^3 279.2 / 282.1, 28^3 436 / 439, 32^3 646.8 / 642.6.
-  const bool gs_chained = n < (std::is_same_v<T, double> ? int64_t(1) << 24 : int64_t(1) << 19);
+  const bool fused_x = fused_p && x_in_apply(P, (const T *)nullptr);
+  const bool gs_chained = chains_gs(P, (const T *)nullptr);
   // The first half of iteration `it`: direction, apply, alpha.  It touches no
   // result (x only to complete the step before), so it is launched before the
   // host has tested that step: the GPU goes on while the test's values travel.
   auto front = [&](int it) -> int {
-    if (fused_p && it > 0) return apply_fused_update(P, w, p, r, minv, x, st, nullptr, gs_chained);
+    if (fused_p && it > 0)
+      return apply_fused_update(P, w, p, r, minv, fused_x ? x : nullptr, st, nullptr, gs_chained);
     int rc = AX_OK;
     if (it > 0)
       rc = ax::launch_chained(true, cg_p_kernel<T>, nb, kRedThreads, 0, st, p, r, minv, P->scal, n);
@@ -1093,7 +1102,7 @@ fcg_update_kernel(T *__restrict__ x, T *__restrict__ r, T *__restrict__ r_old,
     constexpr int NV = 16 / sizeof(T);
     V xv[2], rv[2], pv[2], wv[2], mv[2], cv[2];
     auto at = [](const T *f, int64_t v) { return __ldcg(reinterpret_cast<const V *>(f) + v); };
-    walk2(
+    walk2<sizeof(T) == 4 || !XUP>(
         n / NV,
         [&](int k, int64_t v) {
           xv[k] = XUP ? at(x, v) : V{};
@@ -1307,6 +1316,8 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
   // pcg_loop); the fp32 flexible loop keeps its direction kernel
   const bool fused_p = std::is_same_v<T, double> && fused_parts(P, (const T *)nullptr) > 0 &&
                        fuses_update(P, (const T *)nullptr);
+  const bool fused_x = fused_p && x_in_apply(P, (const T *)nullptr);
+  const bool gs_chained = std::is_same_v<T, float> || chains_gs(P, (const T *)nullptr);
   auto precondition = [&](int first) -> int {
     if (have) {
       int rc = ax::mlp_correction<T>(M, corr, r, minv, mask, c, P->nelv, st,
@@ -1345,16 +1356,17 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
     const bool checked = (it + 1) % P->check_every == 0 || it + 1 == maxit;
     if (fused) {
       if constexpr (std::is_same_v<T, double>)
-        rc = (fused_p && applied > 0) ? apply_fused_update(P, w, p, r, minv, x, st, corr)
-                                      : apply_fused(P, w, p, st);
+        rc = (fused_p && applied > 0)
+                 ? apply_fused_update(P, w, p, r, minv, fused_x ? x : nullptr, st, corr, gs_chained)
+                 : apply_fused(P, w, p, st, gs_chained);
       else
-        rc = apply_fused(P, w, p, st);
+        rc = apply_fused(P, w, p, st, gs_chained);
       ++applied;
       if (rc) return rc;
       // rr only where the host will test it (after this iteration)
-      auto update = checked ? (fused_p ? fcg_update_kernel<T, true, true, !std::is_same_v<T, double>>
+      auto update = checked ? (fused_x ? fcg_update_kernel<T, true, true, !std::is_same_v<T, double>>
                                        : fcg_update_kernel<T, true, true, true>)
-                            : (fused_p ? fcg_update_kernel<T, true, false, !std::is_same_v<T, double>>
+                            : (fused_x ? fcg_update_kernel<T, true, false, !std::is_same_v<T, double>>
                                        : fcg_update_kernel<T, true, false, true>);
       if (ax::launch_chained(true, update, nb, kRedThreads, 0, st, x, r, r_old, p, w, c, cm, P->scal,
                              P->partials, n, checked ? next_mail(P) : ax::CgMailTo{}))
@@ -1386,7 +1398,7 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
     }
   }
   if constexpr (std::is_same_v<T, double>)
-    if (fused_p && applied > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
+    if (fused_x && applied > 0) cg_x_kernel<<<nb, kRedThreads, 0, st>>>(x, p, P->scal, n);
   if ((rc = read_scalars())) return rc;
   if (iters) *iters = it;
   if (relres) *relres = rel;

@@ -127,6 +127,12 @@ struct EopArgs {
   long long drop = -1;  // testing aid: element whose geometry copy is not issued
 };
 bool eop_supported(int lx);
+// The orders whose fused direction update also carries x += alpha p.  At lx 6
+// and 10 the kernel has all 128 registers in use without it and spills with it
+// in the element loop: a CG iteration, with against without, at lx 10 123.6 /
+// 116.4 us (13^3 elements) and 820 / 800 us (26^3), at lx 6 138.5 / 135.1
+// (24^3) and 971 / 953 (48^3).
+constexpr bool eop_x_update(int lx) { return lx == 8 || lx == 12; }
 // The persistent even-odd kernel on the caller's fp64 arrays (ax_helm, no
 // handle): lx in {6, 8, 10, 12} and 16-byte aligned geometry arrays, else
 // AX_EINVAL (the caller then takes another kernel).

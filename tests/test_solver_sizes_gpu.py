@@ -52,3 +52,25 @@ def test_flexible_loop_points_odd_and_even(dims, lx):
         q = P.fcg(b, None, tol=TOL)
         return q[0], q[2]
     _solve_and_check(dims, lx, solve)
+
+
+@pytest.mark.parametrize("lx", [6, 8, 10, 12])
+@pytest.mark.parametrize("flexible", [False, True], ids=["cg", "fcg"])
+def test_solution_belongs_to_the_residual(lx, flexible):
+    """x where it is updated by the update kernel (lx 6, 10) and by the next
+    step's apply (lx 8, 12): after any number of steps, tested at every one of
+    them or at the last, ||b - A x|| is the recurrence's residual norm.  The two
+    differ by rounding: some hundred operations of 2^-53 on terms of ||b||'s
+    size."""
+    P = ax.Poisson(synth.box_vertices(4, 3, 3, seed=lx), lx, h1=ax.fourier_coefficient(2))
+    b = P.rhs(synth.poisson_source)
+    c = P.gs.inverse_multiplicity()
+    norm = lambda v: float((c * v.reshape(-1) * v.reshape(-1)).sum()) ** 0.5
+    for steps in (1, 2, 7, 24):
+        for every in (1, 5, 1000):
+            P.set_check_every(every)
+            f = P.fcg if flexible else P.cg
+            r = f(b, None, tol=0.0, maxit=steps, raise_on_error=False) if flexible else f(
+                b, tol=0.0, maxit=steps, raise_on_error=False)
+            assert r[1] == steps
+            assert abs(norm(P.residual(b, r[0])) / norm(b) - r[2]) <= 1e-12 + 1e-10 * r[2]
