@@ -522,9 +522,33 @@ int apply_fused_update(ax_poisson *P, float *w, float *p, const float *r, const 
   return apply_lowp(P, w, p, st, P->dotp, &up, &job);
 }
 
-// Whether a loop's gather-scatter is chained behind the apply.
+// Whether a loop's gather-scatter is chained behind the apply.  Its blocks, and
+// those of the kernel chained behind it, then stand ready when the apply ends
+// (2 us an iteration on small meshes), but they wait in places that the apply's
+// own blocks would take: worst behind the fp32 applies that fill an SM with
+// many small blocks.  us an iteration, chained against not (n^3 elements):
+//   fp64        lx 8   6^3 22.9 / 24.8, 16^3 90.6 / 92.9, 28^3 413 / 415, 32^3
+//   613 / 609; lx 10   13^3 111 / 119, 20^3 358 / 360, 26^3 769 / 762; the
+//   flexible loop likewise (lx 8 16^3 101 / 104, lx 6 44^3 868 / 845)
+//   fp32 data   lx 8   7^3 16.8 / 18.8, 8^3 22.2 / 20.8, 16^3 42.0 / 39.8, 32^3
+//   282 / 252; lx 10   6^3 18.7 / 20.9, 7^3 25.7 / 24.9, 20^3 177 / 160; lx 6
+//   20^3 44.2 / 45.3, 44^3 330 / 329; lx 12   8^3 31.1 / 31.3, 20^3 254 / 254
+//   bf16 data   lx 8   10^3 20.1 / 21.2, 12^3 25.1 / 24.4, 32^3 248 / 217; lx
+//   6, 10 and 12 chained better or equal (lx 10 20^3 151 / 152)
+//   odd orders (k-loop) chained better at all sizes (lx 5 48^3 291 / 294).
 bool chains_gs(const ax_poisson *P, const double *) { return P->n < (int64_t(1) << 24); }
-bool chains_gs(const ax_poisson *P, const float *) { return P->n < (int64_t(1) << 19); }
+bool chains_gs(const ax_poisson *P, const float *) {
+  if (!P->lowp_eo32 || (P->lx != 8 && P->lx != 10)) return true;
+  if (P->lowp_mode == 2) return P->lx == 10 || P->n < (int64_t(1) << 19);
+  return P->n < (int64_t(1) << 18);
+}
+// The flexible fp32 loop has the network's kernels in front of the next apply:
+// chained better or equal (lx 8 16^3 79.7 / 81.3, 32^3 460 / 462; lx 6 44^3 588
+// / 591), but at lx 12 from 8^3 on (83.8 / 82.0, 20^3 528 / 504).
+bool chains_gs_flexible(const ax_poisson *P, const double *v) { return chains_gs(P, v); }
+bool chains_gs_flexible(const ax_poisson *P, const float *) {
+  return P->lx != 12 || P->n < (int64_t(1) << 19);
+}
 
 // Asks the next reduction that forms rr for its values (address and number)
 ax::CgMailTo next_mail(ax_poisson *P) { return ax::CgMailTo{P->mail, ++P->mail_seq}; }
@@ -1317,7 +1341,7 @@ int fcg_loop(ax_poisson *P, const ax_mlp *M, T *x, const T *b, T *r, T *r_old, T
   const bool fused_p = std::is_same_v<T, double> && fused_parts(P, (const T *)nullptr) > 0 &&
                        fuses_update(P, (const T *)nullptr);
   const bool fused_x = fused_p && x_in_apply(P, (const T *)nullptr);
-  const bool gs_chained = std::is_same_v<T, float> || chains_gs(P, (const T *)nullptr);
+  const bool gs_chained = chains_gs_flexible(P, (const T *)nullptr);
   auto precondition = [&](int first) -> int {
     if (have) {
       int rc = ax::mlp_correction<T>(M, corr, r, minv, mask, c, P->nelv, st,

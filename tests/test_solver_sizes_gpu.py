@@ -74,3 +74,24 @@ def test_solution_belongs_to_the_residual(lx, flexible):
                 b, tol=0.0, maxit=steps, raise_on_error=False)
             assert r[1] == steps
             assert abs(norm(P.residual(b, r[0])) / norm(b) - r[2]) <= 1e-12 + 1e-10 * r[2]
+
+
+# both sides of the lines of the other operators: fp32 data at 2^18 points (lx
+# 8 and 10), the flexible fp32 loop at 2^19 (lx 12), and orders without a line
+@pytest.mark.parametrize("dims,lx,mode", [((7, 8, 8), 8, ax.AX_PREC_F32), ((8, 8, 8), 8, ax.AX_PREC_F32),
+                                          ((6, 6, 7), 10, ax.AX_PREC_F32), ((7, 7, 6), 10, ax.AX_PREC_F32),
+                                          ((7, 7, 6), 10, ax.AX_PREC_BF16), ((14, 14, 14), 6, ax.AX_PREC_F32),
+                                          ((13, 12, 12), 7, ax.AX_PREC_F32)])
+def test_refinement_around_the_other_lines(dims, lx, mode):
+    def solve(P, b):
+        q = P.mpcg(b, mode=mode, tol=TOL, inner_tol=1e-2 if mode == ax.AX_PREC_BF16 else 1e-4)
+        return q[0], q[-2]
+    _solve_and_check(dims, lx, solve)
+
+
+@pytest.mark.parametrize("dims", [(6, 7, 7), (7, 7, 7)])
+def test_flexible_refinement_around_the_line(dims):
+    def solve(P, b):
+        q = P.mpfcg(b, None, tol=TOL)
+        return q[0], q[3]
+    _solve_and_check(dims, 12, solve)
