@@ -200,8 +200,9 @@ __device__ __forceinline__ void df64_body(double *__restrict__ w, const double *
 }
 
 // Blocks per SM the launch bounds ask for: the low orders gain from more warps
-// (64 or 80 registers; lx 4 132 -> 127 us, lx 5 159 -> 147, lx 7 181 -> 170 at
-// 5.8 M points), lx 3 and lx >= 8 do not.
+// (64 or 80 registers; us at 5.8 M points without and with: lx 3 139 / 121, lx
+// 4 134 / 128, lx 5 163 / 148, lx 6 175 / 169, lx 7 212 / 193; at 8^3 elements
+// 8.3 / 9.2, 8.9 / 9.2, 8.6 / 9.4, 9.7 / 9.9, 11.5 / 11.6), lx >= 8 do not.
 constexpr int df64_minb(int lx) { return lx == 3 || lx == 4 ? 4 : lx >= 5 && lx <= 7 ? 3 : 0; }
 template <int LX>
 __global__ void __launch_bounds__(256, df64_minb(LX))

@@ -246,7 +246,7 @@ struct SeqOne {
 // M.coef and M.urange are not used.  (ax_helm on fp64 arrays.)
 // HB: the Helmholtz mass term, w += M.hb .* u with fp64 units as w is stored.
 // As a pass of its own it moved 32 bytes a point more (4096 elements, lx = 10:
-// 134.9 us a call, now 118.5).
+// 134.9 us a call, 118.5 so; 109 with the shorter split).
 // ready(): called once, after the set-up that needs no other kernel's results
 // (the first element's prepared geometry and the coefficients, both the
 // handle's own) and before everything else; RAW calls it first.

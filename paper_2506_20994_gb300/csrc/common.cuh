@@ -121,8 +121,9 @@ inline int launch_chained(bool chained, void (*kern)(P...), dim3 grid, unsigned 
 // wave of two or more blocks per SM, so that no SM takes more than its part.
 // Launched early, the blocks otherwise crowd onto the SMs that the kernel in
 // front has left free first, and those then run for longer than the rest (fp32
-// at lx 13, 400 blocks: 21 us unchained, 30 chained and crowded; bf16 at lx 9
-// 14.9 / 19.8; fp64 at lx 7, 267 blocks, 20.9 / 25.1).  occ: this kernel's
+// at lx 13, 400 blocks: 21.0 us unchained, 29.7 chained and crowded, 20.6 so;
+// bf16 at lx 9, 440 blocks, 15.0 / 19.8 / 13.5; fp64 at lx 7, 267 blocks, 20.9 /
+// 25.1 / 18.7).  occ: this kernel's
 // resident blocks per SM, with the block size they hold for.
 template <typename K>
 inline size_t spread_smem(K kernel, unsigned grid, unsigned block, size_t smem,

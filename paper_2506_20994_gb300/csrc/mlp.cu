@@ -304,7 +304,7 @@ mlp_sym_apply_kernel(T *__restrict__ corr, const T *__restrict__ r,
 
   ax::grid_wait();
   ax::grid_go();
-  // the scaled rows, warp w rows w, w + 4, ... (N even: pairs stay in a row)
+  // the scaled rows, warp w rows w, w + kSymWarps (N even: pairs stay in a row)
   for (int row = wp; row < 16; row += kSymWarps) {
     const size_t base = (size_t)(e0 + (row < nel ? row : 0)) * N;
 #pragma unroll 8
