@@ -91,9 +91,10 @@ inline bool grant_smem(K kernel, size_t bytes, std::atomic<size_t> (&granted)[kM
 // bulk-copy engine): L1 is emptied when a kernel is launched, which here is
 // before the kernel in front of it is done, and read-only loads (const
 // __restrict__, __ldg) would return lines that kernel's neighbours have
-// rewritten since (EopUpd's vectors are the exception).  In front of the wait stands only what no kernel of the
-// stream can be writing: the operator handle's coefficients, written once, and
-// its prepared geometry (see eop_prepare_lx).
+// rewritten since (EopUpd's vectors are the exception).  In front of the wait
+// stands only what no kernel of the stream can be writing: the operator
+// handle's coefficients, written once, and its prepared geometry (see
+// eop_prepare_lx).
 AX_D void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 AX_D void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>

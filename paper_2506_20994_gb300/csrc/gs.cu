@@ -101,8 +101,9 @@ int gs_sum_launch(ax_gs *g, T *v, const ax::AlphaJob *job, cudaStream_t st) {
   if (g->n_shared > 0 && !v) return AX_EINVAL;
   const unsigned grid = (unsigned)((g->n_shared + kGsThreads - 1) / kGsThreads) + (job ? 1 : 0);
   auto kern = job ? gs_sum_kernel<T, true> : gs_sum_kernel<T, false>;
-  return ax::launch_chained(!job || job->chained, kern, grid, kGsThreads, 0, st, v, g->d_pairs, g->n_pairs,
-                            g->d_off, g->d_idx, g->n_multi, job ? *job : ax::AlphaJob{});
+  return ax::launch_chained(!job || job->chained, kern, grid, kGsThreads, 0, st, v, g->d_pairs,
+                            g->n_pairs, g->d_off, g->d_idx, g->n_multi,
+                            job ? *job : ax::AlphaJob{});
 }
 
 }  // namespace

@@ -151,8 +151,8 @@ AX_D bool elem_ok(const Record &r, int le) {
 // the `nt` threads of the element (rank `r`); `sync()` synchronises at least
 // those threads.  `scr` holds 3 lx^3 doubles of shared memory.  u is read past
 // L1 (the kernel in front of a chained launch may have written it, or the
-// caller earlier in the same one).  dot (optional): adds this thread's share of u . w.  Threads with
-// `on` false only take part in the two barriers.
+// caller earlier in the same one).  dot (optional): adds this thread's share of
+// u . w.  Threads with `on` false only take part in the two barriers.
 template <int LX, class Sync>
 __device__ __noinline__ void element_f64(bool on, double *__restrict__ w, const double *u, const double *__restrict__ dx,
                       const double *__restrict__ dy, const double *__restrict__ dz,
